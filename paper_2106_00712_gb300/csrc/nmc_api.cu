@@ -834,7 +834,7 @@ nmc_status ensure_series(nmc_ctx* x, long long need) {
 // first failed index check of the NMC_DEBUG build (0: none, or not a debug build)
 unsigned int debug_failed() {
   unsigned int (*const readers[])() = {debug_fail_flip, debug_fail_stab, debug_fail_gemm,
-                                       debug_fail_gemm_tc, debug_fail_misc};
+                                       debug_fail_gemm_fx, debug_fail_gemm_tc, debug_fail_misc};
   for (auto r : readers)
     if (const unsigned int id = r()) return id;
   return 0u;

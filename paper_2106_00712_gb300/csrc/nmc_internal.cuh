@@ -49,6 +49,7 @@ constexpr uint32_t kPhiloxW1 = 0xBB67AE85u;
 unsigned int debug_fail_flip();
 unsigned int debug_fail_stab();
 unsigned int debug_fail_gemm();
+unsigned int debug_fail_gemm_fx();
 unsigned int debug_fail_gemm_tc();
 unsigned int debug_fail_misc();
 
@@ -129,6 +130,9 @@ struct GemmArgs {
 
 void gemm(const GemmArgs<double>& g, cudaStream_t st);
 void gemm(const GemmArgs<float>& g, cudaStream_t st);
+// gemm's FP64 products as exact integer slices on the tensor cores, K <= 256 (gemm_fx.cu)
+bool gemm_fx_supported(const GemmArgs<double>& g);
+void gemm_fx(const GemmArgs<double>& g, cudaStream_t st);
 // The same FP64-in, FP64-out product with the sums accumulated in FP32 pairs on the FP32
 // pipe (error-free products and sums, ~2^-44 relative to the sum of |a_ik b_kj|)
 void gemm_pair(const GemmArgs<double>& g, cudaStream_t st);
