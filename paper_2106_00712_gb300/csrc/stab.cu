@@ -3,18 +3,16 @@
 //
 // k_qrp: Householder QR with column pivoting (Businger-Golub): at step p the remaining
 //   column of largest norm (lowest index on ties) is swapped into place, a reflector
-//   H_p = I - tau v v^T (v_p = 1) zeroes it below the diagonal, and the trailing columns
-//   are updated; squared column norms are downdated with the usual safeguard (recomputed
-//   when the downdated value has lost more than half its digits). Outputs U = Q (formed in
-//   place by backward accumulation of the reflectors), D = |diag R| and T = D^{-1} R P^T.
+//   H_p = I - tau v v^T zeroes it below the diagonal, and the trailing columns are updated;
+//   squared column norms are downdated and summed again when little of them is left. Outputs
+//   U = Q (formed in place by backward accumulation of the reflectors), D = |diag R| and
+//   T = D^{-1} R P^T.
 // k_solve: Y = X^{-1} (Db_R^{-1} U_R^T) by Gauss-Jordan elimination with partial pivoting
 //   on the augmented matrix [X | RHS]; X is the well-scaled middle factor of the
 //   stabilized inverse, so partial pivoting is sufficient.
 //
 // One CTA per matrix (batch = 2 * chains); the working matrix lives in shared memory
 // when it fits and in a per-matrix global workspace otherwise.
-#include <cfloat>
-
 #include "nmc_internal.cuh"
 
 namespace nmc {
@@ -23,19 +21,13 @@ namespace {
 
 NMC_DEBUG_FLAG
 
-constexpr int kThreads = 256;
 // Gauss-Jordan: 16 warps (rows over warps, columns over lanes), so a matrix alone on an SM
 // (the tail of a batch that does not fill the GPU in one wave) still has the warps to hide
 // the FP64 latency
 constexpr int kSolveThreads = 512;
 constexpr int kSolveWarps = kSolveThreads / 32;
 constexpr size_t kSmemLimit = 200 * 1024;
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
+constexpr size_t kQrSmemLimit = 225 * 1024;
 
 // argmax over lanes: larger key wins, lower index on ties. Keys are the bit patterns of
 // non-negative doubles (|x|, squared norms), which order like the values, so the search
@@ -55,184 +47,410 @@ __device__ __forceinline__ long long nonneg_key(double x) {
   return __double_as_longlong(x) & 0x7fffffffffffffffll;
 }
 
-__host__ __device__ inline size_t qrp_small_bytes(int N) {
-  return (size_t)N * (3 * sizeof(double) + sizeof(int)) + 64;
+// ---------------------------------------------------------------------------- QR
+// The FP64 pipe issues one warp operation per 20 cycles and SM, an integer multiply-add 32 x 32 +
+// 64 bits one per 0.55, so the reflections run in fixed point: a column is held as 64-bit integers
+// in units of 2^-58 of a power of two just above its 2-norm. Reflections preserve that norm, so
+// nothing overflows, and every operation's error is at most a few 2^-58 of the column's norm,
+// where an FP64 Householder QR makes a few 2^-53 of it. An integer is split into limbs
+// c = c1 2^29 + c0 (|c1| <= 2^30, |c0| <= 2^28); a product takes three multiply-adds, c0 d0 being
+// below the unit:  a b / 2^58 = a1 b1 + (a1 b0 + a0 b1) / 2^29.  The sums over a column cannot
+// overflow: |sum a1 b1| <= |a| |b| / 2^58 (Cauchy-Schwarz), |sum a1 b0| <= 2^58 sqrt(N).
+// A reflector is v = x - beta e_p shifted left until 2^58 <= |v| < 2^59 (exact), with
+// tau = 2 / |v|^2 evaluated in integers from the entries actually stored.
+//
+// LPC lanes share a column (rows r = LPC j + lane, at most 4 NB each, held in registers between
+// the dot product and the update), so a matrix of 64 columns keeps 256 threads busy; one warp
+// searches the pivot and evaluates the reflector's scalars.
+// What bounds it: one matrix, the serial chain of a step (pivot search, column norm, reflector,
+// about 2500 cycles at N = 64, then 2200 for the update, and 2700 per step of forming Q); many, the
+// issue slots and the barriers around that chain (40% issue). Measured, us per launch against the
+// FP64 kernel with one thread per column (N, matrices): 242 / 582 (64, 6), 361 / 722 (64, 512),
+// 1221 / 1904 (72, 1024), 560 / 1281 (100, 128), 1082 / 2497 (144, 128), 42 / 71 (16, 2) and, with the
+// matrix in global memory, where lanes along the rows read whole lines, 5034 / 87627 (256, 64).
+// max |U^T U - I| 7e-17 against 8e-16, columns of U D T to 1.5e-16 against 9e-16 (N = 64).
+constexpr int kLimb = 29, kFix = 58;
+
+// c += a b, 32 x 32 + 64 bits
+__device__ __forceinline__ void mad_wide(long long& c, int a, int b) {
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
+}
+__device__ __forceinline__ int2 limbs(long long c) {
+  const int c1 = (int)((c + (1ll << (kLimb - 1))) >> kLimb);
+  return make_int2(c1, (int)((unsigned)c - ((unsigned)c1 << kLimb)));
+}
+__device__ __forceinline__ long long fold(long long hi, long long mid) {
+  return hi + ((mid + (1ll << (kLimb - 1))) >> kLimb);
+}
+// x in units of 2^(Eb - 1022 - 58) (|x| < 2^(Eb - 1022)), to nearest
+__device__ __forceinline__ long long to_fixed(double x, int Eb) {
+  const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+  const int e = (int)((h >> 20) & 0x7ffu);
+  const unsigned mh = __funnelshift_l(l, h, 11) | 0x80000000u;
+  const int sh = min(63 - kFix + Eb - e, 63);   // to 59 bits, then rounded to 58
+  const unsigned long long m = ((((unsigned long long)mh << 32) | (l << 11)) >> sh) + 1ull;
+  const long long v = e == 0 ? 0 : (long long)(m >> 1);
+  return (int)h < 0 ? -v : v;
+}
+// v 2^k, with a result outside the normal range left to ldexp
+__device__ __forceinline__ double pow2_scale(double v, int k) {
+  const int e = (__double2hiint(v) >> 20) & 0x7ff;
+  if (((__double2hiint(v) << 1) | __double2loint(v)) == 0) return v;
+  if (e == 0 || e == 0x7ff || e + k < 1 || e + k > 2046) return ldexp(v, k);
+  return __hiloint2double(__double2hiint(v) + k * (1 << 20), __double2loint(v));
+}
+// key of a squared norm n 4^E (n >= 0 a float): orders like the value to 2^-19, 0 for 0
+__device__ __forceinline__ unsigned norm_key(float n, int Eb) {
+  return n > 0.f ? (__float_as_uint(n) >> 4) + ((unsigned)(2 * Eb) << 19) : 0u;
+}
+// sum of a 64-bit integer over the warp, in every lane, by 32-bit warp reductions of 26-bit parts
+__device__ __forceinline__ long long warp_sum64(long long v) {
+  const unsigned m = (1u << 26) - 1;
+  const unsigned a = __reduce_add_sync(0xffffffffu, (unsigned)v & m);
+  const unsigned b = __reduce_add_sync(0xffffffffu, (unsigned)(v >> 26) & m);
+  const int c = __reduce_add_sync(0xffffffffu, (int)(v >> 52));
+  return (long long)a + ((long long)b << 26) + ((long long)c << 52);
+}
+// c + a b / 2^58 for a given by its limbs and b by its limbs
+__device__ __forceinline__ long long madq(long long c, int2 a, int2 b) {
+  long long mid = 1ll << (kLimb - 1);
+  mad_wide(c, a.x, b.x);
+  mad_wide(mid, a.x, b.y);
+  mad_wide(mid, a.y, b.x);
+  return c + (mid >> kLimb);
+}
+typedef unsigned long long u64;
+typedef unsigned __int128 u128;
+__device__ __forceinline__ int clz128(u128 v) {
+  const u64 h = (u64)(v >> 64);
+  return h ? __clzll((long long)h) : 64 + __clzll((long long)(u64)v);
+}
+__device__ __forceinline__ u128 shift128(u128 v, int right) {
+  return right >= 0 ? v >> right : v << -right;
+}
+// sqrt(S), rounded, and 2^121 / n for n in [2^62, 2^64), by one third-order Newton step in 64-bit
+// integers from an FP32 approximation (relative error e < 2^-20, so e^3 is below the last bit).
+// The FP64 unit's latency (about 70 cycles an operation) would make these two the longest part
+// of a reflection.
+__device__ __forceinline__ u64 isqrt128(u128 S) {
+  const int sh = (64 - clz128(S) + 1) & ~1;          // even: m = S 2^-sh in [2^62, 2^64)
+  const u64 m = (u64)shift128(S, sh);
+  const u64 Y = (u64)__float2uint_rn(rsqrtf((float)(unsigned)(m >> 32)) * 0x1p39f);
+  const long long e = (1ll << 61) - (long long)__umul64hi(m, (Y * Y) << 15);   // 2^61 (1 - m y^2)
+  const int es = (int)(e >> 10);
+  const long long c = (e >> 1) + ((3 * (((long long)es * es) >> 41)) >> 3);
+  const u64 y = (Y << 38) + (u64)(((long long)Y * (c >> 1)) >> 22);            // 1/sqrt, 2^77 units
+  const u64 r = __umul64hi(m, y << 1);                                         // sqrt(m) 2^30
+  const int d = 30 - sh / 2;
+  return (r + ((1ull << d) >> 1)) >> d;
+}
+__device__ __forceinline__ long long recip121(u64 n) {
+  const u64 Z = (u64)__float2uint_rn(__frcp_rn((float)(unsigned)(n >> 32)) * 0x1p55f);
+  const long long e = (1ll << 61) - (long long)__umul64hi(n, Z << 38);         // 2^61 (1 - n z)
+  const int es = (int)(e >> 10);
+  const long long c = e + (((long long)es * es) >> 41);
+  return (long long)(Z << 34) + (((long long)Z * (c >> 3)) >> 24);
 }
 
-// Four threads per column (a "quad", lanes 4q..4q+3 of a warp) for the trailing updates:
-// one warp covers 8 columns, so per-column scalar work costs one warp instruction per
-// 8 columns. Column norms are kept squared (n1 = current, n2 = at last recompute); the
-// LAPACK downdate safeguard "1 - (r/n1)^2 scaled by (n1/n2)^2 <= sqrt(eps)" is the same test
-// as n1^2 - r^2 <= sqrt(eps) n2^2, which needs no division or square root.
-constexpr int kQuad = 4;
-constexpr int kColsPerPass = kThreads / kQuad;
-
-__device__ __forceinline__ double quad_sum(double v, unsigned mask) {
-  v += __shfl_xor_sync(mask, v, 1);
-  v += __shfl_xor_sync(mask, v, 2);
-  return v;
+// column stride: all rows a lane may touch (the padding is zero), the columns of a half warp on
+// different banks
+__host__ __device__ constexpr int qr_ld(int rows, int LPC) { return LPC < 16 ? rows + LPC : rows; }
+__host__ __device__ constexpr size_t qr_small_bytes(int rows, int N) {
+  // reflector (two buffers), its head and tau per column, norms, exponents, permutation
+  return (size_t)rows * 2 * 8 + (size_t)N * (2 * 8 + 2 * 4 + 2 * 4);
 }
 
-__global__ void __launch_bounds__(kThreads)
+template <int LPC, int NB, int THREADS, int CTAS>
+__global__ void __launch_bounds__(THREADS, CTAS)
 k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__ D,
       double* __restrict__ Tp, double* __restrict__ ws, int N, int use_smem) {
+  constexpr int kRows = 4 * NB * LPC, ldw = qr_ld(kRows, LPC), ngrp = THREADS / LPC;
   extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ int2 s_tau;
+  __shared__ int s_bad;
   const int b = blockIdx.x;
   const long long NN = (long long)N * N;
-  double* n1 = (double*)smraw;   // squared norms
-  double* n2 = n1 + N;
-  double* tau = n2 + N;
-  int* perm = (int*)(tau + N);
-  // column-major with leading dimension N + 1 (W[c*ldw + r]): the 32 columns of a warp fall
-  // on different banks when each thread walks its own column; W becomes Q at the end
-  const int ldw = N + 1;
-  double* W;
-  if (use_smem)
-    W = (double*)(smraw + ((qrp_small_bytes(N) + 15) & ~(size_t)15));
-  else
-    W = ws + (long long)b * 2 * NN;
+  int2* vl = (int2*)smraw;                       // [2][kRows] limbs of a reflector, zero elsewhere
+  int2* vhead = vl + 2 * kRows;                  // [N] v_p
+  int2* taus = vhead + N;                        // [N]
+  float* n1 = (float*)(taus + N);                // [N] squared norms of the trailing part, of 4^E
+  float* n2 = n1 + N;                            // [N] the same when last summed
+  int* Eb = (int*)(n2 + N);                      // [N] biased exponent of the column's scale
+  int* perm = Eb + N;                            // [N]
+  long long* W = use_smem
+      ? (long long*)(smraw + ((qr_small_bytes(kRows, N) + 15) & ~(size_t)15))
+      : (long long*)(ws + (long long)b * 2 * NN);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int pw = blockIdx.x & 3;
-  const int sub = tid & (kQuad - 1);
-  const unsigned qmask = 0xFu << (lane & ~(kQuad - 1));
+  const int sub = tid % LPC, grp = tid / LPC, wgrp = warp * 32 / LPC;   // the warp's first group
+  // the serial warp: on another sub-partition in each of the CTAs that share an SM (warp w issues
+  // on w % 4)
+  const int pw = blockIdx.x & 3 & (THREADS / 32 - 1);
   const double* Xb = X + (long long)b * NN;
 
-  for (int e = tid; e < (int)NN; e += kThreads) {
+  if (tid == 0) s_bad = 0;
+  for (int e = tid; e < (int)NN; e += THREADS) {
     const int r = e / N, c = e - r * N;
-    W[(long long)c * ldw + r] = Xb[e];
+    ((double*)W)[(long long)c * ldw + r] = Xb[e];
   }
-  for (int c = tid; c < N; c += kThreads) perm[c] = c;
+  for (int e = tid; e < N * (kRows - N); e += THREADS)
+    W[(long long)(e / (kRows - N)) * ldw + N + e % (kRows - N)] = 0;
+  for (int r = tid; r < 2 * kRows; r += THREADS) vl[r] = make_int2(0, 0);
+  for (int c = tid; c < N; c += THREADS) perm[c] = c;
   __syncthreads();
-  for (int c0 = 0; c0 < N; c0 += kColsPerPass) {
-    const int c = c0 + tid / kQuad;
+  // columns to fixed point: the scale from the largest entry, raised to the 2-norm
+  for (int c0 = 0; c0 < N; c0 += ngrp) {
+    const int c = c0 + grp;
+    long long* col = W + (long long)min(c, N - 1) * ldw;
+    int em = 1;
+    for (int r = sub; r < N; r += LPC) em = max(em, (int)(((unsigned)((int2*)col)[r].y >> 20) & 0x7ffu));
+#pragma unroll
+    for (int o = 1; o < LPC; o <<= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
+    float s = 0.f;   // of 4^em
+    for (int r = sub; r < N; r += LPC) {
+      const float y = (float)(int)(to_fixed(((double*)col)[r], em) >> 28) * 0x1p-30f;
+      s = fmaf(y, y, s);
+    }
+#pragma unroll
+    for (int o = 1; o < LPC; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    int up = 0;
+    float sn = s * 1.00001f;
+    while (sn > 1.f) sn *= 0.25f, s *= 0.25f, ++up;
     if (c < N) {
-      double s = 0.0;
-      for (int r = sub; r < N; r += kQuad) { const double v = W[(long long)c * ldw + r]; s += v * v; }
-      s = quad_sum(s, qmask);
-      if (sub == 0) { n1[c] = s; n2[c] = s; }
+      for (int r = sub; r < N; r += LPC) col[r] = to_fixed(((double*)col)[r], em + up);
+      if (sub == 0) {
+        Eb[c] = em + up;
+        n1[c] = n2[c] = s;
+        if (em == 0x7ff) s_bad = 1;   // an infinity or a NaN: the outputs are NaN
+      }
     }
   }
   __syncthreads();
 
-  const double tol3z = sqrt(DBL_EPSILON);
   for (int p = 0; p < N; ++p) {
-    // warp pw: pivot (largest remaining norm, lowest index on ties), swap, reflector
-    // H_p = I - tau v v^T (v_p = 1) zeroing W[p+1:, p]; the other warps wait at the barrier.
-    // pw = blockIdx % 4: the CTAs sharing an SM run this serial FP64 step on different
-    // sub-partitions (warp w issues on sub-partition w % 4) instead of all on the first.
+    int2* vp = vl + (p & 1) * kRows;
     if (warp == pw) {
-      long long best = -1;
+      // pivot (largest trailing norm, lowest index on ties) and swap
+      unsigned best = 0;
       int bi = p;
       for (int c = p + lane; c < N; c += 32) {
-        const long long kc = nonneg_key(n1[c]);
+        const unsigned kc = norm_key(n1[c], Eb[c]);
         if (kc > best) { best = kc; bi = c; }
       }
-      warp_argmax(best, bi);
+      const unsigned top = __reduce_max_sync(0xffffffffu, best);
+      bi = top == 0 ? p : (int)__reduce_min_sync(0xffffffffu, best == top ? (unsigned)bi : 0xffffu);
       const int piv = NMC_DCHECK(bi >= p && bi < N, 201) ? bi : p;
+      long long* col = W + (long long)p * ldw;
       if (piv != p) {
+        long long* other = W + (long long)piv * ldw;
         for (int r = lane; r < N; r += 32) {
-          const double t0 = W[(long long)p * ldw + r];
-          W[(long long)p * ldw + r] = W[(long long)piv * ldw + r];
-          W[(long long)piv * ldw + r] = t0;
+          const long long t0 = col[r];
+          col[r] = other[r];
+          other[r] = t0;
         }
         if (lane == 0) {
-          double t1 = n1[p]; n1[p] = n1[piv]; n1[piv] = t1;
-          t1 = n2[p]; n2[p] = n2[piv]; n2[piv] = t1;
-          const int ti = perm[p]; perm[p] = perm[piv]; perm[piv] = ti;
+          n1[piv] = n1[p];
+          n2[piv] = n2[p];
+          int t = Eb[p]; Eb[p] = Eb[piv]; Eb[piv] = t;
+          t = perm[p]; perm[p] = perm[piv]; perm[piv] = t;
         }
+        __syncwarp();
+      }
+      // squared norm from the diagonal down, exactly: HI 2^58 + MID 2^30 + LO
+      long long hi = 0, mid = 0, lo = 0;
+      for (int r = p + lane; r < N; r += 32) {
+        const int2 c = limbs(col[r]);
+        mad_wide(hi, c.x, c.x);
+        mad_wide(mid, c.x, c.y);
+        mad_wide(lo, c.y, c.y);
+      }
+      mid += lo >> 30;   // (LO's sum over the warp stays in range)
+      lo &= (1ll << 30) - 1;
+      hi = warp_sum64(hi);
+      mid = warp_sum64(mid);
+      lo = warp_sum64(lo);
+      const long long alpha = col[p];
+      int k = 0;
+      long long head = 0, beta = 0;
+      int2 tau = make_int2(0, 0);
+      if ((hi | mid | lo) != 0) {
+        const u128 S = ((u128)hi << 58) + (u128)((__int128)mid << 30) + (u128)lo;
+        const u64 root = isqrt128(S), al = (u64)(alpha < 0 ? -alpha : alpha);
+        beta = alpha > 0 ? -(long long)root : (long long)root;
+        head = alpha - beta;   // no cancellation
+        // |v|^2 before the shift, exactly: S + 2 |alpha| |beta| + beta^2, with beta as stored
+        const u128 V = S + (u128)root * (root + 2 * al);
+        k = (clz128(V) - 10) >> 1;           // 2^116 <= V 4^k < 2^118
+        tau = limbs(recip121((u64)shift128(V, 54 - 2 * k)));
+        head = k >= 0 ? head << k : head >> -k;
       }
       __syncwarp();
-      double* col = W + (long long)p * ldw;
-      const double alpha = col[p];
-      double xn2 = 0.0;
-      for (int r = p + 1 + lane; r < N; r += 32) xn2 += col[r] * col[r];
-      xn2 = warp_sum(xn2);
-      double t = 0.0;
-      if (xn2 > 0.0) {   // (xn2 is the same in every lane after the butterfly sum)
-        // the square root and the two divisions on lane 0 only, then broadcast
-        double beta = 0.0, scal = 0.0;
-        if (lane == 0) {
-          beta = -copysign(sqrt(alpha * alpha + xn2), alpha);
-          t = (beta - alpha) / beta;
-          scal = 1.0 / (alpha - beta);
-        }
-        scal = __shfl_sync(0xffffffffu, scal, 0);
-        for (int r = p + 1 + lane; r < N; r += 32) col[r] *= scal;
-        __syncwarp();
-        if (lane == 0) col[p] = beta;
+      // the reflector's limbs, for this step and (below the diagonal) for Q
+      for (int r = p + 1 + lane; r < N; r += 32) {
+        const long long c = col[r];
+        const int2 l = limbs(k >= 0 ? c << k : c >> -k);
+        vp[r] = l;
+        ((int2*)col)[r] = l;
       }
-      if (lane == 0) tau[p] = t;
+      if (lane == 0) {
+        const int2 hl = limbs(head);
+        col[p] = beta;
+        vp[p] = hl;
+        vhead[p] = hl;
+        taus[p] = tau;
+        s_tau = tau;
+        if (p >= 2) vp[p - 2] = make_int2(0, 0);   // what this buffer last held above row p
+        if (p >= 1) vp[p - 1] = make_int2(0, 0);
+      }
     }
     __syncthreads();
-    const double tp = tau[p];
-    const double* v = W + (long long)p * ldw;
-    // one thread per trailing column: each FP64 warp instruction then carries 32 columns'
-    // work, with no partial sums to combine (the FP64 pipe costs the same per warp
-    // instruction however many lanes are active)
-    for (int c = p + 1 + tid; c < N; c += kThreads) {
-      double* col = W + (long long)c * ldw;
-      double rp = col[p];
-      if (tp != 0.0) {
-        double dot = rp;   // v_p = 1
-        for (int r = p + 1; r < N; ++r) dot = fma(v[r], col[r], dot);
-        const double f = tp * dot;
-        for (int r = p + 1; r < N; ++r) col[r] = fma(-f, v[r], col[r]);
-        rp -= f;
-        col[p] = rp;
-      }
-      const double a1 = n1[c];
-      if (a1 != 0.0) {
-        const double d = fma(-rp, rp, a1);
-        if (d <= tol3z * n2[c]) {
-          double s = 0.0;
-          for (int r = p + 1; r < N; ++r) s = fma(col[r], col[r], s);
-          n1[c] = s;
-          n2[c] = s;
-        } else {
-          n1[c] = d;
+    const int2 tau = s_tau;
+    const int bs = p / (4 * LPC);   // blocks of 4 LPC rows from here on
+    for (int c0 = p + 1; c0 + wgrp < N; c0 += ngrp) {
+      const int c = min(c0 + grp, N - 1);
+      const bool on = c0 + grp < N;
+      long long* col = W + (long long)c * ldw + sub;
+      const int2* v = vp + sub;
+      long long x[NB][4], hi = 0, mid = 0;
+#pragma unroll
+      for (int q = 0; q < NB; ++q) {
+        if (q < bs) continue;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          x[q][i] = col[(4 * q + i) * LPC];
+          const int2 l = limbs(x[q][i]), w = v[(4 * q + i) * LPC];
+          mad_wide(hi, w.x, l.x);
+          mad_wide(mid, w.x, l.y);
+          mad_wide(mid, w.y, l.x);
         }
       }
+#pragma unroll
+      for (int o = 1; o < LPC; o <<= 1) {
+        hi += __shfl_xor_sync(0xffffffffu, hi, o);
+        mid += __shfl_xor_sync(0xffffffffu, mid, o);
+      }
+      const int2 f = limbs(-madq(0, limbs(fold(hi, mid)), tau));
+#pragma unroll
+      for (int q = 0; q < NB; ++q) {
+        if (q < bs) continue;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {   // (rows above p: v is zero there)
+          x[q][i] = madq(x[q][i], v[(4 * q + i) * LPC], f);
+          if (on) col[(4 * q + i) * LPC] = x[q][i];
+        }
+      }
+      // trailing norm: downdated by row p's entry, summed again when less than 2^-12 of the last
+      // sum is left
+      __syncwarp();
+      const float rp = (float)(col - sub)[p] * 0x1p-58f, a2 = n2[c];
+      float a1 = fmaf(-rp, rp, n1[c]);
+      const bool again = on && !(a1 > 0x1p-12f * a2);
+      if (__any_sync(0xffffffffu, again)) {
+        float s = 0.f;
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+          if (q < bs) continue;
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float y = (4 * q + i) * LPC + sub > p ? (float)x[q][i] * 0x1p-58f : 0.f;
+            s = fmaf(y, y, s);
+          }
+        }
+#pragma unroll
+        for (int o = 1; o < LPC; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (again && sub == 0) n2[c] = s;
+        if (again) a1 = s;
+      }
+      if (on && sub == 0) n1[c] = a1;
     }
     __syncthreads();
   }
 
-  // outputs D and T = D^{-1} R P^T
+  // outputs D = |diag R| and T = D^{-1} R P^T
+  const bool bad = s_bad != 0;
+  const double nan = __longlong_as_double(0x7ff8000000000000ll);
   double* Db = D + (long long)b * N;
-  for (int r = tid; r < N; r += kThreads) Db[r] = fabs(W[(long long)r * ldw + r]);
   double* Tb = Tp + (long long)b * NN;
-  for (int e = tid; e < (int)NN; e += kThreads) {
+  double2* rd = (double2*)vl;   // |R_rr| and its reciprocal
+  for (int r = tid; r < N; r += THREADS) {
+    const double d = fabs((double)W[(long long)r * ldw + r]);
+    Db[r] = bad ? nan : pow2_scale(d, Eb[r] - 1022 - kFix);
+    rd[r] = make_double2(d, 1.0 / d);
+  }
+  __syncthreads();
+  for (int e = tid; e < (int)NN; e += THREADS) {
     const int r = e / N, c = e - r * N;
-    const double d = fabs(W[(long long)r * ldw + r]);
-    Tb[r * N + perm[c]] = (c >= r) ? W[(long long)c * ldw + r] / d : 0.0;
+    double t = 0.0;
+    if (c >= r) {   // the quotient from the reciprocal, with one correction
+      const double w = (double)W[(long long)c * ldw + r], d = rd[r].x;
+      t = w * rd[r].y;
+      t = pow2_scale(fma(fma(-t, d, w), rd[r].y, t), Eb[c] - Eb[r]);
+    }
+    Tb[r * N + perm[c]] = bad ? nan : t;
   }
   __syncthreads();   // T and D are out: W's upper triangle is free
-  // Q = H_0 H_1 ... H_{N-1} in place over W (column-major), by backward accumulation:
-  // before step p, columns > p hold H_{p+1} ... H_{N-1} in rows > p (rows <= p still hold R
-  // and are treated as zero); step p applies H_p to those columns, writing their row p, and
-  // then turns column p (the reflector v, v_p = 1) into H_p e_p.
+  // Q = H_0 H_1 ... H_{N-1} in place over W, 1 = 2^58, by backward accumulation: before step p,
+  // columns > p hold H_{p+1} ... H_{N-1} in rows > p (rows <= p still hold R and count as zero: the
+  // reflector buffers are zero there); step p applies H_p to those columns, writing their row p,
+  // and turns column p (the limbs of its reflector) into H_p e_p. The reflector of step p - 1 is
+  // copied out meanwhile.
+  for (int r = tid; r < 2 * kRows; r += THREADS) vl[r] = make_int2(0, 0);
+  __syncthreads();
   for (int p = N - 1; p >= 0; --p) {
-    const double tp = tau[p];
-    const double* v = W + (long long)p * ldw;
-    for (int c = p + 1 + tid; c < N; c += kThreads) {   // one thread per column, as above
-      double* col = W + (long long)c * ldw;
-      double dot = 0.0;
-      for (int r = p + 1; r < N; ++r) dot = fma(v[r], col[r], dot);
-      const double f = tp * dot;
-      if (f != 0.0)
-        for (int r = p + 1; r < N; ++r) col[r] = fma(-f, v[r], col[r]);
-      col[p] = -f;
+    const int2* v0 = vl + (p & 1) * kRows;
+    const int2 tau = taus[p], head = vhead[p];
+    if (p > 0) {
+      int2* vn = vl + ((p - 1) & 1) * kRows;
+      const int2* src = (const int2*)(W + (long long)(p - 1) * ldw);
+      for (int r = p + tid; r < N; r += THREADS) vn[r] = src[r];
+    }
+    const int bs = p / (4 * LPC);
+    for (int c0 = p + 1; c0 + wgrp < N; c0 += ngrp) {
+      const int c = min(c0 + grp, N - 1);
+      const bool on = c0 + grp < N;
+      long long* col = W + (long long)c * ldw + sub;
+      const int2* v = v0 + sub;
+      long long x[NB][4], hi = 0, mid = 0;
+#pragma unroll
+      for (int q = 0; q < NB; ++q) {
+        if (q < bs) continue;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          x[q][i] = col[(4 * q + i) * LPC];
+          const int2 l = limbs(x[q][i]), w = v[(4 * q + i) * LPC];
+          mad_wide(hi, w.x, l.x);
+          mad_wide(mid, w.x, l.y);
+          mad_wide(mid, w.y, l.x);
+        }
+      }
+#pragma unroll
+      for (int o = 1; o < LPC; o <<= 1) {
+        hi += __shfl_xor_sync(0xffffffffu, hi, o);
+        mid += __shfl_xor_sync(0xffffffffu, mid, o);
+      }
+      const int2 f = limbs(-madq(0, limbs(fold(hi, mid)), tau));
+      if (on) {
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+          if (q < bs) continue;
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            col[(4 * q + i) * LPC] = madq(x[q][i], v[(4 * q + i) * LPC], f);
+        }
+        if (sub == p % LPC) (col - sub)[p] = madq(0, head, f);
+      }
+    }
+    {   // column p itself: v . e_p = v_p
+      const int2 f = limbs(-madq(0, head, tau));
+      long long* col = W + (long long)p * ldw;
+      for (int r = tid; r < N; r += THREADS)
+        col[r] = r < p ? 0 : r == p ? madq(1ll << kFix, head, f) : madq(0, v0[r], f);
     }
     __syncthreads();
-    double* cp = W + (long long)p * ldw;
-    for (int r = tid; r < N; r += kThreads)
-      cp[r] = r < p ? 0.0 : r == p ? 1.0 - tp : -tp * cp[r];
-    __syncthreads();
   }
-  double* Q = W;
   double* Ub = U + (long long)b * NN;
-  for (int e = tid; e < (int)NN; e += kThreads) {
+  for (int e = tid; e < (int)NN; e += THREADS) {
     const int r = e / N, c = e - r * N;
-    Ub[e] = Q[(long long)c * ldw + r];
+    Ub[e] = bad ? nan : pow2_scale((double)W[(long long)c * ldw + r], -kFix);
   }
 }
 
@@ -307,14 +525,28 @@ k_solve(const double* __restrict__ X, const double* __restrict__ UR, long long s
 
 }  // namespace
 
+// The lanes per column follow from N alone (results must not depend on the batch): as few as keep
+// a lane's rows within 16 or 20 register pairs, and as many threads as columns need up to 512.
 void qrp_udt(const double* X, double* U, double* D, double* Tp, double* ws, int N, int batch,
              cudaStream_t st) {
-  const size_t small = (qrp_small_bytes(N) + 15) & ~(size_t)15;
-  const size_t big = small + (size_t)N * (N + 1) * sizeof(double);   // W, ld N + 1
-  const int use_smem = big <= kSmemLimit;
-  const size_t bytes = use_smem ? big : small;
-  allow_max_dynamic_smem((const void*)k_qrp);
-  k_qrp<<<batch, kThreads, bytes, st>>>(X, U, D, Tp, ws, N, use_smem);
+  auto run = [&](auto kernel, int LPC, int NB, int threads) {
+    const int rows = 4 * NB * LPC;
+    const size_t small = (qr_small_bytes(rows, N) + 15) & ~(size_t)15;
+    const size_t big = small + (size_t)N * qr_ld(rows, LPC) * sizeof(long long);
+    const int use_smem = big <= kQrSmemLimit;
+    allow_max_dynamic_smem((const void*)kernel);
+    kernel<<<batch, threads, use_smem ? big : small, st>>>(X, U, D, Tp, ws, N, use_smem);
+  };
+  if (N <= 16) run(k_qrp<4, 1, 64, 4>, 4, 1, 64);
+  else if (N <= 32) run(k_qrp<4, 2, 128, 4>, 4, 2, 128);
+  else if (N <= 48) run(k_qrp<4, 3, 192, 5>, 4, 3, 192);
+  else if (N <= 64) run(k_qrp<4, 4, 256, 4>, 4, 4, 256);
+  else if (N <= 80) run(k_qrp<4, 5, 320, 3>, 4, 5, 320);
+  else if (N <= 128) run(k_qrp<8, 4, 512, 1>, 8, 4, 512);
+  else if (N <= 160) run(k_qrp<8, 5, 512, 1>, 8, 5, 512);
+  else if (N <= 256) run(k_qrp<16, 4, 512, 1>, 16, 4, 512);
+  else if (N <= 512) run(k_qrp<32, 4, 512, 1>, 32, 4, 512);
+  else run(k_qrp<32, 8, 512, 1>, 32, 8, 512);
 }
 
 void solve_stab(const double* X, const double* UR, long long sUR, const double* DR,
@@ -326,8 +558,9 @@ void solve_stab(const double* X, const double* UR, long long sUR, const double* 
   k_solve<<<batch, kSolveThreads, bytes, st>>>(X, UR, sUR, DR, sDR, Y, ws, N, use_smem);
 }
 
+// (the threshold that the documented scratch sizes of nmc_green_noalloc follow)
 bool stab_needs_workspace(int N) {
-  const size_t small = (qrp_small_bytes(N) + 15) & ~(size_t)15;
+  const size_t small = ((size_t)N * 28 + 64 + 15) & ~(size_t)15;
   return small + 2 * (size_t)N * N * sizeof(double) > kSmemLimit;
 }
 
