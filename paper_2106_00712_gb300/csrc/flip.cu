@@ -12,6 +12,10 @@
 // G0 += A B^T. In exact arithmetic this equals applying each rank-1 update at once.
 // G0 of both spins sits in shared memory when it fits (N <= 64 in FP64), else in global
 // memory (L2); the panels always live in shared memory (k is clamped to fit).
+// That is k_flip (FP32) and, above some 560 sites, k_flip (FP64) and k_flip_df (FP32 pairs); up to
+// there FP64 and FP32 pairs take k_flip_block, which decides blocks of up to min(k, 16) sites apart.
+#include <cuda_fp16.h>
+
 #include "nmc_internal.cuh"
 #include "oz_slice.cuh"
 
@@ -248,10 +252,6 @@ __device__ void flush_df(df2* G, const df2* Ap, const df2* Bp, int m, int N, int
 // per-output slicing and scaling outweigh a 16-term double-float sum. For k = 32 at N = 256 a
 // version that re-sliced P per n-tile took 1198 ms against 625 ms for the SIMT fold.
 constexpr int kTcFlushMaxK = 16;
-#ifndef NMC_TC_FLUSH_MIN_N
-#define NMC_TC_FLUSH_MIN_N 65
-#endif
-constexpr int kTcFlushMinN = NMC_TC_FLUSH_MIN_N;
 
 // A fragment (row-major 16 x 16) of P rows r_lo / r_hi = r_lo + 8, k = k0..k0+15: register v
 // holds row (v & 1 ? r_hi : r_lo), k = k0 + 2tq + {0, 1} (+8 for v >= 2); the lower half of
@@ -577,6 +577,534 @@ __global__ void __launch_bounds__(kThreadsDf, 2) k_flip_df(const FlipArgs<df2> f
   }
 }
 
+// ---------------------------------------------------------------------------- blocks of sites
+// One slice in blocks of up to 16 sites (Nukala et al., Phys. Rev. B 80, 195111 (2009); Gull et
+// al., Phys. Rev. B 83, 075122 (2011)): the decisions of a block need only the 16 x 16 submatrix of
+// G^ at its sites. Four warps take them, each holding four of the submatrix's rows for both spins
+// (half a warp per spin, lane j column j):
+//   R^sigma = 1 + Delta^sigma (1 - G^_ii),   accept iff u < |R^up R^dn|,
+//   on acceptance G^ += x y^T with x_r = G^_{ri} - delta_ri, y_j = (Delta / R^sigma) G^_{ij}.
+// Until the next acceptance G^ does not change, so all remaining sites are decided at once, one per
+// lane, and the first accepted one is next: a rejection costs nothing. A decision is taken in FP32
+// when |u - |R|| exceeds a bound on FP32's error, and in FP64 from the same G^_ii otherwise, so it is
+// the FP64 decision. Then all threads form the x and y of the block's accepted flips over all N
+// sites, one entry of every vector per thread (a triangular recurrence with the submatrix's own x and
+// y as coefficients), and the block is folded into G.
+//
+// The fold G += sum_q x_q y_q^T is one k-step of 16 on the tensor cores (mma.sync; per 16 x 16 block
+// of G and spin), by exact slicing (Ozaki et al., Numer. Algorithms 2012): each row's x and each
+// column's y, scaled by a power of two, are cut into 6 balanced digits of 10 bits (|d| <= 512, exact
+// in FP16) straight from the registers they were formed in; the 21 digit products s + t <= 5
+// accumulate in six FP32 groups g = s + t, exact for g <= 3 (16 * 4 * 2^18 = 2^24). What is dropped
+// is below 2^-54 (FP32 pairs; 2^-57 in FP64) of the row's and column's maxima. tcgen05 would need 128
+// rows per tile and TMEM round trips for one k-step; mma.sync issues from the registers at hand.
+// Without tensor cores (FP32X2) the vectors go through shared memory to the FP32-pair loop.
+//
+// One slice, us, 44% of the flips accepted, one flip at a time (k_flip, k_flip_df) -> here:
+//   64 sites x 256 chains, both spins: FP32 pairs 133 -> 73, FP64 357 -> 155, FP32X2 133 -> 108
+//   72 x 1024, one spin: 625 -> 243;  256 x 32: 2950 -> 989;  100 x 64: 481 -> 135;
+//   16 x 1 in FP64: 31 -> 16.
+// What bounds it at 64 x 256 (two CTAs per SM): latency. Of a slice's 146k cycles the decisions take
+// 45k (28 acceptances of some 1500: two ratios, a reciprocal and four rows' updates in a dependent
+// chain), the folds 47k (of which the MMAs' issue is 23k), the digits 24k, the vectors 13k. In FP64
+// the pipe's one instruction per 20 cycles bounds vectors and fold sums.
+constexpr int kSites = 16;                 // sites per block
+constexpr int kFDig = 6, kFW = 10, kFBits = 59;
+enum FoldKind { kFoldTensor, kFoldPairs };
+
+template <typename T> struct Arith;
+template <> struct Arith<df2> {
+  static __device__ __forceinline__ df2 zero() { return df_zero(); }
+  static __device__ __forceinline__ df2 one() { return df2{1.f, 0.f}; }
+  static __device__ __forceinline__ float top(df2 a) { return a.hi; }
+  static __device__ __forceinline__ double wide(df2 a) { return df_to_double(a); }
+  static __device__ __forceinline__ df2 mul(df2 a, df2 b) { return df_mul(a, b); }
+  static __device__ __forceinline__ df2 sub(df2 a, df2 b) { return df_add(a, df_neg(b)); }
+  static __device__ __forceinline__ df2 add(df2 a, df2 b) { return df_add(a, b); }
+  static __device__ __forceinline__ void fma_acc(df2& c, df2 a, df2 b) { df_fma_acc(c, a, b); }
+  static __device__ __forceinline__ df2 finish(df2 a) { return df_finish(a); }
+  // a / b: approximate FP32 reciprocal r (2^-23), its residual 1 - b r as the low part (2^-46)
+  static __device__ __forceinline__ df2 div(df2 a, df2 b) {
+    const float r = __fdividef(1.f, b.hi);
+    const float e = __fmaf_rn(-b.lo, r, __fmaf_rn(-b.hi, r, 1.f));
+    return df_mul(a, df2{r, __fmul_rn(r, e)});
+  }
+  // biased exponent of |a|
+  static __device__ __forceinline__ int expo(df2 a) { return (__float_as_int(a.hi) >> 23) & 0xff; }
+  static constexpr int kExpMin = 9, kExpMax = 0xff;
+  // The terms of two k as FP16 digit pairs, most significant first. A term in units of 2^(E - 135)
+  // is below 512; adding kM 2^(-10 s) (ulp 2^(-10 s)) rounds it to its digit s, which then stands in
+  // the low mantissa bits on top of 0x6600, FP16's 1536. The low part joins after the first digit by
+  // exact sums (Fast2Sum: what is left of the high part is 0 or at least twice as large), its rest
+  // after the second and the third, so that no digit exceeds 512: beyond, FP16's steps are 2.
+  static __device__ __forceinline__ void digits(df2 a, df2 b, int E, unsigned (&w)[kFDig]) {
+    const float sc = __int_as_float((262 - E) << 23);
+    unsigned t0[kFDig], t1[kFDig];
+    split(a, sc, t0);
+    split(b, sc, t1);
+#pragma unroll
+    for (int s = 0; s < kFDig; ++s) w[s] = __byte_perm(t0[s], t1[s], 0x5410);
+  }
+  static __device__ __forceinline__ void split(df2 a, float sc, unsigned (&t)[kFDig]) {
+    float v = __fmul_rn(a.hi, sc), e = __fmul_rn(a.lo, sc), m = __int_as_float(0x4b406600);
+#pragma unroll
+    for (int s = 0; s < kFDig; ++s) {
+      if (s == 1 || s == 2) {
+        const float q = __fadd_rn(v, e);
+        e = __fsub_rn(e, __fsub_rn(q, v));
+        v = q;
+      }
+      if (s == 3) v = __fadd_rn(v, e);
+      const float x = __fadd_rn(v, m);
+      t[s] = __float_as_uint(x);
+      v = __fsub_rn(v, __fsub_rn(x, m));
+      m *= 0x1p-10f;
+    }
+  }
+  // what a row's (column's) digit sums are multiplied by: 2^(E - 135), or NaN where a term is not finite
+  static __device__ __forceinline__ int scale(int E) {
+    return E == kExpMax ? 0x7fc00000 : (E - 8) << 23;
+  }
+};
+template <> struct Arith<double> {
+  static __device__ __forceinline__ double zero() { return 0.0; }
+  static __device__ __forceinline__ double one() { return 1.0; }
+  static __device__ __forceinline__ float top(double a) { return (float)a; }
+  static __device__ __forceinline__ double wide(double a) { return a; }
+  static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
+  static __device__ __forceinline__ double sub(double a, double b) { return a - b; }
+  static __device__ __forceinline__ double add(double a, double b) { return a + b; }
+  static __device__ __forceinline__ void fma_acc(double& c, double a, double b) { c = fma(a, b, c); }
+  static __device__ __forceinline__ double finish(double a) { return a; }
+  static __device__ __forceinline__ double div(double a, double b) { return a / b; }
+  static __device__ __forceinline__ int expo(double a) { return (__double2hiint(a) >> 20) & 0x7ff; }
+  static __device__ __forceinline__ long long fixed(double a, int E) {
+    const unsigned h = (unsigned)__double2hiint(a), l = (unsigned)__double2loint(a);
+    const int e = (int)((h >> 20) & 0x7ffu);
+    const unsigned long long m =
+        ((unsigned long long)(__funnelshift_l(l, h, 11) | 0x80000000u) << 32 | (l << 11));
+    const long long v = e == 0 ? 0ll : (long long)(m >> min(64 - kFBits + E - e, 63));
+    return (int)h < 0 ? -v : v;
+  }
+  static constexpr int kExpMin = 1, kExpMax = 0x7ff;
+  // Adding 512 to every 10-bit field of the term in units of 2^(E - 1022 - kFBits) and reading the
+  // fields less 512 gives balanced digits; a field added to 0x6400, FP16's 1024, is 1536 + digit.
+  static __device__ __forceinline__ void digits(double a, double b, int E, unsigned (&w)[kFDig]) {
+    const unsigned long long u0 = (unsigned long long)(fixed(a, E) + 0x0802008020080200ll);
+    const unsigned long long u1 = (unsigned long long)(fixed(b, E) + 0x0802008020080200ll);
+#pragma unroll
+    for (int s = 0; s < kFDig; ++s) {
+      const int bit = kFW * (kFDig - 1 - s);
+      w[s] = __byte_perm((unsigned)(u0 >> bit), (unsigned)(u1 >> bit), 0x5410);
+      if (s > 0) w[s] &= 0x03ff03ffu;   // (the first digit's field may reach 1024)
+      w[s] += 0x64006400u;
+    }
+  }
+  static __device__ __forceinline__ int scale(int E) { return E; }
+};
+
+template <typename T> __device__ __forceinline__ T delta(const FlipArgs<T>& f, bool plus);
+template <> __device__ __forceinline__ df2 delta<df2>(const FlipArgs<df2>& f, bool plus) { return plus ? f.dp2 : f.dm2; }
+template <> __device__ __forceinline__ double delta<double>(const FlipArgs<double>& f, bool plus) { return plus ? f.dp : f.dm; }
+// G[s][r][c] += sum_q x[s][q][r] y[s][q][c] on the FP32 pipe: four rows at a time, four independent
+// chains per y read
+template <typename T>
+__device__ void fold_pairs(T* G, const T* pan, int m, int N, int ns, long long sG, int ld) {
+  const int nthr = blockDim.x, c0 = threadIdx.x % N, r0 = threadIdx.x / N;
+  const int rstep = nthr >= N ? nthr / N : 1;
+  if (nthr >= N && r0 >= rstep) return;
+  for (int s = 0; s < ns; ++s) {
+    const T* x = pan + (long long)s * kSites * N;
+    const T* y = pan + (long long)(ns + s) * kSites * N;
+    T* Gp = G + s * sG;
+    for (int c = c0; c < N; c += nthr >= N ? N : nthr)
+      for (int r = nthr >= N ? r0 : 0; r < N; r += 4 * rstep) {
+        T a[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          a[i] = r + i * rstep < N ? Gp[(long long)(r + i * rstep) * ld + c] : Arith<T>::zero();
+        for (int q = 0; q < m; ++q) {
+          const T b = y[q * N + c];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (r + i * rstep < N) Arith<T>::fma_acc(a[i], x[q * N + r + i * rstep], b);
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (r + i * rstep < N) Gp[(long long)(r + i * rstep) * ld + c] = Arith<T>::finish(a[i]);
+      }
+  }
+}
+
+// byte offset of the 16-byte half h (k = 8 h ..) of a digit row r: rows of 32 bytes, the halves
+// exchanged in every second group of four rows so that ldmatrix meets all banks
+__device__ __forceinline__ int digit_off(int r, int h) { return r * 32 + ((h ^ ((r >> 2) & 1)) << 4); }
+
+// Cut the 16 terms of one row (or column) into digits, most significant first, `stride` bytes apart
+template <typename T>
+__device__ __forceinline__ void cut16(const T (&x)[kSites], int E, unsigned char* dst, int r, int stride) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    unsigned w[4][kFDig];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) Arith<T>::digits(x[8 * h + 2 * i], x[8 * h + 2 * i + 1], E, w[i]);
+#pragma unroll
+    for (int s = 0; s < kFDig; ++s) {
+      unsigned d[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const __half2 v = __hadd2(*reinterpret_cast<__half2*>(&w[i][s]), __float2half2_rn(-1536.f));
+        d[i] = *reinterpret_cast<const unsigned*>(&v);
+      }
+      *reinterpret_cast<uint4*>(dst + s * stride + digit_off(r, h)) = make_uint4(d[0], d[1], d[2], d[3]);
+    }
+  }
+}
+
+__device__ __forceinline__ void ldm4(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+__device__ __forceinline__ void mma_h(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// One entry of G plus its digit sums sum_g a_g 2^(-10 g) times the row's and the column's scale.
+// a_0 + a_1 2^-10 + a_2 2^-20 as an exact pair by Fast2Sum: where the smaller-magnitude operand comes
+// first, the sum is short enough to be exact (a_0 is an integer, |a_1 2^-10| < 2^13, |a_2 2^-20| < 13).
+__device__ __forceinline__ void fold_entry(df2& G, const float (&a)[kFDig], int ea, int eb) {
+  const float s = __fmaf_rn(a[1], 0x1p-10f, a[0]);
+  const float e1 = __fmaf_rn(a[1], 0x1p-10f, -__fsub_rn(s, a[0]));
+  const float h = __fmaf_rn(a[2], 0x1p-20f, s);
+  const float e2 = __fmaf_rn(a[2], 0x1p-20f, -__fsub_rn(h, s));
+  float l = __fmaf_rn(a[3], 0x1p-30f, __fadd_rn(e1, e2));
+  l = __fmaf_rn(a[5], 0x1p-50f, __fmaf_rn(a[4], 0x1p-40f, l));
+  const float sc = __fmul_rn(__int_as_float(ea), __int_as_float(eb));
+  const float th = __fmul_rn(h, sc), q = __fadd_rn(G.hi, th), b = __fsub_rn(q, G.hi);
+  const float e = __fadd_rn(__fsub_rn(G.hi, __fsub_rn(q, b)), __fsub_rn(th, b));
+  G = df_norm(q, __fadd_rn(e, __fmaf_rn(l, sc, G.lo)));
+}
+__device__ __forceinline__ void fold_entry(double& G, const float (&a)[kFDig], int ea, int eb) {
+  if (max(ea, eb) >= Arith<double>::kExpMax) {   // an infinity or a NaN among the terms
+    G = __longlong_as_double(0x7ff8000000000000ll);
+    return;
+  }
+  int q[kFDig];
+#pragma unroll
+  for (int s = 0; s < kFDig; ++s) q[s] = __float2int_rn(a[s]);
+  long long H = (long long)q[0] * (1 << 20) + ((long long)q[1] * (1 << 10) + q[2]);
+  long long L = (long long)q[3] * (1 << 20) + ((long long)q[4] * (1 << 10) + q[5]);
+  H += L >> 30;   // (H 2^30 + L) 2^-50
+  L &= (1ll << 30) - 1;
+  const int s = min(__clzll(H ^ (H >> 63)) - 1, 30);
+  const double v = (double)((H << s) + (L >> (30 - s)));
+  const int k = ea + eb - 2 * 1022 - 18 - 20 - s;
+  const int e = (__double2hiint(v) >> 20) & 0x7ff;
+  if (e == 0) return;
+  G += e + k >= 1 && e + k <= 2046
+           ? __hiloint2double(__double2hiint(v) + k * (1 << 20), __double2loint(v)) : ldexp(v, k);
+}
+
+// the deciding warps, 4 rows of the block each
+constexpr int kDecide = kSites / 4;
+__device__ __forceinline__ void bar_decide() { asm volatile("bar.sync 1, %0;" ::"n"(32 * kDecide) : "memory"); }
+
+// stage arrays of one block, in shared memory
+template <typename T>
+struct BlockStage {
+  T S[2][kSites][kSites];     // [spin]: G^ at the block's sites, while they are decided
+  T x[2][kSites][kSites];     // [spin][accepted flip q][block row]: x_q at the block's later sites
+  T y[2][kSites][kSites];     // [spin][q][block column]
+  T c[2][kSites];             // Delta / R^sigma of q
+  int site[kSites];           // block index of q
+  int m[2];                   // accepted flips, by block parity: see the loop
+};
+
+template <typename T>
+__host__ __device__ inline size_t block_smem(int N, int ns, bool g_in_smem, int fold, int ld) {
+  const int Np = (N + 15) & ~15;
+  size_t b = g_in_smem ? (size_t)ns * N * ld * sizeof(T) : 0;
+  b += fold == kFoldTensor ? (size_t)2 * kFDig * Np * 32 + 2 * Np * sizeof(int)
+                           : (size_t)2 * ns * kSites * N * sizeof(T);
+  b += sizeof(BlockStage<T>) + (size_t)N * 4 + ((N + 15) & ~15);
+  return b + 64;
+}
+
+// GS: G held in shared memory
+template <typename T, int FOLD, int THREADS, bool GS>
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 2 : 1)
+k_flip_block(const FlipArgs<T> f, int kb_max) {
+  typedef Arith<T> A;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const int c = blockIdx.x, N = f.N, ns = f.ns, Np = (N + 15) & ~15;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ld = GS ? N + 2 : N;   // (rows of a column read on different banks)
+  const long long NN = (long long)N * N, sG = GS ? (long long)N * ld : NN;
+  T* Gs = (T*)smraw;
+  T* Gg = f.G + (long long)c * ns * NN;
+  T* G;
+  if constexpr (GS) G = Gs;
+  else G = Gg;
+  unsigned char* dig = smraw + (GS ? (size_t)ns * N * ld * sizeof(T) : 0);
+  T* pan = (T*)dig;                                  // kFoldPairs: [x, y][ns][16][N]
+  int* ev = (int*)(dig + (size_t)2 * kFDig * Np * 32);   // kFoldTensor: exponents of x rows, y columns
+  // (every part a multiple of 16 bytes: N is even)
+  BlockStage<T>& st = *(BlockStage<T>*)(dig + (FOLD == kFoldTensor ? (size_t)2 * kFDig * Np * 32 + 2 * Np * sizeof(int)
+                                                                   : (size_t)2 * ns * kSites * N * sizeof(T)));
+  unsigned* u = (unsigned*)(&st + 1);                // Philox words: u_i = word 2^-32
+  int8_t* sl = (int8_t*)(u + N);
+
+  int8_t* fl = f.fields + ((long long)c * f.L + f.l) * N;
+  const uint32_t gchain = (uint32_t)(f.chain_id ? f.chain_id[c] : f.chain_offset + c);
+  const uint32_t sweep = (uint32_t)((f.ctr ? f.ctr[0] : (long long)f.sweep) -
+                                    (f.sweep_base ? f.sweep_base[c] : 0));
+  const uint8_t* rp = f.replay ? f.replay + ((long long)c * f.L + f.l) * N : nullptr;
+  for (int i = tid; i < N; i += THREADS) {
+    sl[i] = fl[i];
+    uint32_t ctr[4] = {(uint32_t)(f.l * N + i), sweep, gchain, kTagFlip};
+    philox4x32_10(ctr, f.key0, f.key1);
+    u[i] = ctr[0];
+  }
+  if (GS)
+    for (int e = tid; e < ns * N * (N / 2); e += THREADS) {   // two entries at a time (N is even)
+      const int r = e / (N / 2);
+      *(float4*)(Gs + 2 * e + r * (ld - N)) = *(const float4*)(Gg + 2 * e);
+    }
+  const float fm = (float)f.dm, fp = (float)f.dp;
+  double sign = 1.0;
+  unsigned long long n_acc = 0, n_dis = 0;
+  __syncthreads();
+
+  const int sp = ns == 2 ? lane >> 4 : 0, j = lane & 15;   // deciding warps: this lane's spin and column
+  // (A block without a flip has one barrier: thread 0 may then write the next block's count while
+  // slower warps still read this one's, hence two slots. It writes this slot again only after every
+  // warp has passed the next block's barrier.)
+  for (int i0 = 0, blk = 0; i0 < N; i0 += kb_max, ++blk) {
+    const int kb = min(kb_max, N - i0);
+    if (warp < kDecide) {
+      // ------------------------------------------------------------ decisions of the block
+      T* S = &st.S[sp][0][j];   // this lane's column: row t at S[t * kSites]
+#pragma unroll
+      for (int t = 4 * warp; t < 4 * warp + 4; ++t)
+        S[t * kSites] = t < kb && j < kb ? G[sp * sG + (long long)(i0 + t) * ld + i0 + j] : A::zero();
+      const int jj = min(j, kb - 1), s_j = sl[i0 + jj];   // (read before the first flip's write, see the barrier)
+      const bool pos = s_j > 0;
+      const unsigned u_j = u[i0 + jj];
+      const float uf = (float)u_j * 0x1p-32f, du = pos ? fm : fp, dd = pos ? fp : fm;
+      bar_decide();
+      int m = 0;
+      for (int lo = 0; lo < kb;) {   // sites below lo are decided
+        // every remaining site as if it were the next: lane j site j
+        const T gu = st.S[0][jj][jj], gd = ns == 2 ? st.S[1][jj][jj] : gu;
+        const float hu = 1.f - A::top(gu), hd = ns == 2 ? 1.f - A::top(gd) : A::top(gu);
+        const float R32 = (1.f + du * hu) * (1.f + dd * hd);
+        // FP32's error: a few 2^-24 of (1 + |du| (1 + |g|)) (1 + |dd| (1 + |g|))
+        const float bound = 2e-6f * (1.f + fabsf(du) * (1.f + fabsf(hu))) *
+                            (1.f + fabsf(dd) * (1.f + fabsf(hd)));
+        const bool open = j >= lo && j < kb;
+        bool mine = uf < fabsf(R32), neg = R32 < 0.f;
+        if (open && (rp || !(fabsf(uf - fabsf(R32)) > bound))) {   // in FP64, from the same G^_ii
+          const double g64 = A::wide(gu), h64 = ns == 2 ? 1.0 - A::wide(gd) : g64;
+          const double R = (1.0 + (pos ? f.dm : f.dp) * (1.0 - g64)) *
+                           (1.0 + (pos ? f.dp : f.dm) * h64);
+          mine = (double)u_j * 0x1p-32 < fabs(R);
+          neg = R < 0.0;
+        }
+        bool take = mine;
+        if (rp) take = rp[i0 + jj] != 0;
+        const unsigned takes = __ballot_sync(0xffffffffu, open && take) & 0xffffu;
+        const int b = takes ? __ffs(takes) - 1 : kb;      // the next accepted site; the rest up to it are rejected
+        if (rp)
+          n_dis += __popc(__ballot_sync(0xffffffffu, open && j <= b && take != mine) & 0xffffu);
+        if (b == kb) break;
+        ++n_acc;
+        if (__shfl_sync(0xffffffffu, (int)neg, b)) sign = -sign;
+        const bool posb = __shfl_sync(0xffffffffu, (int)pos, b);
+        // y = (Delta / R) row of G^, on every lane its entry
+        const T d = posb == (sp == 0) ? delta<T>(f, false) : delta<T>(f, true);
+        const T R = A::add(A::one(), A::mul(d, A::sub(A::one(), st.S[sp][b][b])));
+        const T q = A::div(d, R);
+        const T y = A::mul(q, S[b * kSites]);
+        if (!NMC_DCHECK(m < kSites && b < kSites, 121)) break;
+        if (warp == 0) {
+          st.y[sp][m][j] = y;
+          st.c[sp][m] = q;
+          if (lane == 0) {
+            st.site[m] = b;
+            sl[i0 + b] = (int8_t)(posb ? -1 : 1);
+          }
+        }
+        // this warp's rows below b: G^ += x y^T, x the column of site b
+        if (4 * warp + 3 > b) {
+          T z[4], x[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            x[k] = st.S[sp][4 * warp + k][b];
+            z[k] = S[(4 * warp + k) * kSites];
+          }
+          __syncwarp();
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            A::fma_acc(z[k], x[k], y);
+            if (4 * warp + k > b) {
+              S[(4 * warp + k) * kSites] = A::finish(z[k]);
+              st.x[sp][m][4 * warp + k] = x[k];
+            }
+          }
+        }
+        ++m;
+        lo = b + 1;
+        bar_decide();
+      }
+      if (tid == 0) st.m[blk & 1] = m;
+    }
+    __syncthreads();
+    const int m = st.m[blk & 1];
+    if (m > 0) {
+      // ---------------------------------------------------------- the vectors over all sites
+      // entry (kind, spin sv, r): x_q[r] (kind 0) or y_q[r] (kind 1) for every q
+      auto vectors = [&](int kind, int sv, int r, T (&v)[kSites]) {
+        const T* base = G + sv * sG + (kind ? (long long)i0 * ld + r : (long long)r * ld + i0);
+        const T* coef = kind ? &st.x[sv][0][0] : &st.y[sv][0][0];
+        const int step = kind ? ld : 1;
+#pragma unroll
+        for (int p = 0; p < kSites; ++p) {
+          v[p] = A::zero();
+          if (p >= m) continue;
+          const int s = st.site[p];
+          T z = base[(long long)s * step];
+#pragma unroll
+          for (int q = 0; q < p; ++q) A::fma_acc(z, coef[q * kSites + s], v[q]);
+          z = A::finish(z);
+          if (kind) z = A::mul(st.c[sv][p], z);
+          else if (r == i0 + s) z = A::sub(z, A::one());
+          v[p] = z;
+        }
+      };
+      if constexpr (FOLD == kFoldPairs) {
+        for (int t = tid; t < 2 * ns * N; t += THREADS) {
+          const int kind = t / (ns * N), e = t - kind * ns * N, sv = e / N, r = e - sv * N;
+          T v[kSites];
+          vectors(kind, sv, r, v);
+#pragma unroll
+          for (int p = 0; p < kSites; ++p)
+            if (p < m) pan[((kind * ns + sv) * kSites + p) * N + r] = v[p];
+        }
+        __syncthreads();
+        fold_pairs(G, pan, m, N, ns, sG, ld);
+      } else {
+        // digits of one spin at a time: both would not leave room for a second CTA on the SM
+        const int stride = Np * 32;
+        const bool once = 2 * ns * N <= THREADS;   // every thread one entry of one spin
+        T v[kSites];
+        int E = A::kExpMin;
+        auto limit = [&] {
+          E = A::kExpMin;
+#pragma unroll
+          for (int p = 0; p < kSites; ++p) E = max(E, A::expo(v[p]));
+        };
+        const int k0 = tid / (ns * N), e0 = tid - k0 * ns * N, s0 = e0 / N, r0 = e0 - s0 * N;
+        if (once && k0 < 2) {
+          vectors(k0, s0, r0, v);
+          limit();
+        }
+        for (int sf = 0; sf < ns; ++sf) {
+          if (sf) __syncthreads();   // the other spin's digits are read
+          if (once) {
+            if (k0 < 2 && s0 == sf) {
+              ev[k0 * Np + r0] = A::scale(E);
+              cut16(v, E, dig + k0 * kFDig * stride, r0, stride);
+            }
+          } else {
+            for (int t = tid; t < 2 * N; t += THREADS) {
+              const int kind = t / N, r = t - kind * N;
+              vectors(kind, sf, r, v);
+              limit();
+              ev[kind * Np + r] = A::scale(E);
+              cut16(v, E, dig + kind * kFDig * stride, r, stride);
+            }
+          }
+          __syncthreads();
+          const int nb = Np >> 4, per = (nb * nb + THREADS / 32 - 1) / (THREADS / 32);
+          const unsigned dbase = (unsigned)__cvta_generic_to_shared(dig);
+          const int ar = lane & 15, ah = lane >> 4;                       // ldmatrix rows, halves
+          const int br = (lane & 7) + ((lane >> 4) & 1) * 8, bh = (lane >> 3) & 1;
+          T* Gf = G + sf * sG;
+          for (int job = warp * per; job < min((warp + 1) * per, nb * nb); ++job) {
+            const int rb = job / nb * 16, cb = job % nb * 16;
+            float acc[2][4][kFDig];
+#pragma unroll
+            for (int n2 = 0; n2 < 2; ++n2)
+#pragma unroll
+              for (int w = 0; w < 4; ++w)
+#pragma unroll
+                for (int g = 0; g < kFDig; ++g) acc[n2][w][g] = 0.f;
+            float4 g4[2][2];   // G's entries, two each
+#pragma unroll
+            for (int n2 = 0; n2 < 2; ++n2)
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const int r = rb + (lane >> 2) + 8 * h, cc = cb + 8 * n2 + 2 * (lane & 3);
+                if (r < N && cc < N) g4[n2][h] = *(const float4*)(Gf + (long long)r * ld + cc);
+              }
+            unsigned bf[kFDig][4];
+#pragma unroll
+            for (int s = 0; s < kFDig; ++s)
+              ldm4(bf[s], dbase + (kFDig + s) * stride + digit_off(cb + br, bh));
+#pragma unroll
+            for (int s = 0; s < kFDig; ++s) {
+              unsigned af[4];
+              ldm4(af, dbase + s * stride + digit_off(rb + ar, ah));
+#pragma unroll
+              for (int q = 0; q + s < kFDig; ++q)
+#pragma unroll
+                for (int n2 = 0; n2 < 2; ++n2) {
+                  float d[4] = {acc[n2][0][s + q], acc[n2][1][s + q], acc[n2][2][s + q], acc[n2][3][s + q]};
+                  mma_h(d, af, bf[q][2 * n2], bf[q][2 * n2 + 1]);
+#pragma unroll
+                  for (int w = 0; w < 4; ++w) acc[n2][w][s + q] = d[w];
+                }
+            }
+#pragma unroll
+            for (int n2 = 0; n2 < 2; ++n2)
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                const int r = rb + (lane >> 2) + 8 * h, cc = cb + 8 * n2 + 2 * (lane & 3);
+                if (r >= N || cc >= N || !NMC_DCHECK(r < N && cc + 1 < N, 122)) continue;   // N is even
+                T* gp = Gf + (long long)r * ld + cc;
+                const int ea = ev[r], e0c = ev[Np + cc], e1c = ev[Np + cc + 1];
+                T g2[2];
+                memcpy(g2, &g4[n2][h], sizeof g2);
+                fold_entry(g2[0], acc[n2][2 * h], ea, e0c);
+                fold_entry(g2[1], acc[n2][2 * h + 1], ea, e1c);
+                memcpy(&g4[n2][h], g2, sizeof g2);
+                *(float4*)gp = g4[n2][h];
+              }
+          }
+        }
+      }
+      __syncthreads();
+    }
+  }
+  if (GS)
+    for (int e = tid; e < ns * N * (N / 2); e += THREADS) {
+      const int r = e / (N / 2);
+      *(float4*)(Gg + 2 * e) = *(const float4*)(Gs + 2 * e + r * (ld - N));
+    }
+  for (int i = tid; i < N; i += THREADS) fl[i] = sl[i];
+  if (tid == 0) {
+    f.sign[c] *= sign;
+    f.counts[3 * c + 0] += (unsigned long long)N;
+    f.counts[3 * c + 1] += n_acc;
+    f.counts[3 * c + 2] += n_dis;
+  }
+}
+
 }  // namespace
 
 size_t flip_smem_bytes(int N, int kk, size_t elem, int g_in_smem, int ns) {
@@ -588,20 +1116,56 @@ size_t flip_smem_bytes(int N, int kk, size_t elem, int g_in_smem, int ns) {
   return b;
 }
 
+namespace {
+
+constexpr size_t kBlockSmem = 226 * 1024;   // (227 KB are available)
+
+// One slice by k_flip_block; false: the vectors of a block do not fit shared memory. G is held
+// there when it fits with them. 256 threads, two CTAs per SM, when there are more chains than
+// SMs; 512 otherwise. (Neither choice changes a bit of the results.)
+template <typename T, int FOLD>
+bool flip_block(const FlipArgs<T>& f, int n_chains, cudaStream_t st) {
+  size_t bytes = block_smem<T>(f.N, f.ns, true, FOLD, f.N + 2);
+  const bool gs = bytes <= kBlockSmem;
+  if (!gs) bytes = block_smem<T>(f.N, f.ns, false, FOLD, f.N);
+  if (bytes > kBlockSmem) return false;
+  const int kb = f.kk < kSites ? f.kk : kSites;
+  auto run = [&](auto kernel, int threads) {
+    allow_max_dynamic_smem((const void*)kernel);
+    kernel<<<n_chains, threads, bytes, st>>>(f, kb);
+  };
+  if (!gs) run(k_flip_block<T, FOLD, 512, false>, 512);
+  else if (f.N > 48 && (n_chains <= sm_count() || bytes > kBlockSmem / 2)) run(k_flip_block<T, FOLD, 512, true>, 512);
+  else run(k_flip_block<T, FOLD, 256, true>, 256);
+  return true;
+}
+
 template <typename T>
-void flip_slice(const FlipArgs<T>& f, int n_chains, cudaStream_t st) {
+void flip_old(const FlipArgs<T>& f, int n_chains, cudaStream_t st) {
   const size_t bytes = flip_smem_bytes(f.N, f.kk, sizeof(T), f.g_in_smem, f.ns);
   allow_max_dynamic_smem((const void*)k_flip<T>);
   k_flip<T><<<n_chains, kThreads, bytes, st>>>(f);
 }
 
-template void flip_slice<double>(const FlipArgs<double>&, int, cudaStream_t);
-template void flip_slice<float>(const FlipArgs<float>&, int, cudaStream_t);
+}  // namespace
+
+template <>
+void flip_slice<float>(const FlipArgs<float>& f, int n_chains, cudaStream_t st) {
+  flip_old(f, n_chains, st);
+}
+
+template <>
+void flip_slice<double>(const FlipArgs<double>& f, int n_chains, cudaStream_t st) {
+  if (!flip_block<double, kFoldTensor>(f, n_chains, st)) flip_old(f, n_chains, st);
+}
 
 template <>
 void flip_slice<df2>(const FlipArgs<df2>& f, int n_chains, cudaStream_t st) {
+  if (f.tc_fold ? flip_block<df2, kFoldTensor>(f, n_chains, st)
+                : flip_block<df2, kFoldPairs>(f, n_chains, st))
+    return;
   const size_t bytes = flip_smem_bytes(f.N, f.kk, sizeof(df2), f.g_in_smem, f.ns);
-  if (f.tc_fold && f.kk <= kTcFlushMaxK && f.N >= kTcFlushMinN) {
+  if (f.tc_fold && f.kk <= kTcFlushMaxK) {
     allow_max_dynamic_smem((const void*)k_flip_df<true>);
     k_flip_df<true><<<n_chains, kThreadsDf, bytes, st>>>(f);
   } else {
