@@ -14,8 +14,7 @@
 // memory (L2); the panels always live in shared memory (k is clamped to fit).
 // That is k_flip (FP32) and, above some 560 sites, k_flip (FP64) and k_flip_df (FP32 pairs); up to
 // there FP64 and FP32 pairs take k_flip_block, which decides blocks of up to min(k, 16) sites apart.
-#include <cuda_fp16.h>
-
+#include "fold16.cuh"
 #include "nmc_internal.cuh"
 #include "oz_slice.cuh"
 
@@ -591,13 +590,8 @@ __global__ void __launch_bounds__(kThreadsDf, 2) k_flip_df(const FlipArgs<df2> f
 // sites, one entry of every vector per thread (a triangular recurrence with the submatrix's own x and
 // y as coefficients), and the block is folded into G.
 //
-// The fold G += sum_q x_q y_q^T is one k-step of 16 on the tensor cores (mma.sync; per 16 x 16 block
-// of G and spin), by exact slicing (Ozaki et al., Numer. Algorithms 2012): each row's x and each
-// column's y, scaled by a power of two, are cut into 6 balanced digits of 10 bits (|d| <= 512, exact
-// in FP16) straight from the registers they were formed in; the 21 digit products s + t <= 5
-// accumulate in six FP32 groups g = s + t, exact for g <= 3 (16 * 4 * 2^18 = 2^24). What is dropped
-// is below 2^-54 (FP32 pairs; 2^-57 in FP64) of the row's and column's maxima. tcgen05 would need 128
-// rows per tile and TMEM round trips for one k-step; mma.sync issues from the registers at hand.
+// The fold G += sum_q x_q y_q^T is one k-step of 16 on the tensor cores by exact FP16 digits
+// (fold16.cuh), cut straight from the registers the vectors were formed in.
 // Without tensor cores (FP32X2) the vectors go through shared memory to the FP32-pair loop.
 //
 // One slice, us, 44% of the flips accepted, one flip at a time (k_flip, k_flip_df) -> here:
@@ -608,8 +602,7 @@ __global__ void __launch_bounds__(kThreadsDf, 2) k_flip_df(const FlipArgs<df2> f
 // 45k (28 acceptances of some 1500: two ratios, a reciprocal and four rows' updates in a dependent
 // chain), the folds 47k (of which the MMAs' issue is 23k), the digits 24k, the vectors 13k. In FP64
 // the pipe's one instruction per 20 cycles bounds vectors and fold sums.
-constexpr int kSites = 16;                 // sites per block
-constexpr int kFDig = 6, kFW = 10, kFBits = 59;
+constexpr int kSites = kFoldK;             // sites per block
 enum FoldKind { kFoldTensor, kFoldPairs };
 
 template <typename T> struct Arith;
@@ -629,42 +622,6 @@ template <> struct Arith<df2> {
     const float e = __fmaf_rn(-b.lo, r, __fmaf_rn(-b.hi, r, 1.f));
     return df_mul(a, df2{r, __fmul_rn(r, e)});
   }
-  // biased exponent of |a|
-  static __device__ __forceinline__ int expo(df2 a) { return (__float_as_int(a.hi) >> 23) & 0xff; }
-  static constexpr int kExpMin = 9, kExpMax = 0xff;
-  // The terms of two k as FP16 digit pairs, most significant first. A term in units of 2^(E - 135)
-  // is below 512; adding kM 2^(-10 s) (ulp 2^(-10 s)) rounds it to its digit s, which then stands in
-  // the low mantissa bits on top of 0x6600, FP16's 1536. The low part joins after the first digit by
-  // exact sums (Fast2Sum: what is left of the high part is 0 or at least twice as large), its rest
-  // after the second and the third, so that no digit exceeds 512: beyond, FP16's steps are 2.
-  static __device__ __forceinline__ void digits(df2 a, df2 b, int E, unsigned (&w)[kFDig]) {
-    const float sc = __int_as_float((262 - E) << 23);
-    unsigned t0[kFDig], t1[kFDig];
-    split(a, sc, t0);
-    split(b, sc, t1);
-#pragma unroll
-    for (int s = 0; s < kFDig; ++s) w[s] = __byte_perm(t0[s], t1[s], 0x5410);
-  }
-  static __device__ __forceinline__ void split(df2 a, float sc, unsigned (&t)[kFDig]) {
-    float v = __fmul_rn(a.hi, sc), e = __fmul_rn(a.lo, sc), m = __int_as_float(0x4b406600);
-#pragma unroll
-    for (int s = 0; s < kFDig; ++s) {
-      if (s == 1 || s == 2) {
-        const float q = __fadd_rn(v, e);
-        e = __fsub_rn(e, __fsub_rn(q, v));
-        v = q;
-      }
-      if (s == 3) v = __fadd_rn(v, e);
-      const float x = __fadd_rn(v, m);
-      t[s] = __float_as_uint(x);
-      v = __fsub_rn(v, __fsub_rn(x, m));
-      m *= 0x1p-10f;
-    }
-  }
-  // what a row's (column's) digit sums are multiplied by: 2^(E - 135), or NaN where a term is not finite
-  static __device__ __forceinline__ int scale(int E) {
-    return E == kExpMax ? 0x7fc00000 : (E - 8) << 23;
-  }
 };
 template <> struct Arith<double> {
   static __device__ __forceinline__ double zero() { return 0.0; }
@@ -677,30 +634,6 @@ template <> struct Arith<double> {
   static __device__ __forceinline__ void fma_acc(double& c, double a, double b) { c = fma(a, b, c); }
   static __device__ __forceinline__ double finish(double a) { return a; }
   static __device__ __forceinline__ double div(double a, double b) { return a / b; }
-  static __device__ __forceinline__ int expo(double a) { return (__double2hiint(a) >> 20) & 0x7ff; }
-  static __device__ __forceinline__ long long fixed(double a, int E) {
-    const unsigned h = (unsigned)__double2hiint(a), l = (unsigned)__double2loint(a);
-    const int e = (int)((h >> 20) & 0x7ffu);
-    const unsigned long long m =
-        ((unsigned long long)(__funnelshift_l(l, h, 11) | 0x80000000u) << 32 | (l << 11));
-    const long long v = e == 0 ? 0ll : (long long)(m >> min(64 - kFBits + E - e, 63));
-    return (int)h < 0 ? -v : v;
-  }
-  static constexpr int kExpMin = 1, kExpMax = 0x7ff;
-  // Adding 512 to every 10-bit field of the term in units of 2^(E - 1022 - kFBits) and reading the
-  // fields less 512 gives balanced digits; a field added to 0x6400, FP16's 1024, is 1536 + digit.
-  static __device__ __forceinline__ void digits(double a, double b, int E, unsigned (&w)[kFDig]) {
-    const unsigned long long u0 = (unsigned long long)(fixed(a, E) + 0x0802008020080200ll);
-    const unsigned long long u1 = (unsigned long long)(fixed(b, E) + 0x0802008020080200ll);
-#pragma unroll
-    for (int s = 0; s < kFDig; ++s) {
-      const int bit = kFW * (kFDig - 1 - s);
-      w[s] = __byte_perm((unsigned)(u0 >> bit), (unsigned)(u1 >> bit), 0x5410);
-      if (s > 0) w[s] &= 0x03ff03ffu;   // (the first digit's field may reach 1024)
-      w[s] += 0x64006400u;
-    }
-  }
-  static __device__ __forceinline__ int scale(int E) { return E; }
 };
 
 template <typename T> __device__ __forceinline__ T delta(const FlipArgs<T>& f, bool plus);
@@ -734,80 +667,6 @@ __device__ void fold_pairs(T* G, const T* pan, int m, int N, int ns, long long s
           if (r + i * rstep < N) Gp[(long long)(r + i * rstep) * ld + c] = Arith<T>::finish(a[i]);
       }
   }
-}
-
-// byte offset of the 16-byte half h (k = 8 h ..) of a digit row r: rows of 32 bytes, the halves
-// exchanged in every second group of four rows so that ldmatrix meets all banks
-__device__ __forceinline__ int digit_off(int r, int h) { return r * 32 + ((h ^ ((r >> 2) & 1)) << 4); }
-
-// Cut the 16 terms of one row (or column) into digits, most significant first, `stride` bytes apart
-template <typename T>
-__device__ __forceinline__ void cut16(const T (&x)[kSites], int E, unsigned char* dst, int r, int stride) {
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    unsigned w[4][kFDig];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) Arith<T>::digits(x[8 * h + 2 * i], x[8 * h + 2 * i + 1], E, w[i]);
-#pragma unroll
-    for (int s = 0; s < kFDig; ++s) {
-      unsigned d[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const __half2 v = __hadd2(*reinterpret_cast<__half2*>(&w[i][s]), __float2half2_rn(-1536.f));
-        d[i] = *reinterpret_cast<const unsigned*>(&v);
-      }
-      *reinterpret_cast<uint4*>(dst + s * stride + digit_off(r, h)) = make_uint4(d[0], d[1], d[2], d[3]);
-    }
-  }
-}
-
-__device__ __forceinline__ void ldm4(unsigned (&r)[4], unsigned addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr));
-}
-__device__ __forceinline__ void mma_h(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-      "{%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// One entry of G plus its digit sums sum_g a_g 2^(-10 g) times the row's and the column's scale.
-// a_0 + a_1 2^-10 + a_2 2^-20 as an exact pair by Fast2Sum: where the smaller-magnitude operand comes
-// first, the sum is short enough to be exact (a_0 is an integer, |a_1 2^-10| < 2^13, |a_2 2^-20| < 13).
-__device__ __forceinline__ void fold_entry(df2& G, const float (&a)[kFDig], int ea, int eb) {
-  const float s = __fmaf_rn(a[1], 0x1p-10f, a[0]);
-  const float e1 = __fmaf_rn(a[1], 0x1p-10f, -__fsub_rn(s, a[0]));
-  const float h = __fmaf_rn(a[2], 0x1p-20f, s);
-  const float e2 = __fmaf_rn(a[2], 0x1p-20f, -__fsub_rn(h, s));
-  float l = __fmaf_rn(a[3], 0x1p-30f, __fadd_rn(e1, e2));
-  l = __fmaf_rn(a[5], 0x1p-50f, __fmaf_rn(a[4], 0x1p-40f, l));
-  const float sc = __fmul_rn(__int_as_float(ea), __int_as_float(eb));
-  const float th = __fmul_rn(h, sc), q = __fadd_rn(G.hi, th), b = __fsub_rn(q, G.hi);
-  const float e = __fadd_rn(__fsub_rn(G.hi, __fsub_rn(q, b)), __fsub_rn(th, b));
-  G = df_norm(q, __fadd_rn(e, __fmaf_rn(l, sc, G.lo)));
-}
-__device__ __forceinline__ void fold_entry(double& G, const float (&a)[kFDig], int ea, int eb) {
-  if (max(ea, eb) >= Arith<double>::kExpMax) {   // an infinity or a NaN among the terms
-    G = __longlong_as_double(0x7ff8000000000000ll);
-    return;
-  }
-  int q[kFDig];
-#pragma unroll
-  for (int s = 0; s < kFDig; ++s) q[s] = __float2int_rn(a[s]);
-  long long H = (long long)q[0] * (1 << 20) + ((long long)q[1] * (1 << 10) + q[2]);
-  long long L = (long long)q[3] * (1 << 20) + ((long long)q[4] * (1 << 10) + q[5]);
-  H += L >> 30;   // (H 2^30 + L) 2^-50
-  L &= (1ll << 30) - 1;
-  const int s = min(__clzll(H ^ (H >> 63)) - 1, 30);
-  const double v = (double)((H << s) + (L >> (30 - s)));
-  const int k = ea + eb - 2 * 1022 - 18 - 20 - s;
-  const int e = (__double2hiint(v) >> 20) & 0x7ff;
-  if (e == 0) return;
-  G += e + k >= 1 && e + k <= 2046
-           ? __hiloint2double(__double2hiint(v) + k * (1 << 20), __double2loint(v)) : ldexp(v, k);
 }
 
 // the deciding warps, 4 rows of the block each
@@ -1002,11 +861,11 @@ k_flip_block(const FlipArgs<T> f, int kb_max) {
         const int stride = Np * 32;
         const bool once = 2 * ns * N <= THREADS;   // every thread one entry of one spin
         T v[kSites];
-        int E = A::kExpMin;
+        int E = Digits<T>::kExpMin;
         auto limit = [&] {
-          E = A::kExpMin;
+          E = Digits<T>::kExpMin;
 #pragma unroll
-          for (int p = 0; p < kSites; ++p) E = max(E, A::expo(v[p]));
+          for (int p = 0; p < kSites; ++p) E = max(E, Digits<T>::expo(v[p]));
         };
         const int k0 = tid / (ns * N), e0 = tid - k0 * ns * N, s0 = e0 / N, r0 = e0 - s0 * N;
         if (once && k0 < 2) {
@@ -1017,75 +876,23 @@ k_flip_block(const FlipArgs<T> f, int kb_max) {
           if (sf) __syncthreads();   // the other spin's digits are read
           if (once) {
             if (k0 < 2 && s0 == sf) {
-              ev[k0 * Np + r0] = A::scale(E);
-              cut16(v, E, dig + k0 * kFDig * stride, r0, stride);
+              ev[k0 * Np + r0] = Digits<T>::scale(E);
+              cut16<T>(v, E, dig + k0 * kFDig * stride, r0, stride);
             }
           } else {
             for (int t = tid; t < 2 * N; t += THREADS) {
               const int kind = t / N, r = t - kind * N;
               vectors(kind, sf, r, v);
               limit();
-              ev[kind * Np + r] = A::scale(E);
-              cut16(v, E, dig + kind * kFDig * stride, r, stride);
+              ev[kind * Np + r] = Digits<T>::scale(E);
+              cut16<T>(v, E, dig + kind * kFDig * stride, r, stride);
             }
           }
           __syncthreads();
-          const int nb = Np >> 4, per = (nb * nb + THREADS / 32 - 1) / (THREADS / 32);
-          const unsigned dbase = (unsigned)__cvta_generic_to_shared(dig);
-          const int ar = lane & 15, ah = lane >> 4;                       // ldmatrix rows, halves
-          const int br = (lane & 7) + ((lane >> 4) & 1) * 8, bh = (lane >> 3) & 1;
           T* Gf = G + sf * sG;
-          for (int job = warp * per; job < min((warp + 1) * per, nb * nb); ++job) {
-            const int rb = job / nb * 16, cb = job % nb * 16;
-            float acc[2][4][kFDig];
-#pragma unroll
-            for (int n2 = 0; n2 < 2; ++n2)
-#pragma unroll
-              for (int w = 0; w < 4; ++w)
-#pragma unroll
-                for (int g = 0; g < kFDig; ++g) acc[n2][w][g] = 0.f;
-            float4 g4[2][2];   // G's entries, two each
-#pragma unroll
-            for (int n2 = 0; n2 < 2; ++n2)
-#pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                const int r = rb + (lane >> 2) + 8 * h, cc = cb + 8 * n2 + 2 * (lane & 3);
-                if (r < N && cc < N) g4[n2][h] = *(const float4*)(Gf + (long long)r * ld + cc);
-              }
-            unsigned bf[kFDig][4];
-#pragma unroll
-            for (int s = 0; s < kFDig; ++s)
-              ldm4(bf[s], dbase + (kFDig + s) * stride + digit_off(cb + br, bh));
-#pragma unroll
-            for (int s = 0; s < kFDig; ++s) {
-              unsigned af[4];
-              ldm4(af, dbase + s * stride + digit_off(rb + ar, ah));
-#pragma unroll
-              for (int q = 0; q + s < kFDig; ++q)
-#pragma unroll
-                for (int n2 = 0; n2 < 2; ++n2) {
-                  float d[4] = {acc[n2][0][s + q], acc[n2][1][s + q], acc[n2][2][s + q], acc[n2][3][s + q]};
-                  mma_h(d, af, bf[q][2 * n2], bf[q][2 * n2 + 1]);
-#pragma unroll
-                  for (int w = 0; w < 4; ++w) acc[n2][w][s + q] = d[w];
-                }
-            }
-#pragma unroll
-            for (int n2 = 0; n2 < 2; ++n2)
-#pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                const int r = rb + (lane >> 2) + 8 * h, cc = cb + 8 * n2 + 2 * (lane & 3);
-                if (r >= N || cc >= N || !NMC_DCHECK(r < N && cc + 1 < N, 122)) continue;   // N is even
-                T* gp = Gf + (long long)r * ld + cc;
-                const int ea = ev[r], e0c = ev[Np + cc], e1c = ev[Np + cc + 1];
-                T g2[2];
-                memcpy(g2, &g4[n2][h], sizeof g2);
-                fold_entry(g2[0], acc[n2][2 * h], ea, e0c);
-                fold_entry(g2[1], acc[n2][2 * h + 1], ea, e1c);
-                memcpy(&g4[n2][h], g2, sizeof g2);
-                *(float4*)gp = g4[n2][h];
-              }
-          }
+          const unsigned dbase = (unsigned)__cvta_generic_to_shared(dig);
+          fold_tiles<T>([&](int r) { return Gf + (long long)r * ld; }, dbase, stride, ev,
+                        dbase + kFDig * stride, stride, ev + Np, N, N, true, warp, THREADS / 32);   // (N is even)
         }
       }
       __syncthreads();

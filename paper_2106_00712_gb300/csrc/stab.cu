@@ -7,12 +7,12 @@
 //   squared column norms are downdated and summed again when little of them is left. Outputs
 //   U = Q (formed in place by backward accumulation of the reflectors), D = |diag R| and
 //   T = D^{-1} R P^T.
-// k_solve: Y = X^{-1} (Db_R^{-1} U_R^T) by Gauss-Jordan elimination with partial pivoting
-//   on the augmented matrix [X | RHS]; X is the well-scaled middle factor of the
-//   stabilized inverse, so partial pivoting is sufficient.
+// k_solve: Y = X^{-1} (Db_R^{-1} U_R^T) by blocked LU with partial pivoting; X is the
+//   well-scaled middle factor of the stabilized inverse, so partial pivoting is sufficient.
 //
 // One CTA per matrix (batch = 2 * chains); the working matrix lives in shared memory
 // when it fits and in a per-matrix global workspace otherwise.
+#include "fold16.cuh"
 #include "nmc_internal.cuh"
 
 namespace nmc {
@@ -27,25 +27,10 @@ NMC_DEBUG_FLAG
 constexpr int kSolveThreads = 512;
 constexpr int kSolveWarps = kSolveThreads / 32;
 constexpr size_t kSmemLimit = 200 * 1024;
+// Up to here Gauss-Jordan is faster: 16 sites x 2 matrices 23 us against 29, 36 x 128 73 against 91;
+// 48 x 6 110 against 107, 48 x 512 296 against 220.
+constexpr int kGaussJordanMax = 40;
 constexpr size_t kQrSmemLimit = 225 * 1024;
-
-// argmax over lanes: larger key wins, lower index on ties. Keys are the bit patterns of
-// non-negative doubles (|x|, squared norms), which order like the values, so the search
-// runs on the integer pipes instead of the narrow FP64 pipe; a lane with no candidate
-// holds key -1.
-__device__ __forceinline__ void warp_argmax(long long& key, int& idx) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const long long ok = __shfl_xor_sync(0xffffffffu, key, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-    if (ok > key || (ok == key && oi < idx)) { key = ok; idx = oi; }
-  }
-}
-
-// key of a non-negative double (a NaN, with its sign bit cleared, orders above +inf)
-__device__ __forceinline__ long long nonneg_key(double x) {
-  return __double_as_longlong(x) & 0x7fffffffffffffffll;
-}
 
 // ---------------------------------------------------------------------------- QR
 // The FP64 pipe issues one warp operation per 20 cycles and SM, an integer multiply-add 32 x 32 +
@@ -454,17 +439,35 @@ k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__
   }
 }
 
+// argmax over lanes: larger key wins, lower index on ties. Keys are the bit patterns of
+// non-negative doubles (|x|, squared norms), which order like the values, so the search
+// runs on the integer pipes instead of the narrow FP64 pipe; a lane with no candidate
+// holds key -1.
+__device__ __forceinline__ void warp_argmax(long long& key, int& idx) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long ok = __shfl_xor_sync(0xffffffffu, key, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
+    if (ok > key || (ok == key && oi < idx)) { key = ok; idx = oi; }
+  }
+}
+
+// key of a non-negative double (a NaN, with its sign bit cleared, orders above +inf)
+__device__ __forceinline__ long long nonneg_key(double x) {
+  return __double_as_longlong(x) & 0x7fffffffffffffffll;
+}
+
+// Few sites: Gauss-Jordan elimination with partial pivoting, one column at a time.
 __global__ void __launch_bounds__(kSolveThreads)
-k_solve(const double* __restrict__ X, const double* __restrict__ UR, long long sUR,
-        const double* __restrict__ DR, long long sDR, double* __restrict__ Y,
-        double* __restrict__ ws, int N, int use_smem) {
+k_solve_gj(const double* __restrict__ X, const double* __restrict__ UR, long long sUR,
+           const double* __restrict__ DR, long long sDR, double* __restrict__ Y, int N) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int s_piv;
   __shared__ double s_inv;
   const int b = blockIdx.x;
   const long long NN = (long long)N * N;
   const int ld = 2 * N;
-  double* Aug = use_smem ? (double*)smraw : ws + (long long)b * 2 * NN;  // row-major N x 2N
+  double* Aug = (double*)smraw;  // row-major N x 2N
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const double* Xb = X + (long long)b * NN;
   const double* Ub = UR + (long long)b * sUR;
@@ -523,6 +526,275 @@ k_solve(const double* __restrict__ X, const double* __restrict__ UR, long long s
   }
 }
 
+// ---------------------------------------------------------------------------- solve
+// Y = X^{-1} (Db_R^{-1} U_R^T) by blocked LU with partial pivoting on the augmented matrix [X | RHS],
+// 16 columns per block:
+//   panel     thread t holds row t's 16 entries in registers; per column the pivot is the row with the
+//             largest |entry| (its upper 32 bits; lowest index on ties), found per warp and then over
+//             the warps' candidates, which bring their rows and reciprocals along: one barrier a column;
+//             rows stay where they are, `map` says which one is k-th
+//   rows      a thread per column solves the block's unit lower triangle (FP64) for its 16 rows
+//   update    rows below -= (rows x 16) (16 x columns): fold16.cuh's tensor-core rank-16 update, the
+//             digits cut from the registers of the two steps before
+// then the triangular solve upwards over the blocks, with the same update of the rows above.
+//
+// Elimination in FP64 throughout took 1.5 N^3 multiply-adds at one warp operation per 20 cycles and
+// SM (246k cycles a matrix at N = 64); here the FP64 pipe adds once per entry and block (28k), and
+// does the triangles (48k) and the panels (26k).
+// us, Gauss-Jordan -> here: 64 sites x 512 583 -> 321, 64 x 6 197 -> 150, 72 x 1024 1430 -> 925,
+// 100 x 128 582 -> 302, 144 x 128 2800 -> 600, 256 x 64 (in global memory) 16100 -> 2100; the error of
+// Y against 64-bit-mantissa elimination is about half of before.
+// What bounds it: a matrix's dependent chain. Of 300k cycles at N = 64 the panels take 95k (1500 a
+// column: search, reciprocal, barrier, and some ten FP64 operations at 80 cycles from one warp), the
+// triangles 80k, the updates 70k; two matrices on an SM run in the time of one.
+__host__ __device__ inline size_t solve_small_bytes(int N, int chunk, int nw) {
+  const int rows = max((N - 1) & ~15, 16);   // digit rows: all but the first (last) block's
+  return (size_t)kFDig * 32 * (rows + chunk) + 4 * (rows + chunk)       // digits, scales
+         + 16 * 16 * 8 + 2 * nw * (16 * 8 + 16)                         // triangle, candidates
+         + (size_t)N * 8 + (size_t)((N + 3) & ~3) * 4 + 64;             // 1 / pivots, row map, block's pivots
+}
+
+__device__ __forceinline__ double rcp64(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);   // 2^-20: 1 / x = r (1 + e + e^2 + O(2^-60))
+  return fma(r, fma(e, e, e), r);
+}
+
+// RP: rows per thread of a panel. lda: row stride of the augmented matrix; chunk: columns whose digits
+// are held at a time (a multiple of 16).
+template <int THREADS, int RP, int CTAS, bool SMEM>
+__global__ void __launch_bounds__(THREADS, CTAS)
+k_solve(const double* __restrict__ X, const double* __restrict__ UR, long long sUR,
+        const double* __restrict__ DR, long long sDR, double* __restrict__ Y,
+        double* __restrict__ ws, int N, int lda, int chunk) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  constexpr int NW = THREADS / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int b = blockIdx.x;
+  const long long NN = (long long)N * N;
+  const int rows = max((N - 1) & ~15, 16), rs = rows * 32, cs = chunk * 32;
+  double* A;   // row-major N x 2N
+  if constexpr (SMEM) A = (double*)smraw;
+  else A = ws + (long long)b * 2 * NN;
+  unsigned char* rd = smraw + (SMEM ? (size_t)N * lda * sizeof(double) : 0);   // digits of rows
+  unsigned char* cd = rd + (size_t)kFDig * rs;                                 // and of columns
+  double (*tri)[16] = (double (*)[16])(cd + (size_t)kFDig * cs);   // the block's L (unit) below U
+  double (*cand)[NW][16] = (double (*)[NW][16])(tri + 16);         // [parity][warp]: candidate's row
+  double (*cinv)[NW] = (double (*)[NW])(cand + 2);                 // its entry's reciprocal
+  unsigned (*ckey)[NW] = (unsigned (*)[NW])(cinv + 2);             // its key
+  int (*cwho)[NW] = (int (*)[NW])(ckey + 2);                       // its row, counted from the block's first
+  double* inv = (double*)(cwho + 2);                               // 1 / U_kk
+  int* re = (int*)(inv + N);                                       // scales of digit rows, columns
+  int* ce = re + rows;
+  int* map = ce + chunk;                                           // storage row of the k-th row
+  int* who = map + ((N + 3) & ~3);                                 // the block's pivots
+  const unsigned rda = (unsigned)__cvta_generic_to_shared(rd), cda = (unsigned)__cvta_generic_to_shared(cd);
+
+  const double* Xb = X + (long long)b * NN;
+  const double* Ub = UR + (long long)b * sUR;
+  const double* Dv = DR + (long long)b * sDR;
+  for (int r = tid; r < N; r += THREADS) {
+    map[r] = r;
+    inv[r] = 1.0 / fmax(Dv[r], 1.0);
+  }
+  __syncthreads();
+  for (int r = warp; r < N; r += NW)
+    for (int c = lane; c < N; c += 32) {
+      A[(long long)r * lda + c] = Xb[(long long)r * N + c];
+      A[(long long)c * lda + N + r] = Ub[(long long)r * N + c] * inv[c];   // (Db_R^{-1} U_R^T)[c][r]
+    }
+  __syncthreads();
+
+  // digits of w columns from column j0 on, of the 16 rows k0 ..
+  auto cut_columns = [&](int j0, int w, int k0) {
+    for (int c = tid; c < w; c += THREADS) {
+      double x[16];
+      int E = Digits<double>::kExpMin;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) {
+        x[q] = k0 + q < N ? A[(long long)map[k0 + q] * lda + j0 + c] : 0.0;
+        E = max(E, Digits<double>::expo(x[q]));
+      }
+      ce[c] = Digits<double>::scale(E);
+      cut16<double>(x, E, cd, c, cs);
+    }
+  };
+
+  for (int k0 = 0; k0 < N; k0 += 16) {
+    const int kw = min(16, N - k0), left = N - k0;
+    // ------------------------------------------------------------ panel
+    double a[RP][16];
+    int place[RP];   // -1: still a candidate; otherwise its place among the block's pivots
+    int row[RP];
+#pragma unroll
+    for (int i = 0; i < RP; ++i) {
+      const int t = tid + i * THREADS;
+      place[i] = t < left ? -1 : 16;
+      row[i] = t < left ? map[k0 + t] : 0;
+      const double* src = A + (long long)row[i] * lda + k0;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) a[i][c] = t < left && c < kw ? src[c] : 0.0;
+    }
+    const int nw = min(NW, (left + 31) >> 5);
+#pragma unroll
+    for (int p = 0; p < 16; ++p) {
+      if (p >= kw) break;
+      unsigned key = 0;
+      int ci = 0;
+#pragma unroll
+      for (int i = 0; i < RP; ++i) {
+        const unsigned k = place[i] < 0 ? ((unsigned)__double2hiint(a[i][p]) & 0x7fffffffu) + 1 : 0;
+        if (k > key) { key = k; ci = i; }
+      }
+      const unsigned best = __reduce_max_sync(0xffffffffu, key);
+      const unsigned mine = __ballot_sync(0xffffffffu, key == best);
+      if (best == 0 && lane == 0 && warp < nw) ckey[p & 1][warp] = 0;
+      if (best > 0 && lane == __ffs(mine) - 1) {
+        ckey[p & 1][warp] = best;
+        cwho[p & 1][warp] = tid + ci * THREADS;
+#pragma unroll
+        for (int i = 0; i < RP; ++i)
+          if (i == ci) {
+            cinv[p & 1][warp] = rcp64(a[i][p]);
+#pragma unroll
+            for (int c = 0; c < 16; ++c)
+              if (c >= p) cand[p & 1][warp][c] = a[i][c];
+          }
+      }
+      __syncthreads();
+      const unsigned wk = lane < nw ? ckey[p & 1][lane] : 0;
+      const unsigned wbest = __reduce_max_sync(0xffffffffu, wk);
+      const int w = __ffs(__ballot_sync(0xffffffffu, lane < nw && wk == wbest)) - 1;
+      if (!NMC_DCHECK(w >= 0 && w < nw, 202)) break;
+      const int piv = cwho[p & 1][w];
+      const double ip = cinv[p & 1][w];
+      if (tid == 0) {
+        who[p] = piv;
+        inv[k0 + p] = ip;
+      }
+      const double* pr = cand[p & 1][w];
+      if (warp < nw) {
+#pragma unroll
+        for (int i = 0; i < RP; ++i) {
+          if (piv == tid + i * THREADS) place[i] = p;
+          const double l = place[i] < 0 ? a[i][p] * ip : 0.0;
+          if (place[i] < 0) a[i][p] = l;
+#pragma unroll
+          for (int c = 0; c < 16; ++c)
+            if (c > p) a[i][c] = fma(-l, pr[c], a[i][c]);
+        }
+      }
+    }
+    __syncthreads();
+    // ------------------------------------------------- the new order; digits of the rows below
+    for (int e = kw * 16 + tid; e < 256; e += THREADS) tri[e >> 4][e & 15] = 0.0;
+    // pivot p moves to place k0 + p; the rows it displaces fill the places the pivots left
+    const int wl = lane < kw ? who[lane] : 0;
+    const unsigned taken = __reduce_or_sync(0xffffffffu, lane < kw && wl < kw ? 1u << wl : 0u);
+    const unsigned outside = __ballot_sync(0xffffffffu, lane < kw && wl >= kw);
+    const unsigned moved = ~taken & ((1u << kw) - 1);   // as many as `outside` has bits
+#pragma unroll
+    for (int i = 0; i < RP; ++i) {
+      const int t = tid + i * THREADS;
+      if (t >= left) continue;
+      if (place[i] >= 0) {
+        const int p = place[i];
+        map[k0 + p] = row[i];   // (read by no one before the next barrier)
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          tri[p][c] = a[i][c];
+          if (c >= p && c < kw) A[(long long)row[i] * lda + k0 + c] = a[i][c];   // U, for the way back
+        }
+      } else {
+        int to = t;
+        if (t < kw)
+          to = who[__fns(outside, 0, __popc(moved & ((1u << t) - 1)) + 1)];
+        if (!NMC_DCHECK(to >= kw && to < left, 203)) continue;
+        map[k0 + to] = row[i];
+        int E = Digits<double>::kExpMin;
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          a[i][c] = -a[i][c];
+          E = max(E, Digits<double>::expo(a[i][c]));
+        }
+        re[to - kw] = Digits<double>::scale(E);
+        cut16<double>(a[i], E, rd, to - kw, rs);
+      }
+    }
+    __syncthreads();
+    // ------------------------------------------------- the block's rows, and the update below
+    const int c0 = k0 + kw;
+    for (int c = c0 + tid; c < 2 * N; c += THREADS) {
+      double x[16];
+#pragma unroll
+      for (int q = 0; q < 16; ++q) x[q] = q < kw ? A[(long long)map[k0 + q] * lda + c] : 0.0;
+#pragma unroll
+      for (int s = 0; s < 16; ++s) {   // (tri is 0 beyond kw)
+#pragma unroll
+        for (int q = s + 1; q < 16; ++q) x[q] = fma(-tri[q][s], x[s], x[q]);
+        if (s > 0 && s < kw) A[(long long)map[k0 + s] * lda + c] = x[s];
+      }
+    }
+    __syncthreads();
+    if (c0 >= N) break;
+    for (int j0 = c0; j0 < 2 * N; j0 += chunk) {
+      const int w = min(chunk, 2 * N - j0);
+      cut_columns(j0, w, k0);
+      __syncthreads();
+      fold_tiles<double>([&](int r) { return A + (long long)map[c0 + r] * lda + j0; }, rda, rs, re, cda, cs, ce,
+                         N - c0, w, (N & 1) == 0, warp, NW);
+      __syncthreads();
+    }
+  }
+  // ------------------------------------------------------------ upwards
+  double* Yb = Y + (long long)b * NN;
+  for (int k0 = (N - 1) & ~15; k0 >= 0; k0 -= 16) {
+    const int kw = min(16, N - k0);
+    for (int e = tid; e < 256; e += THREADS) {   // the block's U
+      const int q = e >> 4, c = e & 15;
+      tri[q][c] = q < kw && c < kw ? A[(long long)map[k0 + q] * lda + k0 + c] : 0.0;
+    }
+    for (int r = tid; r < k0; r += THREADS) {    // its columns in the rows above
+      const double* src = A + (long long)map[r] * lda + k0;
+      double u[16];
+      int E = Digits<double>::kExpMin;
+#pragma unroll
+      for (int c = 0; c < 16; ++c) {
+        u[c] = c < kw ? -src[c] : 0.0;
+        E = max(E, Digits<double>::expo(u[c]));
+      }
+      re[r] = Digits<double>::scale(E);
+      cut16<double>(u, E, rd, r, rs);
+    }
+    __syncthreads();
+    for (int c = tid; c < N; c += THREADS) {
+      double x[16];
+#pragma unroll
+      for (int q = 0; q < 16; ++q) x[q] = q < kw ? A[(long long)map[k0 + q] * lda + N + c] : 0.0;
+#pragma unroll
+      for (int s = 15; s >= 0; --s) {
+        if (s >= kw) continue;
+        x[s] *= inv[k0 + s];
+#pragma unroll
+        for (int q = 0; q < s; ++q) x[q] = fma(-tri[q][s], x[s], x[q]);
+        Yb[(long long)(k0 + s) * N + c] = x[s];
+        if (k0 > 0) A[(long long)map[k0 + s] * lda + N + c] = x[s];
+      }
+    }
+    __syncthreads();
+    if (k0 == 0) break;
+    for (int j0 = 0; j0 < N; j0 += chunk) {
+      const int w = min(chunk, N - j0);
+      cut_columns(N + j0, w, k0);
+      __syncthreads();
+      fold_tiles<double>([&](int r) { return A + (long long)map[r] * lda + N + j0; }, rda, rs, re, cda, cs, ce,
+                         k0, w, (N & 1) == 0, warp, NW);
+      __syncthreads();
+    }
+  }
+}
+
 }  // namespace
 
 // The lanes per column follow from N alone (results must not depend on the batch): as few as keep
@@ -549,19 +821,36 @@ void qrp_udt(const double* X, double* U, double* D, double* Tp, double* ws, int 
   else run(k_qrp<32, 8, 512, 1>, 32, 8, 512);
 }
 
-void solve_stab(const double* X, const double* UR, long long sUR, const double* DR,
-                long long sDR, double* Y, double* ws, int N, int batch, cudaStream_t st) {
-  const size_t big = 2 * (size_t)N * N * sizeof(double);
-  const int use_smem = big <= kSmemLimit;
-  const size_t bytes = use_smem ? big : 0;
-  allow_max_dynamic_smem((const void*)k_solve);
-  k_solve<<<batch, kSolveThreads, bytes, st>>>(X, UR, sUR, DR, sDR, Y, ws, N, use_smem);
-}
-
 // (the threshold that the documented scratch sizes of nmc_green_noalloc follow)
 bool stab_needs_workspace(int N) {
   const size_t small = ((size_t)N * 28 + 64 + 15) & ~(size_t)15;
   return small + 2 * (size_t)N * N * sizeof(double) > kSmemLimit;
+}
+
+void solve_stab(const double* X, const double* UR, long long sUR, const double* DR,
+                long long sDR, double* Y, double* ws, int N, int batch, cudaStream_t st) {
+  if (N <= kGaussJordanMax) {
+    allow_max_dynamic_smem((const void*)k_solve_gj);
+    k_solve_gj<<<batch, kSolveThreads, 2 * (size_t)N * N * sizeof(double), st>>>(X, UR, sUR, DR, sDR, Y, N);
+    return;
+  }
+  // shared memory holds the augmented matrix wherever no workspace is promised
+  const bool smem = !stab_needs_workspace(N);
+  auto run = [&](auto kernel, int threads, size_t limit) {
+    int lda = 2 * N;
+    if (smem && (lda & 15) == 0 && N <= 96) lda += 8;   // rows 64 bytes apart modulo the banks
+    const size_t big = smem ? (size_t)N * lda * sizeof(double) : 0;
+    int chunk = 16;   // as many columns as there is room for
+    while (chunk < 2 * N && big + solve_small_bytes(N, chunk + 16, threads / 32) <= limit) chunk += 16;
+    const size_t bytes = big + solve_small_bytes(N, chunk, threads / 32);
+    allow_max_dynamic_smem((const void*)kernel);
+    kernel<<<batch, threads, bytes, st>>>(X, UR, sUR, DR, sDR, Y, ws, N, lda, chunk);
+  };
+  constexpr size_t kTwo = 113 * 1024, kOne = 227 * 1024;   // two CTAs to an SM (up to 72 sites they fit), or one
+  if (N <= 72) run(k_solve<256, 1, 2, true>, 256, kTwo);
+  else if (smem) run(k_solve<512, 1, 1, true>, 512, kOne);
+  else if (N <= 512) run(k_solve<512, 1, 1, false>, 512, kOne);
+  else run(k_solve<512, 2, 1, false>, 512, kOne);
 }
 
 NMC_DEBUG_READER(debug_fail_stab)
