@@ -12,7 +12,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libnmc.so")
-SOURCES = ["gemm.cu", "gemm_fx.cu", "gemm_df.cu", "gemm_tc.cu", "stab.cu", "flip.cu", "misc.cu", "nmc_api.cu", "noalloc.cu",
+SOURCES = ["gemm.cu", "gemm_fx.cu", "gemm_df.cu", "gemm_tc.cu", "wrap.cu", "stab.cu", "flip.cu", "misc.cu", "nmc_api.cu", "noalloc.cu",
            "nimc.cu", "cgen.cu", "probe.cu", "lattice.cpp"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC,-O3",

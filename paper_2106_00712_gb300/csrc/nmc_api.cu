@@ -24,6 +24,7 @@
 #include "../../include/nmc.h"
 #include "../../include/nmc_gen.h"
 #include "nmc_internal.cuh"
+#include "wrap.cuh"
 
 // nimc.cu: Bernoulli fields from a generator (stream 1, samples n0..n0+n-1), synchronised
 nmc_status nmc_gen_fill_fields(nmc_gen* g, int N, int Lt, long long n0, int n, int8_t* d_fields,
@@ -105,6 +106,9 @@ struct nmc_ctx {
   // [constant][0: on the left, 1: on the right], their exponents and TMA tensor maps
   void* dOz[4][2] = {};
   int* dOzExp[4][2] = {};
+  // operand fragments of the constants, up to kFragMaxN sites (FP64 and NMC_SPLIT_BF16): indices as dOz
+  uint4* dFrag[4][2] = {};
+  int* dFragScale[4][2] = {};
   alignas(64) unsigned char tmap[4][2][128] = {};
   bool oz = false;
   int* dErr = nullptr;   // device flag: a bounded device-side wait expired (NMC_ETIMEOUT)
@@ -152,6 +156,8 @@ struct nmc_ctx {
   // compensated FP32-pair propagation: products on the tensor cores (SPLIT_BF16) or SIMT
   bool dfp() const { return opt.precision == NMC_SPLIT_BF16 || opt.precision == NMC_FP32X2; }
   bool tc() const { return opt.precision == NMC_SPLIT_BF16; }
+  // wraps and block products a whole matrix per CTA (wrap.cu, where the bounds' reasons stand)
+  bool frags() const { return N <= kFragMaxN && (tc() || (opt.precision == NMC_FP64 && N > 16)); }
 };
 
 namespace {
@@ -244,7 +250,10 @@ void free_all(nmc_ctx* x) {
   x->dGf = x->dT1f = nullptr;
   x->dG2 = x->dT12 = x->dEm2 = x->dEp2 = x->dXa = x->dXb = x->dEmh2 = x->dEph2 = nullptr;
   for (int a = 0; a < 4; ++a)
-    for (int r = 0; r < 2; ++r) x->dOz[a][r] = nullptr, x->dOzExp[a][r] = nullptr;
+    for (int r = 0; r < 2; ++r) {
+      x->dOz[a][r] = nullptr, x->dOzExp[a][r] = nullptr;
+      x->dFrag[a][r] = nullptr, x->dFragScale[a][r] = nullptr;
+    }
   x->oz = false;
   x->dErr = nullptr;
   x->slot.clear();
@@ -332,13 +341,15 @@ nmc_status alloc_all(nmc_ctx* x) {
     NMC_TRY(dalloc(x, &x->dEm2, NN));
     NMC_TRY(dalloc(x, &x->dEp2, NN));
     NMC_TRY(dalloc(x, &x->dG2, mats));
-    NMC_TRY(dalloc(x, &x->dT12, mats));
-    NMC_TRY(dalloc(x, &x->dXa, mats));
-    NMC_TRY(dalloc(x, &x->dXb, mats));
+    if (!x->frags()) {
+      NMC_TRY(dalloc(x, &x->dT12, mats));
+      NMC_TRY(dalloc(x, &x->dXa, mats));
+      NMC_TRY(dalloc(x, &x->dXb, mats));
+    }
     NMC_TRY(dalloc(x, &x->dEmh2, NN));
     NMC_TRY(dalloc(x, &x->dEph2, NN));
-    x->oz = x->tc();
-    if (x->oz && !x->dry && !gemm_tc_supported(x->N))
+    x->oz = x->tc() && !x->frags();
+    if (x->tc() && !x->dry && !gemm_tc_supported(x->N))
       return fail(x, NMC_EINVAL, "NMC_SPLIT_BF16 needs N <= 320 and the TMA tensor-map encoder");
     if (x->oz)
       for (int a = 0; a < 4; ++a)
@@ -349,6 +360,13 @@ nmc_status alloc_all(nmc_ctx* x) {
           NMC_TRY(dalloc(x, &x->dOzExp[a][r], x->N));
         }
   }
+  if (x->frags())
+    for (int a = 0; a < 4; ++a)
+      for (int r = 0; r < 2; ++r) {
+        const size_t bytes = x->tc() ? frag_bytes<df2>(x->N) : frag_bytes<double>(x->N);
+        NMC_TRY(dalloc(x, &x->dFrag[a][r], bytes / sizeof(uint4)));
+        NMC_TRY(dalloc(x, &x->dFragScale[a][r], (x->N + 15) / 16 * 16));
+      }
   x->slot.assign(x->nb + 1, UDTBuf{});
   auto alloc_udt = [&](UDTBuf& u) -> nmc_status {
     NMC_TRY(dalloc(x, &u.U, mats));
@@ -398,6 +416,14 @@ nmc_status alloc_all(nmc_ctx* x) {
           if (!tc_prepare_const(src[a], x->N, r, x->dOz[a][r], x->dOzExp[a][r], x->tmap[a][r], st))
             return fail(x, NMC_ECUDA, "cuTensorMapEncodeTiled failed for the constant's slices");
     }
+  }
+  if (x->frags()) {
+    const double* src[4] = {x->dEm, x->dEp, x->dEmh, x->dEph};
+    for (int a = 0; a < 4; ++a)
+      for (int r = 0; r < 2; ++r) {
+        if (x->tc()) prepare_frags<df2>(src[a], x->N, r == 1, x->dFrag[a][r], x->dFragScale[a][r], st);
+        else prepare_frags<double>(src[a], x->N, r == 1, x->dFrag[a][r], x->dFragScale[a][r], st);
+      }
   }
   NMC_CUDA(x, cudaGetLastError());
   NMC_CUDA(x, cudaStreamSynchronize(st));
@@ -474,6 +500,12 @@ DfGemmArgs df_base(const nmc_ctx* x, const df2* A, long long sA, const df2* B, l
   return g;
 }
 
+void set_value(double& y, double v) { y = v; }
+void set_value(df2& y, double v) {
+  y.hi = (float)v;
+  y.lo = (float)(v - (double)y.hi);
+}
+
 enum ConstId { OZ_EM = 0, OZ_EP = 1, OZ_EMH = 2, OZ_EPH = 3 };
 
 // Double-float product with one constant operand: tensor cores (exact BF16 slicing) when
@@ -490,6 +522,37 @@ void df_gemm(nmc_ctx* x, DfGemmArgs& g, int const_id, bool const_is_a) {
   }
 }
 
+// Whole-matrix products of wrap.cu: C = constant `left` X constant `right` with the slice's field
+template <typename T>
+void wrap_frags(nmc_ctx* x, const T* X, T* C, double* Cd, int left, int right, const int8_t* fields, bool before) {
+  WrapArgs<T> g;
+  g.N = x->N; g.batch = x->batch(); g.ns = x->ns();
+  g.X = X; g.sX = x->NN();
+  g.C = C; g.Cd = Cd;
+  g.L = x->dFrag[left][0]; g.Le = x->dFragScale[left][0];
+  g.R = x->dFrag[right][1]; g.Re = x->dFragScale[right][1];
+  g.fields = fields; g.fstride = (long long)x->Lt * x->N; g.before = before;
+  set_value(g.e2, std::exp(2.0 * x->lam));
+  set_value(g.em2, std::exp(-2.0 * x->lam));
+  launch(x, KC_GEMM_TC, [&] { wrap_product(g, x->st()); });
+}
+// X = (block j's product, transposed for the left stack) U D
+template <typename T>
+void chain_frags(nmc_ctx* x, int j, const UDTView& src, double* X, bool right) {
+  ChainArgs<T> g;
+  g.N = x->N; g.batch = x->batch(); g.ns = x->ns(); g.w = x->w;
+  g.l0 = right ? j * x->w : (j + 1) * x->w - 1;
+  g.dl = right ? 1 : -1;
+  g.U = src.U; g.sU = src.sU; g.Dv = src.D; g.sD = src.sD;
+  g.X = X;
+  g.L = x->dFrag[OZ_EM][0]; g.Le = x->dFragScale[OZ_EM][0];
+  g.fields = x->dS; g.fstride = (long long)x->Lt * x->N; g.before = right;
+  g.d1 = std::exp(x->lam); g.dm1 = std::exp(-x->lam);
+  set_value(g.e1, g.d1);
+  set_value(g.em1, g.dm1);
+  launch(x, KC_GEMM_TC, [&] { chain_product(g, x->st()); });
+}
+
 UDTView identity_view(const nmc_ctx* x) { return UDTView{x->dI, 0, x->dOnes, 0, x->dI, 0}; }
 UDTView view_of(const nmc_ctx* x, const UDTBuf& b) {
   return UDTView{b.U, x->NN(), b.D, x->N, b.T, x->NN()};
@@ -499,6 +562,13 @@ UDTView view_of(const nmc_ctx* x, const UDTBuf& b) {
 void wrap(nmc_ctx* x, int l, bool up) {
   cudaStream_t st = x->st();
   const long long NN = x->NN();
+  if (x->frags()) {   // up: Em (e^V G e^-V) Ep; down: e^-V (Ep G Em) e^V
+    const int8_t* fl = x->dS + (long long)l * x->N;
+    const int a = up ? OZ_EM : OZ_EP, c = up ? OZ_EP : OZ_EM;
+    if (x->tc()) wrap_frags<df2>(x, x->dG2, x->dG2, nullptr, a, c, fl, up);
+    else wrap_frags<double>(x, x->dG, x->dG, nullptr, a, c, fl, up);
+    return;
+  }
   if (x->dfp()) {
     const int8_t* fl = x->dS + (long long)l * x->N;
     if (up) {  // T1 = Em (e^V G e^-V); G = T1 Ep
@@ -601,6 +671,13 @@ void stack_update(nmc_ctx* x, int j, const UDTView& src, const UDTBuf& dst, bool
   const int w = x->w;
   double* X = x->dX;
   double* X2 = x->dX2;
+  if (x->frags()) {
+    if (x->tc()) chain_frags<df2>(x, j, src, X, right);
+    else chain_frags<double>(x, j, src, X, right);
+    launch(x, KC_QRP, [&] { qrp_udt(X, dst.U, dst.D, x->dTp, x->dWS, x->N, x->batch(), st); });
+    stab_gemm(x, gemm_base<double>(x, x->dTp, NN, src.T, src.sT, dst.T));
+    return;
+  }
   if (x->dfp()) {
     // (B_block U) in double-float, then X = (B_block U) D in FP64 for the QR:
     // right: B_block = B_{(j+1)w-1} ... B_{jw}; left (transposed): B_{jw}^T ... B_{(j+1)w-1}^T
@@ -702,6 +779,12 @@ void measure_now(nmc_ctx* x) {
   cudaStream_t st = x->st();
   const long long NN = x->NN();
   double* acc = x->dSeries;   // + (device series index) * chains * 8
+  if (x->frags()) {   // G~ = e^{dtau K/2} G e^{-dtau K/2}
+    if (x->tc()) wrap_frags<df2>(x, x->dG2, nullptr, x->dM1, OZ_EPH, OZ_EMH, nullptr, false);
+    else wrap_frags<double>(x, x->dG, nullptr, x->dM1, OZ_EPH, OZ_EMH, nullptr, false);
+    launch(x, KC_MEASURE, [&] { nmc::measure(x->dM1, x->dK, x->dSign, x->N, x->Lx, x->lattice, x->U, acc, x->chains(), x->ns(), st, x->dCtr + 1); });
+    return;
+  }
   if (x->dfp()) {  // G~ = e^{dtau K/2} G e^{-dtau K/2} from the pair copy of the recomputed G
     DfGemmArgs g = df_base(x, x->dEph2, 0, x->dG2, NN);
     g.C = x->dT12;
@@ -834,7 +917,7 @@ nmc_status ensure_series(nmc_ctx* x, long long need) {
 // first failed index check of the NMC_DEBUG build (0: none, or not a debug build)
 unsigned int debug_failed() {
   unsigned int (*const readers[])() = {debug_fail_flip, debug_fail_stab, debug_fail_gemm,
-                                       debug_fail_gemm_fx, debug_fail_gemm_tc, debug_fail_misc};
+                                       debug_fail_gemm_fx, debug_fail_gemm_tc, debug_fail_wrap, debug_fail_misc};
   for (auto r : readers)
     if (const unsigned int id = r()) return id;
   return 0u;

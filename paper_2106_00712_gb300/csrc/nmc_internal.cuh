@@ -51,6 +51,7 @@ unsigned int debug_fail_stab();
 unsigned int debug_fail_gemm();
 unsigned int debug_fail_gemm_fx();
 unsigned int debug_fail_gemm_tc();
+unsigned int debug_fail_wrap();
 unsigned int debug_fail_misc();
 
 constexpr uint32_t kTagFlip = 0u;
