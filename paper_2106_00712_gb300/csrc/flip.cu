@@ -14,9 +14,13 @@
 // memory (L2); the panels always live in shared memory (k is clamped to fit).
 // That is k_flip (FP32) and, above some 560 sites, k_flip (FP64) and k_flip_df (FP32 pairs); up to
 // there FP64 and FP32 pairs take k_flip_block, which decides blocks of up to min(k, 16) sites apart.
+#include <cooperative_groups.h>
+
 #include "fold16.cuh"
 #include "nmc_internal.cuh"
 #include "oz_slice.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace nmc {
 
@@ -595,8 +599,8 @@ __global__ void __launch_bounds__(kThreadsDf, 2) k_flip_df(const FlipArgs<df2> f
 // Without tensor cores (FP32X2) the vectors go through shared memory to the FP32-pair loop.
 //
 // One slice, us, 44% of the flips accepted, one flip at a time (k_flip, k_flip_df) -> here:
-//   64 sites x 256 chains, both spins: FP32 pairs 133 -> 73, FP64 357 -> 155, FP32X2 133 -> 108
-//   72 x 1024, one spin: 625 -> 243;  256 x 32: 2950 -> 989;  100 x 64: 481 -> 135;
+//   64 sites x 256 chains, both spins: FP32 pairs 133 -> 75, FP64 357 -> 147, FP32X2 133 -> 110
+//   72 x 1024, one spin: 625 -> 242;  256 x 32: 2950 -> 391;  100 x 64: 481 -> 118;
 //   16 x 1 in FP64: 31 -> 16.
 // What bounds it at 64 x 256 (two CTAs per SM): latency. Of a slice's 146k cycles the decisions take
 // 45k (28 acceptances of some 1500: two ratios, a reciprocal and four rows' updates in a dependent
@@ -635,6 +639,13 @@ template <> struct Arith<double> {
   static __device__ __forceinline__ double finish(double a) { return a; }
   static __device__ __forceinline__ double div(double a, double b) { return a / b; }
 };
+
+// a load that does not look into the SM's own cache
+__device__ __forceinline__ double ld_l2(const double* p) { return __ldcg(p); }
+__device__ __forceinline__ df2 ld_l2(const df2* p) {
+  const float2 v = __ldcg((const float2*)p);
+  return df2{v.x, v.y};
+}
 
 template <typename T> __device__ __forceinline__ T delta(const FlipArgs<T>& f, bool plus);
 template <> __device__ __forceinline__ df2 delta<df2>(const FlipArgs<df2>& f, bool plus) { return plus ? f.dp2 : f.dm2; }
@@ -684,6 +695,118 @@ struct BlockStage {
   int m[2];                   // accepted flips, by block parity: see the loop
 };
 
+// The decisions of the block of kb sites from i0 on, by the first kDecide warps: entry(s, t, j) is G^'s
+// row t and column j of the block for spin s. Leaves the accepted flips in st, their number in
+// st.m[slot], and the flipped signs in sl.
+template <typename T, typename F>
+__device__ __forceinline__ void decide_block(const FlipArgs<T>& f, BlockStage<T>& st, int i0, int kb, int slot,
+                                             const unsigned* u, int8_t* sl, const uint8_t* rp, double& sign,
+                                             unsigned long long& n_acc, unsigned long long& n_dis, F entry) {
+  typedef Arith<T> A;
+  const int ns = f.ns, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int sp = ns == 2 ? lane >> 4 : 0, j = lane & 15;   // this lane's spin and column
+  const float fm = (float)f.dm, fp = (float)f.dp;
+  T* S = &st.S[sp][0][j];   // this lane's column: row t at S[t * kSites]
+#pragma unroll
+  for (int t = 4 * warp; t < 4 * warp + 4; ++t)
+    S[t * kSites] = t < kb && j < kb ? entry(sp, t, j) : A::zero();
+  const int jj = min(j, kb - 1), s_j = sl[i0 + jj];   // (read before the first flip's write, see the barrier)
+  const bool pos = s_j > 0;
+  const unsigned u_j = u[i0 + jj];
+  const float uf = (float)u_j * 0x1p-32f, du = pos ? fm : fp, dd = pos ? fp : fm;
+  bar_decide();
+  int m = 0;
+  for (int lo = 0; lo < kb;) {   // sites below lo are decided
+    // every remaining site as if it were the next: lane j site j
+    const T gu = st.S[0][jj][jj], gd = ns == 2 ? st.S[1][jj][jj] : gu;
+    const float hu = 1.f - A::top(gu), hd = ns == 2 ? 1.f - A::top(gd) : A::top(gu);
+    const float R32 = (1.f + du * hu) * (1.f + dd * hd);
+    // FP32's error: a few 2^-24 of (1 + |du| (1 + |g|)) (1 + |dd| (1 + |g|))
+    const float bound = 2e-6f * (1.f + fabsf(du) * (1.f + fabsf(hu))) *
+                        (1.f + fabsf(dd) * (1.f + fabsf(hd)));
+    const bool open = j >= lo && j < kb;
+    bool mine = uf < fabsf(R32), neg = R32 < 0.f;
+    if (open && (rp || !(fabsf(uf - fabsf(R32)) > bound))) {   // in FP64, from the same G^_ii
+      const double g64 = A::wide(gu), h64 = ns == 2 ? 1.0 - A::wide(gd) : g64;
+      const double R = (1.0 + (pos ? f.dm : f.dp) * (1.0 - g64)) *
+                       (1.0 + (pos ? f.dp : f.dm) * h64);
+      mine = (double)u_j * 0x1p-32 < fabs(R);
+      neg = R < 0.0;
+    }
+    bool take = mine;
+    if (rp) take = rp[i0 + jj] != 0;
+    const unsigned takes = __ballot_sync(0xffffffffu, open && take) & 0xffffu;
+    const int b = takes ? __ffs(takes) - 1 : kb;      // the next accepted site; the rest up to it are rejected
+    if (rp)
+      n_dis += __popc(__ballot_sync(0xffffffffu, open && j <= b && take != mine) & 0xffffu);
+    if (b == kb) break;
+    ++n_acc;
+    if (__shfl_sync(0xffffffffu, (int)neg, b)) sign = -sign;
+    const bool posb = __shfl_sync(0xffffffffu, (int)pos, b);
+    // y = (Delta / R) row of G^, on every lane its entry
+    const T d = posb == (sp == 0) ? delta<T>(f, false) : delta<T>(f, true);
+    const T R = A::add(A::one(), A::mul(d, A::sub(A::one(), st.S[sp][b][b])));
+    const T q = A::div(d, R);
+    const T y = A::mul(q, S[b * kSites]);
+    if (!NMC_DCHECK(m < kSites && b < kSites, 121)) break;
+    if (warp == 0) {
+      st.y[sp][m][j] = y;
+      st.c[sp][m] = q;
+      if (lane == 0) {
+        st.site[m] = b;
+        sl[i0 + b] = (int8_t)(posb ? -1 : 1);
+      }
+    }
+    // this warp's rows below b: G^ += x y^T, x the column of site b
+    if (4 * warp + 3 > b) {
+      T z[4], x[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        x[k] = st.S[sp][4 * warp + k][b];
+        z[k] = S[(4 * warp + k) * kSites];
+      }
+      __syncwarp();
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        A::fma_acc(z[k], x[k], y);
+        if (4 * warp + k > b) {
+          S[(4 * warp + k) * kSites] = A::finish(z[k]);
+          st.x[sp][m][4 * warp + k] = x[k];
+        }
+      }
+    }
+    ++m;
+    lo = b + 1;
+    bar_decide();
+  }
+  if (threadIdx.x == 0) st.m[slot] = m;
+}
+
+// x_q[r] (kind 0) or y_q[r] (kind 1) of the block's m flips for spin sv; rel: r less the block's first
+// site; entry(s): G's entry at row r and the block's column s (kind 1: row s and column r)
+template <typename T, typename F>
+__device__ __forceinline__ void block_vectors(const BlockStage<T>& st, int kind, int sv, int rel, int m,
+                                              T (&v)[kSites], F entry) {
+  typedef Arith<T> A;
+  const T* coef = kind ? &st.x[sv][0][0] : &st.y[sv][0][0];
+  T g[kSites];
+#pragma unroll
+  for (int p = 0; p < kSites; ++p) g[p] = p < m ? entry(st.site[p]) : A::zero();
+#pragma unroll
+  for (int p = 0; p < kSites; ++p) {
+    v[p] = A::zero();
+    if (p >= m) continue;
+    const int s = st.site[p];
+    T z = g[p];
+#pragma unroll
+    for (int q = 0; q < p; ++q) A::fma_acc(z, coef[q * kSites + s], v[q]);
+    z = A::finish(z);
+    if (kind) z = A::mul(st.c[sv][p], z);
+    else if (rel == s) z = A::sub(z, A::one());
+    v[p] = z;
+  }
+}
+
 template <typename T>
 __host__ __device__ inline size_t block_smem(int N, int ns, bool g_in_smem, int fold, int ld) {
   const int Np = (N + 15) & ~15;
@@ -701,7 +824,7 @@ k_flip_block(const FlipArgs<T> f, int kb_max) {
   typedef Arith<T> A;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int c = blockIdx.x, N = f.N, ns = f.ns, Np = (N + 15) & ~15;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = tid >> 5;
   const int ld = GS ? N + 2 : N;   // (rows of a column read on different banks)
   const long long NN = (long long)N * N, sG = GS ? (long long)N * ld : NN;
   T* Gs = (T*)smraw;
@@ -734,116 +857,26 @@ k_flip_block(const FlipArgs<T> f, int kb_max) {
       const int r = e / (N / 2);
       *(float4*)(Gs + 2 * e + r * (ld - N)) = *(const float4*)(Gg + 2 * e);
     }
-  const float fm = (float)f.dm, fp = (float)f.dp;
   double sign = 1.0;
   unsigned long long n_acc = 0, n_dis = 0;
   __syncthreads();
 
-  const int sp = ns == 2 ? lane >> 4 : 0, j = lane & 15;   // deciding warps: this lane's spin and column
   // (A block without a flip has one barrier: thread 0 may then write the next block's count while
   // slower warps still read this one's, hence two slots. It writes this slot again only after every
   // warp has passed the next block's barrier.)
   for (int i0 = 0, blk = 0; i0 < N; i0 += kb_max, ++blk) {
     const int kb = min(kb_max, N - i0);
-    if (warp < kDecide) {
-      // ------------------------------------------------------------ decisions of the block
-      T* S = &st.S[sp][0][j];   // this lane's column: row t at S[t * kSites]
-#pragma unroll
-      for (int t = 4 * warp; t < 4 * warp + 4; ++t)
-        S[t * kSites] = t < kb && j < kb ? G[sp * sG + (long long)(i0 + t) * ld + i0 + j] : A::zero();
-      const int jj = min(j, kb - 1), s_j = sl[i0 + jj];   // (read before the first flip's write, see the barrier)
-      const bool pos = s_j > 0;
-      const unsigned u_j = u[i0 + jj];
-      const float uf = (float)u_j * 0x1p-32f, du = pos ? fm : fp, dd = pos ? fp : fm;
-      bar_decide();
-      int m = 0;
-      for (int lo = 0; lo < kb;) {   // sites below lo are decided
-        // every remaining site as if it were the next: lane j site j
-        const T gu = st.S[0][jj][jj], gd = ns == 2 ? st.S[1][jj][jj] : gu;
-        const float hu = 1.f - A::top(gu), hd = ns == 2 ? 1.f - A::top(gd) : A::top(gu);
-        const float R32 = (1.f + du * hu) * (1.f + dd * hd);
-        // FP32's error: a few 2^-24 of (1 + |du| (1 + |g|)) (1 + |dd| (1 + |g|))
-        const float bound = 2e-6f * (1.f + fabsf(du) * (1.f + fabsf(hu))) *
-                            (1.f + fabsf(dd) * (1.f + fabsf(hd)));
-        const bool open = j >= lo && j < kb;
-        bool mine = uf < fabsf(R32), neg = R32 < 0.f;
-        if (open && (rp || !(fabsf(uf - fabsf(R32)) > bound))) {   // in FP64, from the same G^_ii
-          const double g64 = A::wide(gu), h64 = ns == 2 ? 1.0 - A::wide(gd) : g64;
-          const double R = (1.0 + (pos ? f.dm : f.dp) * (1.0 - g64)) *
-                           (1.0 + (pos ? f.dp : f.dm) * h64);
-          mine = (double)u_j * 0x1p-32 < fabs(R);
-          neg = R < 0.0;
-        }
-        bool take = mine;
-        if (rp) take = rp[i0 + jj] != 0;
-        const unsigned takes = __ballot_sync(0xffffffffu, open && take) & 0xffffu;
-        const int b = takes ? __ffs(takes) - 1 : kb;      // the next accepted site; the rest up to it are rejected
-        if (rp)
-          n_dis += __popc(__ballot_sync(0xffffffffu, open && j <= b && take != mine) & 0xffffu);
-        if (b == kb) break;
-        ++n_acc;
-        if (__shfl_sync(0xffffffffu, (int)neg, b)) sign = -sign;
-        const bool posb = __shfl_sync(0xffffffffu, (int)pos, b);
-        // y = (Delta / R) row of G^, on every lane its entry
-        const T d = posb == (sp == 0) ? delta<T>(f, false) : delta<T>(f, true);
-        const T R = A::add(A::one(), A::mul(d, A::sub(A::one(), st.S[sp][b][b])));
-        const T q = A::div(d, R);
-        const T y = A::mul(q, S[b * kSites]);
-        if (!NMC_DCHECK(m < kSites && b < kSites, 121)) break;
-        if (warp == 0) {
-          st.y[sp][m][j] = y;
-          st.c[sp][m] = q;
-          if (lane == 0) {
-            st.site[m] = b;
-            sl[i0 + b] = (int8_t)(posb ? -1 : 1);
-          }
-        }
-        // this warp's rows below b: G^ += x y^T, x the column of site b
-        if (4 * warp + 3 > b) {
-          T z[4], x[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            x[k] = st.S[sp][4 * warp + k][b];
-            z[k] = S[(4 * warp + k) * kSites];
-          }
-          __syncwarp();
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            A::fma_acc(z[k], x[k], y);
-            if (4 * warp + k > b) {
-              S[(4 * warp + k) * kSites] = A::finish(z[k]);
-              st.x[sp][m][4 * warp + k] = x[k];
-            }
-          }
-        }
-        ++m;
-        lo = b + 1;
-        bar_decide();
-      }
-      if (tid == 0) st.m[blk & 1] = m;
-    }
+    if (warp < kDecide)
+      decide_block(f, st, i0, kb, blk & 1, u, sl, rp, sign, n_acc, n_dis,
+                   [&](int s, int t, int k) { return G[s * sG + (long long)(i0 + t) * ld + i0 + k]; });
     __syncthreads();
     const int m = st.m[blk & 1];
     if (m > 0) {
       // ---------------------------------------------------------- the vectors over all sites
-      // entry (kind, spin sv, r): x_q[r] (kind 0) or y_q[r] (kind 1) for every q
       auto vectors = [&](int kind, int sv, int r, T (&v)[kSites]) {
         const T* base = G + sv * sG + (kind ? (long long)i0 * ld + r : (long long)r * ld + i0);
-        const T* coef = kind ? &st.x[sv][0][0] : &st.y[sv][0][0];
         const int step = kind ? ld : 1;
-#pragma unroll
-        for (int p = 0; p < kSites; ++p) {
-          v[p] = A::zero();
-          if (p >= m) continue;
-          const int s = st.site[p];
-          T z = base[(long long)s * step];
-#pragma unroll
-          for (int q = 0; q < p; ++q) A::fma_acc(z, coef[q * kSites + s], v[q]);
-          z = A::finish(z);
-          if (kind) z = A::mul(st.c[sv][p], z);
-          else if (r == i0 + s) z = A::sub(z, A::one());
-          v[p] = z;
-        }
+        block_vectors(st, kind, sv, r - i0, m, v, [&](int s) { return base[(long long)s * step]; });
       };
       if constexpr (FOLD == kFoldPairs) {
         for (int t = tid; t < 2 * ns * N; t += THREADS) {
@@ -912,6 +945,111 @@ k_flip_block(const FlipArgs<T> f, int kb_max) {
   }
 }
 
+// The same for G in global memory and fewer chains than SMs: a cluster of CTAs per chain. Every CTA takes
+// all decisions (from the same G, so the same ones), forms and folds the rows of its share of 16-row
+// tiles, and forms the columns of the same share, whose digits it writes to every CTA of the cluster.
+// Each entry sees the operations of k_flip_block in the same order. The barriers do not depend on what
+// was decided. 256 sites x 32 chains, us: one CTA per chain 966, two 557, four 391; eight (x 16 chains)
+// 585 for four's 383. 100 x 64 with two 118 against 133 with G in shared memory; 64 x 32 59 against 55,
+// hence kClusterMinN where shared memory would do.
+constexpr int kClusterMinN = 96;
+
+template <typename T>
+__host__ __device__ inline size_t cluster_smem(int N, int ns, int cs) {
+  const int tiles = (N + 15) >> 4, own = (tiles + cs - 1) / cs * 16, Np = tiles * 16;
+  return (size_t)ns * (own + Np) * (kFDig * 32 + 4) + sizeof(BlockStage<T>) + (size_t)N * 4 + ((N + 15) & ~15) + 64;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(512, 1)
+k_flip_cluster(const FlipArgs<T> f, int kb_max) {
+  constexpr int THREADS = 512;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  cg::cluster_group cl = cg::this_cluster();
+  const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int c = blockIdx.x / cs, N = f.N, ns = f.ns, tiles = (N + 15) >> 4, Np = tiles * 16;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  const int own = (tiles + cs - 1) / cs * 16;                    // rows of the largest share
+  const int r0 = tiles * rank / cs * 16, nr = max(min(tiles * (rank + 1) / cs * 16, N) - r0, 0);
+  const long long NN = (long long)N * N;
+  T* G = f.G + (long long)c * ns * NN;
+  const int xs = own * 32, ys = Np * 32;                         // bytes per digit
+  unsigned char* xd = smraw;                                     // [spin][digit][own rows]
+  unsigned char* yd = xd + (size_t)ns * kFDig * xs;              // [spin][digit][columns]
+  int* xe = (int*)(yd + (size_t)ns * kFDig * ys);
+  int* ye = xe + ns * own;
+  BlockStage<T>& st = *(BlockStage<T>*)(ye + ns * Np);
+  unsigned* u = (unsigned*)(&st + 1);
+  int8_t* sl = (int8_t*)(u + N);
+
+  int8_t* fl = f.fields + ((long long)c * f.L + f.l) * N;
+  const uint32_t gchain = (uint32_t)(f.chain_id ? f.chain_id[c] : f.chain_offset + c);
+  const uint32_t sweep = (uint32_t)((f.ctr ? f.ctr[0] : (long long)f.sweep) -
+                                    (f.sweep_base ? f.sweep_base[c] : 0));
+  const uint8_t* rp = f.replay ? f.replay + ((long long)c * f.L + f.l) * N : nullptr;
+  for (int i = tid; i < N; i += THREADS) {
+    sl[i] = fl[i];
+    uint32_t ctr[4] = {(uint32_t)(f.l * N + i), sweep, gchain, kTagFlip};
+    philox4x32_10(ctr, f.key0, f.key1);
+    u[i] = ctr[0];
+  }
+  double sign = 1.0;
+  unsigned long long n_acc = 0, n_dis = 0;
+  cl.sync();   // (no CTA writes the fields or another's memory before all have begun)
+
+  for (int i0 = 0, blk = 0; i0 < N; i0 += kb_max, ++blk) {
+    const int kb = min(kb_max, N - i0);
+    if (warp < kDecide)   // (rows of other shares: past the L1)
+      decide_block(f, st, i0, kb, blk & 1, u, sl, rp, sign, n_acc, n_dis,
+                   [&](int s, int t, int k) { return ld_l2(G + s * NN + (long long)(i0 + t) * N + i0 + k); });
+    __syncthreads();
+    const int m = st.m[blk & 1];
+    if (m > 0) {
+      for (int t = tid; t < 2 * ns * nr; t += THREADS) {
+        const int kind = t / (ns * nr), e = t - kind * ns * nr, sv = e / nr, k = e - sv * nr, r = r0 + k;
+        const T* base = G + sv * NN + (kind ? (long long)i0 * N + r : (long long)r * N + i0);
+        const int step = kind ? N : 1;
+        T v[kSites];
+        block_vectors(st, kind, sv, r - i0, m, v, [&](int s) { return ld_l2(base + (long long)s * step); });
+        int E = Digits<T>::kExpMin;
+#pragma unroll
+        for (int p = 0; p < kSites; ++p) E = max(E, Digits<T>::expo(v[p]));
+        if (kind == 0) {
+          xe[sv * own + k] = Digits<T>::scale(E);
+          cut16<T>(v, E, xd + (size_t)sv * kFDig * xs, k, xs);
+        } else {
+          for (int q = 0; q < cs; ++q) cl.map_shared_rank(ye, q)[sv * Np + r] = Digits<T>::scale(E);
+          unsigned char* dst = yd + (size_t)sv * kFDig * ys;
+          cut16_to(v, E, [&](int s, int h, uint4 w) {
+            for (int q = 0; q < cs; ++q)
+              *reinterpret_cast<uint4*>(cl.map_shared_rank(dst, q) + s * ys + digit_off(r, h)) = w;
+          });
+        }
+      }
+    }
+    cl.sync();
+    if (m > 0 && nr > 0)
+      for (int sv = 0; sv < ns; ++sv) {
+        T* Gf = G + sv * NN + (long long)r0 * N;
+        fold_tiles<T>([&](int r) { return Gf + (long long)r * N; },
+                      (unsigned)__cvta_generic_to_shared(xd + (size_t)sv * kFDig * xs), xs, xe + sv * own,
+                      (unsigned)__cvta_generic_to_shared(yd + (size_t)sv * kFDig * ys), ys, ye + sv * Np,
+                      nr, N, true, warp, THREADS / 32);
+      }
+    __threadfence();
+    cl.sync();
+  }
+  if (rank == 0) {
+    for (int i = tid; i < N; i += THREADS) fl[i] = sl[i];
+    if (tid == 0) {
+      f.sign[c] *= sign;
+      f.counts[3 * c + 0] += (unsigned long long)N;
+      f.counts[3 * c + 1] += n_acc;
+      f.counts[3 * c + 2] += n_dis;
+    }
+  }
+}
+
 }  // namespace
 
 size_t flip_smem_bytes(int N, int kk, size_t elem, int g_in_smem, int ns) {
@@ -927,6 +1065,23 @@ namespace {
 
 constexpr size_t kBlockSmem = 226 * 1024;   // (227 KB are available)
 
+template <typename T>
+void flip_cluster(const FlipArgs<T>& f, int n_chains, int kb, int cs, cudaStream_t st) {
+  allow_max_dynamic_smem((const void*)k_flip_cluster<T>);
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cs;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(n_chains * cs);
+  cfg.blockDim = dim3(512);
+  cfg.dynamicSmemBytes = cluster_smem<T>(f.N, f.ns, cs);
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_flip_cluster<T>, f, kb);   // (an error is seen by the launch's next check)
+}
+
 // One slice by k_flip_block; false: the vectors of a block do not fit shared memory. G is held
 // there when it fits with them. 256 threads, two CTAs per SM, when there are more chains than
 // SMs; 512 otherwise. (Neither choice changes a bit of the results.)
@@ -935,8 +1090,17 @@ bool flip_block(const FlipArgs<T>& f, int n_chains, cudaStream_t st) {
   size_t bytes = block_smem<T>(f.N, f.ns, true, FOLD, f.N + 2);
   const bool gs = bytes <= kBlockSmem;
   if (!gs) bytes = block_smem<T>(f.N, f.ns, false, FOLD, f.N);
-  if (bytes > kBlockSmem) return false;
   const int kb = f.kk < kSites ? f.kk : kSites;
+  if constexpr (FOLD == kFoldTensor)
+    if (!gs || f.N >= kClusterMinN) {
+      int cs = 4;
+      while (cs > 1 && (n_chains * cs > sm_count() || cluster_smem<T>(f.N, f.ns, cs) > kBlockSmem)) cs >>= 1;
+      if (cs > 1) {
+        flip_cluster(f, n_chains, kb, cs, st);
+        return true;
+      }
+    }
+  if (bytes > kBlockSmem) return false;
   auto run = [&](auto kernel, int threads) {
     allow_max_dynamic_smem((const void*)kernel);
     kernel<<<n_chains, threads, bytes, st>>>(f, kb);

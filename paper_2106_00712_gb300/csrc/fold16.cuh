@@ -89,9 +89,10 @@ template <> struct Digits<double> {
 // exchanged in every second group of four rows so that ldmatrix meets all banks
 __device__ __forceinline__ int digit_off(int r, int h) { return r * 32 + ((h ^ ((r >> 2) & 1)) << 4); }
 
-// Cut the 16 terms of one row (or column) into digits, most significant first, `stride` bytes apart
-template <typename T>
-__device__ __forceinline__ void cut16(const T (&x)[kFoldK], int E, unsigned char* dst, int r, int stride) {
+// Cut the 16 terms of one row (or column) into digits, most significant first: store(s, h, .) takes
+// half h of digit s
+template <typename T, typename F>
+__device__ __forceinline__ void cut16_to(const T (&x)[kFoldK], int E, F store) {
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     unsigned w[4][kFDig];
@@ -105,9 +106,14 @@ __device__ __forceinline__ void cut16(const T (&x)[kFoldK], int E, unsigned char
         const __half2 v = __hadd2(*reinterpret_cast<__half2*>(&w[i][s]), __float2half2_rn(-1536.f));
         d[i] = *reinterpret_cast<const unsigned*>(&v);
       }
-      *reinterpret_cast<uint4*>(dst + s * stride + digit_off(r, h)) = make_uint4(d[0], d[1], d[2], d[3]);
+      store(s, h, make_uint4(d[0], d[1], d[2], d[3]));
     }
   }
+}
+// to row r at dst, `stride` bytes apart
+template <typename T>
+__device__ __forceinline__ void cut16(const T (&x)[kFoldK], int E, unsigned char* dst, int r, int stride) {
+  cut16_to(x, E, [&](int s, int h, uint4 v) { *reinterpret_cast<uint4*>(dst + s * stride + digit_off(r, h)) = v; });
 }
 
 __device__ __forceinline__ void ldm4(unsigned (&r)[4], unsigned addr) {

@@ -78,3 +78,21 @@ def test_forced_decisions(nmc, mode):
             for ch in range(2):
                 assert abs(per[ch].accept - accept[ch].mean()) < 1e-15
     assert got[0] == got[1] > 0
+
+
+@pytest.mark.parametrize("mode", ["fp64", "split"])
+@pytest.mark.parametrize("lattice,Lx,Ly", [("honeycomb", 7, 7), ("square", 12, 12), ("honeycomb", 9, 9)])
+def test_clusters_change_no_bit(nmc, mode, lattice, Lx, Ly):
+    """Few chains take several CTAs each, many one: 4 (2 chains), 2 (60) and 1 (160), with 16-row
+    tiles that do not divide evenly (N = 98, 144, 162): the same bits."""
+    prec = nmc.NMC_FP64 if mode == "fp64" else nmc.NMC_SPLIT_BF16
+    got = []
+    for chains in (2, 60, 160):
+        with nmc.Context(Lx, Ly, 1.0, 4.0, 0.5, 0.1, 5, seed=2, lattice=lattice, n_chains=chains,
+                         precision=prec, drift_tol=1e-3) as c:
+            c.generate()
+            c.sweep(1, measure=1)
+            got.append((c.fields()[:2].copy(), [c.green(ch, sp).copy() for ch in (0, 1) for sp in (0, 1)]))
+    for f, G in got[1:]:
+        assert np.array_equal(f, got[0][0])
+        assert all(np.array_equal(a, b) for a, b in zip(G, got[0][1]))
