@@ -301,7 +301,7 @@ nmc_status nmc_graph_stats(const nmc_ctx* ctx, long long* recorded, long long* r
  *   d_fields: device, int8 [n_chains][L_tau][N], values +-1;
  *   d_G: device output, [n_chains][2][N][N] row-major (spin 0 = up).
  * Work is enqueued on cuda_stream (NULL = legacy default stream); outputs are valid once
- * the stream reaches that point. Scratch: a fixed array of 4,194,304 doubles (32 MiB) in
+ * the stream reaches that point (until then d_G holds intermediate products). Scratch: a fixed array of 4,194,304 doubles (32 MiB) in
  * the library, held by every GPU that loads it until exit. Chains are processed in chunks
  * that fit; one chain needs 20 N^2 + 4 N doubles (24 N^2 + 4 N when N > 111), so
  * NMC_EINVAL is returned, before any work is enqueued, when that exceeds the array

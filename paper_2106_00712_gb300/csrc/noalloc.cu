@@ -15,6 +15,7 @@
 
 #include "../../include/nmc.h"
 #include "nmc_internal.cuh"
+#include "wrap.cuh"
 
 namespace nmc {
 bool stab_needs_workspace(int N);
@@ -107,12 +108,21 @@ extern "C" nmc_status nmc_green_noalloc(int N, int L_tau, int n_wrap, double lam
     return NMC_EINVAL;
   const long long NN = (long long)N * N;
   const bool ws_needed = stab_needs_workspace(N);
-  // per chain (2 matrices): X, X2, Tp, U x2, T x2, M1, Xs, Y (10 N^2), D x2 (2 N), and the
-  // QR / solve workspace (2 N^2) when a matrix does not fit in shared memory.
-  const size_t per_chain = 2 * (10 * (size_t)NN + 2 * (size_t)N + (ws_needed ? 2 * (size_t)NN : 0));
-  const size_t shared = round256(NN) + round256(N) + 16 * 32;  // I, ones, alignment slack
-  if (shared + per_chain > kScratchDoubles) return NMC_EINVAL;  // one chain does not fit
-  const int chunk = (int)((kScratchDoubles - shared) / per_chain);
+  // A chain is accepted by the documented bound, 20 N^2 + 4 N doubles (24 N^2 with the QR's and the
+  // solve's workspace). What it takes is less: U, the two T, D and the workspace; the output holds
+  // Tp and X until G is written.
+  const size_t bound = 2 * (10 * (size_t)NN + 2 * (size_t)N + (ws_needed ? 2 * (size_t)NN : 0));
+  const size_t per_chain = 2 * (3 * (size_t)NN + (size_t)N + (ws_needed ? 2 * (size_t)NN : 0));
+  size_t shared = round256(NN) + round256(N) + 16 * 32;  // I, ones, alignment slack
+  if (shared + bound > kScratchDoubles) return NMC_EINVAL;  // one chain does not fit
+  // block products by wrap.cu under the rule of a context in FP64
+  const bool frags = N % 2 == 0 && N > 16 && N <= kFragMaxN;
+  const size_t frag_doubles = frags ? round256(frag_bytes<double>(N) / sizeof(double)) : 0;
+  shared += frag_doubles + round256(kFragMaxN);
+  const int fit = (int)((kScratchDoubles - shared) / per_chain);
+  // equal chunks: 256 chains of 64 sites take two of 128 (with the bound's memory, five of 51 and one of
+  // 1: 13.0 ms a call of 40 slices with a launch per product, 4.6 now)
+  const int chunk = (n_chains + (n_chains + fit - 1) / fit - 1) / ((n_chains + fit - 1) / fit);
 
   // An error left pending by earlier work (not ours) is reported, not consumed.
   if (cudaPeekAtLastError() != cudaSuccess) return NMC_ECUDA;
@@ -123,8 +133,11 @@ extern "C" nmc_status nmc_green_noalloc(int N, int L_tau, int n_wrap, double lam
 
   double* I = base_ptr;
   double* ones = I + round256(NN);
-  double* p = ones + round256(N);
+  double* frag = ones + round256(N);
+  int* frag_scale = (int*)(frag + frag_doubles);
+  double* p = frag + frag_doubles + round256(kFragMaxN);
   set_identity_batch(I, ones, nullptr, N, 1, st);
+  if (frags) prepare_frags<double>(d_expK_m, N, false, frag, frag_scale, st);
 
   for (int c0 = 0; c0 < n_chains; c0 += chunk) {
     const int cc = (n_chains - c0 < chunk) ? n_chains - c0 : chunk;
@@ -132,16 +145,11 @@ extern "C" nmc_status nmc_green_noalloc(int N, int L_tau, int n_wrap, double lam
     const size_t m = round256((size_t)NN * B);  // one batch of matrices, stride N^2
     const size_t v = round256((size_t)N * B);   // one batch of vectors, stride N
     double* q = p;
-    double* X = q; q += m;
-    double* X2 = q; q += m;
-    double* Tp = q; q += m;
-    double* Ub[2] = {q, q + m}; q += 2 * m;
+    double* U = q; q += m;
     double* Tb[2] = {q, q + m}; q += 2 * m;
-    double* M1 = q; q += m;
-    double* Xs = q; q += m;
-    double* Y = q; q += m;
-    double* Db[2] = {q, q + v}; q += 2 * v;
+    double* D = q; q += v;
     double* ws = ws_needed ? q : nullptr;
+    double* Gc = d_G + (long long)c0 * 2 * NN;
     const int8_t* f = d_fields + (long long)c0 * L_tau * N;
 
     // left stack L_j, j = nb-1..0, starting from L_nb = I (identity, batch stride 0)
@@ -149,24 +157,37 @@ extern "C" nmc_status nmc_green_noalloc(int N, int L_tau, int n_wrap, double lam
     int out = 0;
     for (int j = nb - 1; j >= 0; --j) {
       const int lt = (j + 1) * n_wrap - 1;
-      GemmArgs<double> g = base(N, B, d_expK_m, 0, src.U, src.sU, X);
-      g.bcol = vscale(src.D, src.sD, SC_VEC);
-      g.crow = fscale(f, lt, N, L_tau, lam);
-      gemm(g, st);
-      double* x = X;
-      double* x2 = X2;
-      for (int l = lt - 1; l >= j * n_wrap; --l) {
-        GemmArgs<double> h = base(N, B, d_expK_m, 0, x, NN, x2);
-        h.crow = fscale(f, l, N, L_tau, lam);
-        gemm(h, st);
-        double* t = x; x = x2; x2 = t;
+      double* X = Tb[out];   // the block's product, until the new T takes its place
+      if (frags) {
+        ChainArgs<double> g;
+        g.N = N; g.batch = B; g.ns = 2; g.w = n_wrap; g.l0 = lt; g.dl = -1;
+        g.U = src.U; g.sU = src.sU; g.Dv = src.D; g.sD = src.sD;
+        g.X = X;
+        g.L = (const uint4*)frag; g.Le = frag_scale;
+        g.fields = f; g.fstride = (long long)L_tau * N;
+        g.e1 = g.d1 = std::exp(lam); g.em1 = g.dm1 = std::exp(-lam);
+        chain_product(g, st);
+      } else {
+        double* x = n_wrap % 2 ? X : Gc;   // (so that the last product lands in X)
+        double* x2 = n_wrap % 2 ? Gc : X;
+        GemmArgs<double> g = base(N, B, d_expK_m, 0, src.U, src.sU, x);
+        g.bcol = vscale(src.D, src.sD, SC_VEC);
+        g.crow = fscale(f, lt, N, L_tau, lam);
+        gemm(g, st);
+        for (int l = lt - 1; l >= j * n_wrap; --l) {
+          GemmArgs<double> h = base(N, B, d_expK_m, 0, x, NN, x2);
+          h.crow = fscale(f, l, N, L_tau, lam);
+          gemm(h, st);
+          double* t = x; x = x2; x2 = t;
+        }
       }
-      qrp_udt(x, Ub[out], Db[out], Tp, ws, N, B, st);
-      GemmArgs<double> gt = base(N, B, Tp, NN, src.T, src.sT, Tb[out]);
+      qrp_udt(X, U, D, Gc, ws, N, B, st);
+      GemmArgs<double> gt = base(N, B, Gc, NN, src.T, src.sT, Tb[out]);
       gemm(gt, st);
-      src = View{Ub[out], NN, Db[out], N, Tb[out], NN};
+      src = View{U, NN, D, N, Tb[out], NN};
       out ^= 1;
     }
+    double *M1 = Tb[out], *Xs = Gc, *Y = Tb[out];
     // G = (I + R L_0)^{-1} with R = I
     const View R{I, 0, ones, 0, I, 0};
     GemmArgs<double> g1 = base(N, B, R.U, R.sU, src.U, src.sU, M1);
@@ -181,7 +202,7 @@ extern "C" nmc_status nmc_green_noalloc(int N, int L_tau, int n_wrap, double lam
     g2.Cin = M1; g2.sCin = NN; g2.ldcin = N; g2.beta = 1.0;
     gemm(g2, st);
     solve_stab(Xs, R.U, R.sU, R.D, R.sD, Y, ws, N, B, st);
-    GemmArgs<double> g3 = base(N, B, src.U, src.sU, Y, NN, d_G + (long long)c0 * 2 * NN);
+    GemmArgs<double> g3 = base(N, B, src.U, src.sU, Y, NN, Gc);
     g3.brow = vscale(src.D, src.sD, SC_INV_MAX1);
     gemm(g3, st);
     // stop at the first failed launch instead of queueing later chunks behind it
