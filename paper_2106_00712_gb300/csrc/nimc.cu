@@ -452,19 +452,31 @@ __global__ void k_loss_gbar(const double* __restrict__ Gt, const double* __restr
 }
 
 // grad[c][l][i] = -lam sum_sigma sigma sum_a H_sigma[a][i] Q_sigma[a][i]   (one CTA per config)
-__global__ void k_grad_slice(const double* __restrict__ H, const double* __restrict__ Q, int N,
-                             double lam, double* __restrict__ grad, long long gstride) {
-  const int c = blockIdx.x;
+// One slice's derivative, 32 sites per block: lane = site, the sum over a shared out to the warps. (One
+// block per configuration with a thread per site waited out N dependent FP64 steps: 38 us at N = 72 and
+// 3 configurations, 7.4 now.)
+__global__ void __launch_bounds__(kThreads)
+k_grad_slice(const double* __restrict__ H, const double* __restrict__ Q, int N, double lam,
+             double* __restrict__ grad, long long gstride) {
+  constexpr int kWarps = kThreads / 32;
+  __shared__ double part[kWarps][32];
+  const int c = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, i = blockIdx.y * 32 + lane;
   const long long NN = (long long)N * N;
   const double* Hu = H + (long long)(2 * c) * NN;
   const double* Qu = Q + (long long)(2 * c) * NN;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    double su = 0.0, sd = 0.0;
-    for (int a = 0; a < N; ++a) {
+  double su = 0.0, sd = 0.0;
+  if (i < N)
+    for (int a = warp; a < N; a += kWarps) {
       su = fma(Hu[(long long)a * N + i], Qu[(long long)a * N + i], su);
       sd = fma(Hu[NN + (long long)a * N + i], Qu[NN + (long long)a * N + i], sd);
     }
-    grad[(long long)c * gstride + i] = -lam * (su - sd);
+  part[warp][lane] = su - sd;
+  __syncthreads();
+  if (warp == 0 && i < N) {
+    double s = part[0][lane];
+#pragma unroll
+    for (int w = 1; w < kWarps; ++w) s += part[w][lane];
+    grad[(long long)c * gstride + i] = -lam * s;
   }
 }
 
@@ -495,6 +507,8 @@ struct nmc_gen {
   int Bf = 0;      // configurations per generator chunk
   int device = 0;
   cudaStream_t stream = nullptr;
+  cudaStream_t side = nullptr;                  // right stacks (loss_chunk)
+  cudaEvent_t ready[2] = {}, used[2] = {};
   long long steps = 0;
   long long epochs = 0;   // epochs trained since creation / set_params (shuffle counter)
   double clip = 0.0;      // global gradient-norm bound (0: none)
@@ -513,7 +527,7 @@ struct nmc_gen {
   double *dLU = nullptr, *dLD = nullptr, *dLT = nullptr;  // left stacks, slots 0..nb-1
   double *dRU = nullptr, *dRD = nullptr, *dRT = nullptr;  // right stack (current)
   double *dRU2 = nullptr, *dRD2 = nullptr, *dRT2 = nullptr;
-  double *dW1 = nullptr, *dW2 = nullptr, *dTp = nullptr, *dWS = nullptr;
+  double *dW1 = nullptr, *dW2 = nullptr, *dTp = nullptr, *dWS = nullptr, *dWS2 = nullptr;
   double *dM1 = nullptr, *dXs = nullptr, *dXi = nullptr, *dT1 = nullptr, *dT2 = nullptr;
   double *dGl = nullptr, *dGl2 = nullptr, *dH = nullptr, *dH2 = nullptr;
   double *dG0 = nullptr, *dGt = nullptr, *dGbt = nullptr, *dGbar = nullptr, *dQ = nullptr;
@@ -577,9 +591,10 @@ GemmArgs<double> gbase(const nmc_gen* g, int batch, const double* A, long long s
 }
 
 // UDT-QRP of X into dst; dst.T = Tp * src.T
-void qrp_into(nmc_gen* g, int nb2, const double* X, const UDT& dst, const UDT& src) {
-  qrp_udt(X, dst.U, dst.D, g->dTp, g->dWS, g->N, nb2, g->stream);
-  gemm(gbase(g, nb2, g->dTp, g->NN(), src.T, src.sT, dst.T), g->stream);
+void qrp_into(nmc_gen* g, int nb2, const double* X, const UDT& dst, const UDT& src, double* ws,
+              cudaStream_t st) {
+  qrp_udt(X, dst.U, dst.D, g->dTp, ws, g->N, nb2, st);
+  gemm(gbase(g, nb2, g->dTp, g->NN(), src.T, src.sT, dst.T), st);
 }
 
 UDT identity_udt(const nmc_gen* g) { return UDT{g->dI, g->dOnes, g->dI, 0, 0, 0}; }
@@ -605,10 +620,11 @@ void left_update(nmc_gen* g, int nb2, int j, const UDT& src, const UDT& dst) {
     gemm(h, g->stream);
     std::swap(X, X2);
   }
-  qrp_into(g, nb2, X, dst, src);
+  qrp_into(g, nb2, X, dst, src, g->dWS, g->stream);
 }
 
-// R_{j+1} = B_{(j+1)w-1} ... B_{jw} R_j
+// R_{j+1} = B_{(j+1)w-1} ... B_{jw} R_j, on the side stream with its own workspace (W1, W2 and Tp are
+// the left stacks', which are complete by then)
 void right_update(nmc_gen* g, int nb2, int j, const UDT& src, const UDT& dst) {
   const long long LN = (long long)g->Lt * g->N;
   double* X = g->dW1;
@@ -617,14 +633,14 @@ void right_update(nmc_gen* g, int nb2, int j, const UDT& src, const UDT& dst) {
   auto a = gbase(g, nb2, g->dEm, 0, src.U, src.sU, X);
   a.brow = vscale(g->dVv + (long long)l0 * g->N, LN, SC_VEC);
   a.bcol = vscale(src.D, src.sD, SC_VEC);
-  gemm(a, g->stream);
+  gemm(a, g->side);
   for (int l = l0 + 1; l < l0 + g->w; ++l) {
     auto h = gbase(g, nb2, g->dEm, 0, X, g->NN(), X2);
     h.brow = vscale(g->dVv + (long long)l * g->N, LN, SC_VEC);
-    gemm(h, g->stream);
+    gemm(h, g->side);
     std::swap(X, X2);
   }
-  qrp_into(g, nb2, X, dst, src);
+  qrp_into(g, nb2, X, dst, src, g->dWS2, g->side);
 }
 
 // From R (= B_{l-1}...B_0) and L (= B_{L-1}...B_l, transposed): G(l,0) -> dGl,
@@ -704,13 +720,23 @@ nmc_status loss_chunk(nmc_gen* g, int n, const double* targets, double w1, doubl
   if (!want_grad) return NMC_OK;
   gemm(gbase(g, nb2, g->dEph, 0, g->dGbt, NN, g->dT1), st);
   gemm(gbase(g, nb2, g->dT1, NN, g->dEmh, 0, g->dGbar), st);
-  UDT R = identity_udt(g);
+  // The right stacks need nothing of the blocks' work but the fields: R_{j+1} is formed on the side
+  // stream while block j is at work here (a QR of a training batch's 6 matrices occupies 6 SMs for 356
+  // us). ready[j & 1]: R_j is complete; used[j & 1]: the anchor of block j has read it, so R_{j+2} may
+  // take its place.
   UDT Rbuf[2] = {UDT{g->dRU, g->dRD, g->dRT, NN, g->N, NN}, UDT{g->dRU2, g->dRD2, g->dRT2, NN, g->N, NN}};
+  GEN_CUDA(g, cudaEventRecord(g->used[0], st));
+  GEN_CUDA(g, cudaStreamWaitEvent(g->side, g->used[0], 0));   // dVv, and W1 .. Tp are free
   for (int j = 0; j < g->nb; ++j) {
+    if (j + 1 < g->nb) {
+      if (j > 1) GEN_CUDA(g, cudaStreamWaitEvent(g->side, g->used[(j + 1) & 1], 0));
+      right_update(g, nb2, j, j > 0 ? Rbuf[j & 1] : identity_udt(g), Rbuf[(j + 1) & 1]);
+      GEN_CUDA(g, cudaEventRecord(g->ready[(j + 1) & 1], g->side));
+    }
     if (j > 0) {
-      right_update(g, nb2, j - 1, R, Rbuf[j & 1]);
-      R = Rbuf[j & 1];
-      anchor(g, nb2, R, left_slot(g, j), false);
+      GEN_CUDA(g, cudaStreamWaitEvent(st, g->ready[j & 1], 0));
+      anchor(g, nb2, Rbuf[j & 1], left_slot(g, j), false);
+      GEN_CUDA(g, cudaEventRecord(g->used[j & 1], st));
     }
     double* Gl = g->dGl;
     double* Gl2 = g->dGl2;
@@ -721,7 +747,7 @@ nmc_status loss_chunk(nmc_gen* g, int n, const double* targets, double w1, doubl
       auto q = gbase(g, nb2, g->dGbar, NN, Gl, NN, g->dQ);
       q.transB = 1;
       gemm(q, st);
-      k_grad_slice<<<n, kThreads, 0, st>>>(H, g->dQ, g->N, g->lam, grad + (long long)l * g->N, LN);
+      k_grad_slice<<<dim3(n, (g->N + 31) / 32), kThreads, 0, st>>>(H, g->dQ, g->N, g->lam, grad + (long long)l * g->N, LN);
       if (k + 1 < g->w) {
         auto pg = gbase(g, nb2, g->dEm, 0, Gl, NN, Gl2);
         pg.brow = vscale(g->dVv + (long long)l * g->N, LN, SC_VEC);
@@ -849,6 +875,11 @@ nmc_status nmc_gen_create(int lattice, int Lx, int Ly, double t, double U, doubl
   };
   if (cudaGetDevice(&g->device) != cudaSuccess) { cudaGetLastError(); return bail(NMC_ECUDA); }
 
+  bool made = cudaStreamCreateWithFlags(&g->side, cudaStreamNonBlocking) == cudaSuccess;
+  for (cudaEvent_t* e : {&g->ready[0], &g->ready[1], &g->used[0], &g->used[1]})
+    made = made && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+  if (!made) { cudaGetLastError(); return bail(NMC_ECUDA); }
+
   // host set-up: K and the four exponentials
   std::vector<double> K, Kc, wv, V, Em, Ep, Emh, Eph;
   nmc_host::hopping(lattice, Lx, Ly, t, K);
@@ -880,6 +911,7 @@ nmc_status nmc_gen_create(int lattice, int Lx, int Ly, double t, double U, doubl
                      &g->dQ})
     A_(*p, M2 * NN);
   A_(g->dWS, 2 * M2 * NN);
+  A_(g->dWS2, 2 * M2 * NN);
   A_(g->dAcc, 8LL * g->Bc); A_(g->dSign, g->Bc); A_(g->dTarg, 2LL * g->Bf);
   A_(g->dLoss, g->Bf); A_(g->dGx, (long long)g->Bc * LN);
   A_(g->dBad, 1);
@@ -1132,6 +1164,12 @@ const char* nmc_gen_last_error(const nmc_gen* g) { return g ? g->err.c_str() : "
 void nmc_gen_destroy(nmc_gen* g) {
   if (!g) return;
   if (g->stream) cudaStreamSynchronize(g->stream);
+  if (g->side) {
+    cudaStreamSynchronize(g->side);
+    cudaStreamDestroy(g->side);
+  }
+  for (cudaEvent_t e : {g->ready[0], g->ready[1], g->used[0], g->used[1]})
+    if (e) cudaEventDestroy(e);
   for (void* p : g->allocs) cudaFree(p);
   cudaGetLastError();
   delete g;
