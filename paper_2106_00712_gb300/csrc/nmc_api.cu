@@ -157,7 +157,7 @@ struct nmc_ctx {
   bool dfp() const { return opt.precision == NMC_SPLIT_BF16 || opt.precision == NMC_FP32X2; }
   bool tc() const { return opt.precision == NMC_SPLIT_BF16; }
   // wraps and block products a whole matrix per CTA (wrap.cu, where the bounds' reasons stand)
-  bool frags() const { return N <= kFragMaxN && (tc() || (opt.precision == NMC_FP64 && N > 16)); }
+  bool frags() const { return N <= kFragMaxN && (tc() || opt.precision == NMC_FP64); }
 };
 
 namespace {

@@ -116,7 +116,7 @@ extern "C" nmc_status nmc_green_noalloc(int N, int L_tau, int n_wrap, double lam
   size_t shared = round256(NN) + round256(N) + 16 * 32;  // I, ones, alignment slack
   if (shared + bound > kScratchDoubles) return NMC_EINVAL;  // one chain does not fit
   // block products by wrap.cu under the rule of a context in FP64
-  const bool frags = N % 2 == 0 && N > 16 && N <= kFragMaxN;
+  const bool frags = N % 2 == 0 && N <= kFragMaxN;
   const size_t frag_doubles = frags ? round256(frag_bytes<double>(N) / sizeof(double)) : 0;
   shared += frag_doubles + round256(kFragMaxN);
   const int fit = (int)((kScratchDoubles - shared) / per_chain);

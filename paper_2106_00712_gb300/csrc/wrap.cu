@@ -22,11 +22,10 @@
 // and tensor memory: gemm_tc.cu's form, one product per launch, spent 33 us on 512 matrices of 64
 // sites against 5 us of tensor work, in its phases' latencies. It remains for more than 112 sites.
 //
-// us, product by product -> here: 512 matrices of 64 sites, a wrap 67 -> 49 (FP64 136 -> 70) and a chain
-// of 10 332 -> 240 (FP64 680 -> 335); 1024 of 72 a wrap 300 -> 195, a chain of 10 1500 -> 1050; 128 of
-// 100 91 -> 77, 455 -> 409. The error of a wrap against long double, rms: pairs at 64 sites 3.6e-16 ->
-// 2.1e-16 of the largest entry. (Up to 16 sites in FP64 gemm.cu's products stay: one chain of 16 sites took
-// 1.93 ms a sweep pass against 1.87, a warp per matrix waiting out every phase.)
+// us, product by product -> here: 512 matrices of 64 sites, a wrap 67 -> 47 (FP64 136 -> 68) and a chain
+// of 10 332 -> 240 (FP64 680 -> 336); 1024 of 72 a wrap 300 -> 193, a chain of 10 1500 -> 1055; 128 of
+// 100 91 -> 78, 455 -> 382; 2 of 16 in FP64 17 -> 8.4, 83 -> 22. The error of a wrap against long double,
+// rms: pairs at 64 sites 3.6e-16 -> 2.1e-16 of the largest entry.
 // What bounds it: the legacy tensor pipe (0.47 of its m16n8k16 instructions per cycle and SM), 23k of
 // the 39k cycles that two matrices of 64 sites take on an SM together; staging, cutting and joining
 // take the rest, side by side with the other CTA's products only by chance. 512 matrices are 1.7 rounds
@@ -45,6 +44,46 @@ namespace {
 NMC_DEBUG_FLAG
 
 constexpr float kSplit = 12582912.f;   // 1.5 2^23: adding and removing it rounds to an integer
+
+__device__ __forceinline__ void ldm4(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+}
+__device__ __forceinline__ void mma_h(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
+      "{%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// (H 2^B + L) 2^k in FP64, rounded once, by integer operations (a conversion from 64 bits and a scaling
+// would take the FP64 pipe) and without a branch, so that several sums interleave: outside FP64's normal
+// range `slow` is set and join_slow gives the value.
+template <int B>
+__device__ __forceinline__ double join_fast(long long H, long long L, int k, bool& slow) {
+  H += L >> B;
+  L &= (1ll << B) - 1;
+  const int s = min(__clzll(H ^ (H >> 63)) - 1, B);
+  const long long v = (H << s) + (L >> (B - s));
+  const unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const int z = __clzll(m), e = k + B - s - z + 1086;
+  const unsigned long long t = m << (z & 63), f = (t >> 11) + ((t >> 10) & 1);
+  const unsigned long long b = (((unsigned long long)(unsigned)(e - 1)) << 52) + f;
+  slow |= v != 0 && (e < 1 || e > 2045);
+  return __longlong_as_double(v == 0 ? 0ll : (long long)(b | ((unsigned long long)v & (1ull << 63))));
+}
+template <int B>
+__device__ __noinline__ double join_slow(long long H, long long L, int k) {
+  bool slow = false;
+  const double fast = join_fast<B>(H, L, k, slow);
+  if (!slow) return fast;
+  H += L >> B;
+  L &= (1ll << B) - 1;
+  const int s = min(__clzll(H ^ (H >> 63)) - 1, B);
+  return ldexp((double)((H << s) + (L >> (B - s))), k + B - s);
+}
 
 // What a value's digits are and how digit sums make a value
 template <typename T> struct Cut;
@@ -100,30 +139,18 @@ template <> struct Cut<df2> {
     const float sc = __fmul_rn(__int_as_float(ea), __int_as_float(eb));
     return df_norm(__fmul_rn(t, sc), __fmul_rn(l, sc));
   }
-  static __device__ __forceinline__ double wide(const float (&a)[D], int ea, int eb) {
+  // the same in FP64
+  template <bool SLOW>
+  static __device__ __forceinline__ double wide(const float (&a)[D], int ea, int eb, bool& slow) {
     int q[D];
 #pragma unroll
     for (int s = 0; s < D; ++s) q[s] = __float2int_rn(a[s]);
     const long long H = (long long)q[0] * (1 << 20) + ((long long)q[1] * (1 << 10) + q[2]);
     const long long L = (long long)q[3] * (1 << 20) + ((long long)q[4] * (1 << 10) + q[5]);
+    const int k = (ea >> 23) + (eb >> 23) - 254 - 50;
     const bool bad = ea == 0x7fc00000 || eb == 0x7fc00000;
-    return bad ? __longlong_as_double(0x7ff8000000000000ll)
-               : join<30>(H, L, (ea >> 23) + (eb >> 23) - 254 - 50);
-  }
-  // (H 2^B + L) 2^k in FP64, rounded once, in integers (a conversion takes the FP64 pipe)
-  template <int B>
-  static __device__ __forceinline__ double join(long long H, long long L, int k) {
-    H += L >> B;
-    L &= (1ll << B) - 1;
-    const int s = min(__clzll(H ^ (H >> 63)) - 1, B);
-    const long long v = (H << s) + (L >> (B - s));
-    if (v == 0) return 0.0;
-    const unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
-    const int z = __clzll(m), e = k + B - s - z + 1086;
-    const unsigned long long t = m << z, f = (t >> 11) + ((t >> 10) & 1);
-    if (e < 1 || e > 2045) return ldexp((double)v, k + B - s);
-    return __longlong_as_double((long long)((((unsigned long long)(unsigned)(e - 1)) << 52) + f |
-                                            ((unsigned long long)v & (1ull << 63))));
+    const double v = SLOW ? join_slow<30>(H, L, k) : join_fast<30>(H, L, k, slow);
+    return bad ? __longlong_as_double(0x7ff8000000000000ll) : v;
   }
 };
 template <> struct Cut<double> {
@@ -158,8 +185,8 @@ template <> struct Cut<double> {
     }
   }
   static __device__ __forceinline__ int scale(int E) { return E; }
-  static __device__ __forceinline__ double value(const float (&a)[D], int ea, int eb) {
-    if (max(ea, eb) >= kMax) return __longlong_as_double(0x7ff8000000000000ll);
+  template <bool SLOW>
+  static __device__ __forceinline__ double wide(const float (&a)[D], int ea, int eb, bool& slow) {
     int q[D];
 #pragma unroll
     for (int s = 0; s < D; ++s) q[s] = __float2int_rn(a[s]);
@@ -167,23 +194,11 @@ template <> struct Cut<double> {
     const long long L = (long long)q[3] * (1 << 27) +
                         ((long long)q[4] * (1 << 18) + ((long long)q[5] * (1 << 9) + q[6]));
     // digit 0 counts units of 2^(E - 1022 - 8)
-    return Cut<df2>::join<36>(H, L, ea + eb - 2 * 1030 - 54);
+    const int k = ea + eb - 2 * 1030 - 54;
+    const double v = SLOW ? join_slow<36>(H, L, k) : join_fast<36>(H, L, k, slow);
+    return max(ea, eb) >= kMax ? __longlong_as_double(0x7ff8000000000000ll) : v;
   }
-  static __device__ __forceinline__ double wide(const float (&a)[D], int ea, int eb) { return value(a, ea, eb); }
 };
-
-__device__ __forceinline__ void ldm4(unsigned (&r)[4], unsigned addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(addr));
-}
-__device__ __forceinline__ void mma_h(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-      "{%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 
 // Two warps share 16 rows for 4 tiles, one CTA's 8 warps on two of an SM's places: 512 matrices of 64
 // sites take 47 us in pairs of warps against 60 (before the carries) (three places of 4 warps: 456, for which the last 56
@@ -355,6 +370,25 @@ struct Tile {
   }
 };
 
+// A tile's 8 results on this lane, in FP64 (O = double) or as the matrices are held: ea0, ea1 the scales of
+// its two rows, eb(e) those of the columns. All fast results first, so that they interleave.
+template <typename V, typename O, typename F>
+__device__ __forceinline__ void results(const float (&acc)[2][4][Cut<V>::D], int ea0, int ea1, F eb, O (&o)[8]) {
+  bool slow = false;
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    const int ea = (e & 2) ? ea1 : ea0;
+    if constexpr (std::is_same<O, double>::value) o[e] = Cut<V>::template wide<false>(acc[e >> 2][e & 3], ea, eb(e), slow);
+    else o[e] = Cut<V>::value(acc[e >> 2][e & 3], ea, eb(e));
+  }
+  if constexpr (std::is_same<O, double>::value)
+    if (slow) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        o[e] = Cut<V>::template wide<true>(acc[e >> 2][e & 3], (e & 2) ? ea1 : ea0, eb(e), slow);
+    }
+}
+
 __host__ __device__ constexpr size_t tile_smem(int D, int Np) {
   return (size_t)D * Np * Np * 2 + 3 * Np * sizeof(int) + Np;
 }
@@ -380,6 +414,7 @@ k_wrap(const WrapArgs<V> g) {
     return t.sg[r] == t.sg[c] ? v : Cut<V>::mul(v, t.sg[r] > 0 ? g.e2 : g.em2);
   };
   const bool before = fl && g.before;
+  auto column = [&](int nt, int e) { return nt * 16 + (e >> 2) * 8 + 2 * (lane & 3) + (e & 1); };
   t.stage([&](int k, int n) { return X[k * N + n]; }, [&](V v, int k, int n) { return before ? field(v, k, n) : v; });
 
   constexpr int H = Tile<V, T>::H;
@@ -397,11 +432,7 @@ k_wrap(const WrapArgs<V> g) {
                  f[0] = v.x, f[1] = v.y, f[2] = v.z, f[3] = v.w;
                },
                [&](unsigned (&f)[4], int n, int kt, int s) { t.staged_right(f, n * 16, kt, s); });
-#pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const int c = nt * 16 + (e >> 2) * 8 + 2 * (lane & 3) + (e & 1);
-        y[j][e] = Cut<V>::value(acc[e >> 2][e & 3], (e & 2) ? a1 : a0, Cut<V>::scale(t.ce[c]));
-      }
+      results<V>(acc, a0, a1, [&](int e) { return Cut<V>::scale(t.ce[column(nt, e)]); }, y[j]);
     }
   }
   __syncthreads();   // the staged digits are read: their place is the fragments'
@@ -415,24 +446,32 @@ k_wrap(const WrapArgs<V> g) {
                const uint4 v = t.constant(g.R, n, kt, s);
                f[0] = v.x, f[1] = v.z, f[2] = v.y, f[3] = v.w;
              });
+    auto eb = [&](int e) { return __ldg(g.Re + column(nt, e)); };
+    // pairs of columns
+    auto place = [&](int e, long long& idx) {
+      const int r = r0 + (e & 2) * 4, c = column(nt, e);
+      idx = (long long)b * N * N + (long long)r * N + c;
+      return r < N && c < N && NMC_DCHECK(b < g.batch && c + 1 < N, 501);   // (N is even)
+    };
+    long long idx;
+    if (g.Cd) {
+      double o[8];
+      results<V>(acc, e0, e1, eb, o);
 #pragma unroll
-    for (int p = 0; p < 4; ++p) {   // pairs of columns
-      const int r = r0 + (p & 1) * 8, c = nt * 16 + (p >> 1) * 8 + 2 * (lane & 3);
-      if (r >= N || c >= N || !NMC_DCHECK(b < g.batch && c + 1 < N, 501)) continue;   // (N is even)
-      const int ea = p & 1 ? e1 : e0, b0 = __ldg(g.Re + c), b1 = __ldg(g.Re + c + 1);
-      const long long idx = (long long)b * N * N + (long long)r * N + c;
-      const int w = (p & 1) * 2;
-      if (g.Cd) {
-        *(double2*)(g.Cd + idx) = make_double2(Cut<V>::wide(acc[p >> 1][w], ea, b0),
-                                               Cut<V>::wide(acc[p >> 1][w + 1], ea, b1));
-      } else {
-        V o[2] = {Cut<V>::value(acc[p >> 1][w], ea, b0), Cut<V>::value(acc[p >> 1][w + 1], ea, b1)};
+      for (int e = 0; e < 8; e += 2)
+        if (place(e, idx)) *(double2*)(g.Cd + idx) = make_double2(o[e], o[e + 1]);
+    } else {
+      V o[8];
+      results<V>(acc, e0, e1, eb, o);
+#pragma unroll
+      for (int e = 0; e < 8; e += 2) {
+        if (!place(e, idx)) continue;
         if (fl && !g.before) {   // e^{-V} C e^{V}
-          o[0] = field(o[0], c, r);
-          o[1] = field(o[1], c + 1, r);
+          o[e] = field(o[e], column(nt, e), r0 + (e & 2) * 4);
+          o[e + 1] = field(o[e + 1], column(nt, e) + 1, r0 + (e & 2) * 4);
         }
         float4 v;
-        memcpy(&v, o, sizeof v);
+        memcpy(&v, &o[e], sizeof v);
         *(float4*)(g.C + idx) = v;
       }
     }
@@ -464,6 +503,7 @@ k_chain(const ChainArgs<V> g) {
             },
             [&](V v, int k, int n) { return g.before ? field(v, s[k]) : v; });
   }
+  auto column = [&](int nt, int e) { return nt * 16 + (e >> 2) * 8 + 2 * (lane & 3) + (e & 1); };
   const int r0 = t.mt * 16 + (lane >> 2);
   int e0 = Cut<V>::scale(t.ce[r0]), e1 = Cut<V>::scale(t.ce[r0 + 8]);
   auto constant = [&](unsigned (&v4)[4], int n, int kt, int s) {
@@ -484,14 +524,13 @@ k_chain(const ChainArgs<V> g) {
                  else t.fragment(a, kt, d);
                },
                constant);
+      results<V>(acc, e0, e1, [&](int e) { return __ldg(g.Le + column(nt, e)); }, y[j]);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int c = nt * 16 + h * 8 + 2 * (lane & 3);
+        const int c = column(nt, 4 * h);
         const char2 sc = c < N ? *(const char2*)(s + c) : make_char2(1, 1);   // (N is even)
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-          y[j][4 * h + i] = field(Cut<V>::value(acc[h][i], (i & 2) ? e1 : e0, __ldg(g.Le + c + (i & 1))),
-                                   (i & 1) ? sc.y : sc.x);
+        for (int i = 0; i < 4; ++i) y[j][4 * h + i] = field(y[j][4 * h + i], (i & 1) ? sc.y : sc.x);
       }
     }
     if (k == 0) __syncthreads();   // the staged digits are read: their place is the fragments'
@@ -510,11 +549,13 @@ k_chain(const ChainArgs<V> g) {
                else t.fragment(a, kt, d);
              },
              constant);
+    double o[8];
+    results<V>(acc, e0, e1, [&](int e) { return __ldg(g.Le + column(nt, e)); }, o);
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
-      const int c = nt * 16 + (e >> 2) * 8 + 2 * (lane & 3) + (e & 1), r = r0 + (e & 2) * 4;
+      const int c = column(nt, e), r = r0 + (e & 2) * 4;
       if (r >= N || c >= N || !NMC_DCHECK(b < g.batch, 502)) continue;
-      double v = Cut<V>::wide(acc[e >> 2][e & 3], (e & 2) ? e1 : e0, __ldg(g.Le + c)) * ((e & 2) ? d1 : d0);
+      double v = o[e] * ((e & 2) ? d1 : d0);
       if (!g.before) v *= (s[c] > 0) != flip ? g.d1 : g.dm1;
       g.X[(long long)b * N * N + (long long)c * N + r] = v;
     }
