@@ -599,7 +599,7 @@ __global__ void __launch_bounds__(kThreadsDf, 2) k_flip_df(const FlipArgs<df2> f
 // Without tensor cores (FP32X2) the vectors go through shared memory to the FP32-pair loop.
 //
 // One slice, us, 44% of the flips accepted, one flip at a time (k_flip, k_flip_df) -> here:
-//   64 sites x 256 chains, both spins: FP32 pairs 133 -> 75, FP64 357 -> 147, FP32X2 133 -> 110
+//   64 sites x 256 chains, both spins: FP32 pairs 133 -> 75, FP64 357 -> 139, FP32X2 133 -> 110
 //   72 x 1024, one spin: 625 -> 242;  256 x 32: 2950 -> 391;  100 x 64: 481 -> 118;
 //   16 x 1 in FP64: 31 -> 16.
 // What bounds it at 64 x 256 (two CTAs per SM): latency. Of a slice's 146k cycles the decisions take
@@ -637,7 +637,14 @@ template <> struct Arith<double> {
   static __device__ __forceinline__ double add(double a, double b) { return a + b; }
   static __device__ __forceinline__ void fma_acc(double& c, double a, double b) { c = fma(a, b, c); }
   static __device__ __forceinline__ double finish(double a) { return a; }
-  static __device__ __forceinline__ double div(double a, double b) { return a / b; }
+  // a / b to an ulp or two: the division's dozen FP64 operations take 80 cycles each from a warp alone
+  // (a slice of 64 sites x 256 chains 147 us with it, 139 so)
+  static __device__ __forceinline__ double div(double a, double b) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
+    const double e = fma(-b, r, 1.0);   // 2^-20: 1 / b = r (1 + e + e^2 + O(2^-60))
+    return a * fma(r, fma(e, e, e), r);
+  }
 };
 
 // a load that does not look into the SM's own cache
