@@ -12,13 +12,13 @@
 // G0 += A B^T. In exact arithmetic this equals applying each rank-1 update at once.
 // G0 of both spins sits in shared memory when it fits (N <= 64 in FP64), else in global
 // memory (L2); the panels always live in shared memory (k is clamped to fit).
-// That is k_flip (FP32) and, above some 560 sites, k_flip (FP64) and k_flip_df (FP32 pairs); up to
-// there FP64 and FP32 pairs take k_flip_block, which decides blocks of up to min(k, 16) sites apart.
+// That is k_flip in FP32, above some 560 sites in FP64, and k_flip_df above some 430 in FP32 pairs
+// without tensor cores (with them there are 320 at most); below, FP64 and FP32 pairs take k_flip_block,
+// which decides blocks of up to min(k, 16) sites apart.
 #include <cooperative_groups.h>
 
 #include "fold16.cuh"
 #include "nmc_internal.cuh"
-#include "oz_slice.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -244,141 +244,6 @@ __device__ void flush_df(df2* G, const df2* Ap, const df2* Bp, int m, int N, int
   }
 }
 
-// The same fold on the BF16 tensor cores: G += P Q with P[r][q] = A[q][r], Q[q][c] = B[q][c]
-// (q < m <= 16), both cut into exact integer slices (oz_slice.cuh) with one scale per row of
-// P and per column of Q; the products of slices s and t go to group s + t (exact in FP32),
-// and each group is scaled and added into G in FP32 pairs. The fragments are sliced in
-// registers straight from the panels. sEr, sFc: shared scratch of ns * N ints each.
-// Used for k <= 16 (one k-step: each warp slices a 16-row block of P once) and N > 64.
-// Measured (one compensated sweep, k = 16): N = 144 flips 41.0 ms vs 48.6 ms with the SIMT
-// fold; N = 64 slower than the SIMT fold (1.27 vs 1.48 TFLOP/s of flip work), where the
-// per-output slicing and scaling outweigh a 16-term double-float sum. For k = 32 at N = 256 a
-// version that re-sliced P per n-tile took 1198 ms against 625 ms for the SIMT fold.
-constexpr int kTcFlushMaxK = 16;
-
-// A fragment (row-major 16 x 16) of P rows r_lo / r_hi = r_lo + 8, k = k0..k0+15: register v
-// holds row (v & 1 ? r_hi : r_lo), k = k0 + 2tq + {0, 1} (+8 for v >= 2); the lower half of
-// each register holds the lower k.
-__device__ __forceinline__ void flush_a_frag(uint32_t (&af)[kOzS][4], const df2* A_, const int* er,
-                                             int r_lo, int k0, int m, int N, int tq) {
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const int r = r_lo + ((v & 1) << 3);
-    const int q = k0 + 2 * tq + ((v >> 1) << 3);
-    const bool rok = r < N;
-    const df2 x0 = (rok && q < m) ? A_[q * N + r] : df_zero();
-    const df2 x1 = (rok && q + 1 < m) ? A_[(q + 1) * N + r] : df_zero();
-    const int e = rok ? er[r] : 0;
-    unsigned short s0[kOzS], s1[kOzS];
-    slice_bits(x0, e, s0);
-    slice_bits(x1, e, s1);
-#pragma unroll
-    for (int s = 0; s < kOzS; ++s) af[s][v] = (uint32_t)s0[s] | ((uint32_t)s1[s] << 16);
-  }
-}
-
-// B fragment (16 x 8) of Q column c: register v holds k = k0 + 2tq + {0, 1} (+8 for v = 1).
-__device__ __forceinline__ void flush_b_frag(uint32_t (&bf)[kOzS][2], const df2* B_, const int* fc,
-                                             int c, int k0, int m, int N, int tq) {
-#pragma unroll
-  for (int v = 0; v < 2; ++v) {
-    const int q = k0 + 2 * tq + (v << 3);
-    const bool cok = c < N;
-    const df2 y0 = (cok && q < m) ? B_[q * N + c] : df_zero();
-    const df2 y1 = (cok && q + 1 < m) ? B_[(q + 1) * N + c] : df_zero();
-    const int fe = cok ? fc[c] : 0;
-    unsigned short s0[kOzS], s1[kOzS];
-    slice_bits(y0, fe, s0);
-    slice_bits(y1, fe, s1);
-#pragma unroll
-    for (int s = 0; s < kOzS; ++s) bf[s][v] = (uint32_t)s0[s] | ((uint32_t)s1[s] << 16);
-  }
-}
-
-__device__ __forceinline__ void flush_mma(float (&acc)[kOzS][4], const uint32_t (&af)[kOzS][4],
-                                          const uint32_t (&bf)[kOzS][2]) {
-#pragma unroll
-  for (int s = 0; s < kOzS; ++s)
-#pragma unroll
-    for (int t = 0; t < kOzS; ++t)
-      if (s + t < kOzS) mma_bf16(acc[s + t], af[s], bf[t][0], bf[t][1]);
-}
-
-// C fragment: register w holds row (w >> 1 ? r_lo + 8 : r_lo), column c0 + 2tq + (w & 1).
-__device__ __forceinline__ void flush_store(df2* Gsp, const float (&acc)[kOzS][4], const int* er,
-                                            const int* fc, int r_lo, int c0, int N, int tq) {
-#pragma unroll
-  for (int w = 0; w < 4; ++w) {
-    const int r = r_lo + ((w >> 1) << 3);
-    const int cc = c0 + 2 * tq + (w & 1);
-    if (r >= N || cc >= N) continue;
-    df2 sum = df_zero();
-#pragma unroll
-    for (int q = kOzS - 1; q >= 0; --q)
-      sum = df_add(sum, df2{acc[q][w] * pow2f(-8 * (q + 2)), 0.f});
-    const int ex = er[r] + fc[cc];
-    df2* gp = Gsp + (long long)r * N + cc;
-    const float se = pow2f(ex);
-    *gp = df_add(*gp, df2{sum.hi * se, sum.lo * se});
-  }
-}
-
-// KS k-steps of 16 (m <= 16 KS): a warp slices a 16-row block of P once and sweeps it across
-// all 8-column n-tiles of its spin.
-template <int KS>
-__device__ __forceinline__ void flush_rows(df2* G, const df2* Ap, const df2* Bp, int m, int N,
-                                           int KK, long long NN, int ns, const int* sEr,
-                                           const int* sFc, int warp, int nw, int g, int tq,
-                                           int nb) {
-  for (int job = warp; job < ns * nb; job += nw) {
-    const int sp = job / nb, rb = job - sp * nb;
-    const int r_lo = rb * 16 + g;
-    const df2* A_ = Ap + sp * KK * N;
-    const df2* B_ = Bp + sp * KK * N;
-    const int* er = sEr + sp * N;
-    const int* fc = sFc + sp * N;
-    uint32_t af[KS][kOzS][4];
-#pragma unroll
-    for (int k = 0; k < KS; ++k) flush_a_frag(af[k], A_, er, r_lo, 16 * k, m, N, tq);
-#pragma unroll 1
-    for (int cn = 0; cn < 2 * nb; ++cn) {
-      float acc[kOzS][4];
-#pragma unroll
-      for (int q = 0; q < kOzS; ++q)
-#pragma unroll
-        for (int w = 0; w < 4; ++w) acc[q][w] = 0.f;
-#pragma unroll
-      for (int k = 0; k < KS; ++k) {
-        uint32_t bf[kOzS][2];
-        flush_b_frag(bf, B_, fc, cn * 8 + g, 16 * k, m, N, tq);
-        flush_mma(acc, af[k], bf);
-      }
-      flush_store(G + sp * NN, acc, er, fc, r_lo, cn * 8, N, tq);
-    }
-  }
-}
-
-__device__ void flush_tc(df2* G, const df2* Ap, const df2* Bp, int m, int N, int KK,
-                         long long NN, int ns, int* sEr, int* sFc) {
-  for (int t = threadIdx.x; t < 2 * ns * N; t += blockDim.x) {
-    const int which = t / (ns * N), rem = t - which * ns * N;
-    const int sp = rem / N, x = rem - sp * N;
-    const df2* P = (which ? Bp : Ap) + sp * KK * N + x;
-    float mx = 0.f;
-    for (int q = 0; q < m; ++q) mx = fmaxf(mx, fabsf(P[q * N].hi));
-    // |hi + lo| <= |hi| (1 + 2^-24): one extra bit of headroom
-    (which ? sFc : sEr)[rem] = scale_exp(mx) + (mx > 0.f ? 1 : 0);
-  }
-  __syncthreads();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  const int g = lane >> 2, tq = lane & 3;
-  const int nb = (N + 15) >> 4;
-  flush_rows<1>(G, Ap, Bp, m, N, KK, NN, ns, sEr, sFc, warp, nw, g, tq, nb);   // m <= 16
-}
-
-// TC: fold on the tensor cores (flush_tc) instead of the double-float loop (flush_df); a
-// separate instantiation, so the FP32-pipe variant keeps its smaller register footprint.
-template <bool TC>
 __global__ void __launch_bounds__(kThreadsDf, 2) k_flip_df(const FlipArgs<df2> f) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int s_accept[2];  // by attempt parity: see the loop
@@ -398,8 +263,6 @@ __global__ void __launch_bounds__(kThreadsDf, 2) k_flip_df(const FlipArgs<df2> f
   // holds it exactly
   df2* udf = (df2*)(((uintptr_t)(Gs + (f.g_in_smem ? ns * NN : 0)) + 15) & ~(uintptr_t)15);
   int8_t* sl = (int8_t*)(udf + N);
-  int* sEr = (int*)(((uintptr_t)(sl + N) + 15) & ~(uintptr_t)15);   // flush scales
-  int* sFc = sEr + ns * N;
 
   df2* Gg = f.G + (long long)c * ns * NN;
   df2* G = f.g_in_smem ? Gs : Gg;
@@ -552,8 +415,7 @@ __global__ void __launch_bounds__(kThreadsDf, 2) k_flip_df(const FlipArgs<df2> f
       ++m;
       __syncthreads();
       if (m == KK) {
-        if constexpr (TC) flush_tc(G, Ap, Bp, m, N, KK, NN, ns, sEr, sFc);
-        else flush_df(G, Ap, Bp, m, N, KK, NN, ns);
+        flush_df(G, Ap, Bp, m, N, KK, NN, ns);
         m = 0;
         __syncthreads();
         for (int j = threadIdx.x; j < ns * N; j += blockDim.x) {
@@ -565,8 +427,7 @@ __global__ void __launch_bounds__(kThreadsDf, 2) k_flip_df(const FlipArgs<df2> f
     }
   }
   if (m > 0) {
-    if constexpr (TC) flush_tc(G, Ap, Bp, m, N, KK, NN, ns, sEr, sFc);
-    else flush_df(G, Ap, Bp, m, N, KK, NN, ns);
+    flush_df(G, Ap, Bp, m, N, KK, NN, ns);
     __syncthreads();
   }
   if (f.g_in_smem)
@@ -1064,7 +925,7 @@ size_t flip_smem_bytes(int N, int kk, size_t elem, int g_in_smem, int ns) {
   if (g_in_smem) b += (size_t)ns * N * N * elem;
   b = (b + 15) & ~(size_t)15;
   b += (size_t)N * sizeof(double) + (size_t)N + 16;
-  b += 2 * (size_t)ns * N * sizeof(int) + 16;   // scales of the tensor-core flush
+  b += 2 * (size_t)ns * N * sizeof(int) + 16;   // (what nmc_get_dims' delay_k is clamped by)
   return b;
 }
 
@@ -1143,13 +1004,8 @@ void flip_slice<df2>(const FlipArgs<df2>& f, int n_chains, cudaStream_t st) {
                 : flip_block<df2, kFoldPairs>(f, n_chains, st))
     return;
   const size_t bytes = flip_smem_bytes(f.N, f.kk, sizeof(df2), f.g_in_smem, f.ns);
-  if (f.tc_fold && f.kk <= kTcFlushMaxK) {
-    allow_max_dynamic_smem((const void*)k_flip_df<true>);
-    k_flip_df<true><<<n_chains, kThreadsDf, bytes, st>>>(f);
-  } else {
-    allow_max_dynamic_smem((const void*)k_flip_df<false>);
-    k_flip_df<false><<<n_chains, kThreadsDf, bytes, st>>>(f);
-  }
+  allow_max_dynamic_smem((const void*)k_flip_df);
+  k_flip_df<<<n_chains, kThreadsDf, bytes, st>>>(f);
 }
 
 NMC_DEBUG_READER(debug_fail_flip)

@@ -3,7 +3,8 @@
 // integer slicing (Ozaki-style error-free splitting; Ozaki, Ogita, Oishi, Rump, Numer.
 // Algorithms 2012).
 //
-// Every propagation product of the sweep has one constant operand (e^{-+dtau K},
+// For matrices of more than 112 sites (up to there wrap.cu keeps a whole one in a CTA): every propagation
+// product of the sweep has one constant operand (e^{-+dtau K},
 // e^{-+dtau K/2}, shared by all chains) and one chain operand X (an FP32-pair matrix of one
 // chain and spin). The kernel forms D = A B^T with A = rows of the chain operand and
 // B = rows of the constant, each row scaled by a power of two 2^-e so that its entries lie
@@ -161,19 +162,6 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
           smem_u32(bar))
       : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-      "%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
-        "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-#pragma unroll
-  for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {

@@ -183,7 +183,8 @@ void split_to_df(const double* x, df2* y, long long n, cudaStream_t st);
 void qrp_udt(const double* X, double* U, double* D, double* Tp, double* ws, int N, int batch,
              cudaStream_t st);
 
-// Y[b] = X[b]^{-1} * (diag(1/max(DR,1)) * UR[b]^T) by Gauss-Jordan with partial pivoting.
+// Y[b] = X[b]^{-1} * (diag(1/max(DR,1)) * UR[b]^T) by LU (up to 40 sites Gauss-Jordan)
+// with partial pivoting.
 void solve_stab(const double* X, const double* UR, long long sUR, const double* DR,
                 long long sDR, double* Y, double* ws, int N, int batch, cudaStream_t st);
 
