@@ -8,7 +8,7 @@ every chain (N * L_tau flip attempts per chain, with the wraps, UDV stabilizatio
 measurements the sweep contains). Metric: flip attempts per second, whole job.
 
 Paths timed: "fp64" (all propagation in FP64), "split_bf16" (G, flips and delayed updates
-in compensated FP32 pairs, every propagation product on the BF16 tensor cores by exact
+in compensated FP32 pairs, every propagation product on the tensor cores by exact
 integer slicing; QR, recompute, ratios and measurements in FP64), "fp32x2" (the same with
 every product in FP32 pairs on the FP32 pipes) and "fp32" (plain FP32 propagation), plus the
 particle-hole single-spin variants. A path counts for `value` only if its max
@@ -43,10 +43,10 @@ NOMINAL_TFLOPS = {"fp64": 1.259, "fp32": 80.55}
 # Compensated FP32 pairs: one multiply-add costs 12 FP32-pipe instructions (TwoProd by FMA,
 # TwoSum, two cross-term FMAs, two adds); a secondary ceiling for the pair kernels.
 PAIR_INSTR_PER_FMA = 12
-# exact-slicing tensor-core products: 7 BF16 slices per operand, the 28 slice pairs (s, t)
-# with s + t <= 6 issued per FP64-class product
-OZ_PRODUCTS = 28
-TC_KERNEL = "k_gemm_tc (tcgen05.mma kind::f16, TMEM accumulators, TMA-staged constant slices)"
+# exact-slicing tensor-core products of FP32 pairs: 6 FP16 digits per operand, the 21 digit
+# pairs (s, t) with s + t <= 5 issued per FP64-class product
+OZ_PRODUCTS = 21
+TC_KERNEL = "k_wrap, k_chain (mma.sync on exact FP16 digits, a whole matrix per CTA)"
 
 
 def _measured_peaks_file():
@@ -64,15 +64,14 @@ BF16_PEAK, BF16_PEAK_SUSTAINED, HBM_PEAK_GBS = _measured_peaks_file()
 # (dram__bytes_read.sum + dram__bytes_write.sum), keyed by the hash of the kernel source at
 # capture time; reported as null once the source has changed.
 TRAFFIC = {
-    # k_gemm_tc, bench launch configuration (512 products of 64 x 64 in 304 tiles of 108 rows),
-    # ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum: constant on the left 16.93 MB
-    # read, 0 written; on the right 18.22 MB read, 1.35 MB written -- the chain operand
-    # (16.78 MB as FP32 pairs) once plus the constant's slices; weighted by the sweep's launch
-    # mix (84 : 44)
-    "gemm_tc.cu": ("57ee5e38a167fac9", 17.83e6),
-    # k_flip_df<false> (the FP32-pipe fold used at N = 64), same configuration (one slice of
-    # 256 chains x 2 spins): 16.89 MB read (G as FP32 pairs, once), 0 written (stays in L2)
-    "flip.cu": ("a6c5108ea7f07fd0", 16.89e6),
+    # k_wrap and k_chain, bench launch configuration (512 matrices of 64 x 64), ncu --metrics
+    # dram__bytes_read.sum,dram__bytes_write.sum: a wrap reads 16.98 MB (the operand as FP32
+    # pairs, once), a chain 10.5 MB (its FP64 operand is partly in L2), neither writes (the
+    # results stay in L2); weighted by the sweep's launch mix (88 : 8)
+    "wrap.cu": ("39b15370818c6987", 16.44e6),
+    # k_flip_block (FP32 pairs), same configuration (one slice of 256 chains x 2 spins): 16.91 MB
+    # read (G as FP32 pairs, once), 0 written (stays in L2)
+    "flip.cu": ("8f4cc10c59ca6120", 16.91e6),
 }
 
 
@@ -94,11 +93,17 @@ def step_flop(N, L, nb, chains, ns, acc):
     return per_matrix * ns * chains
 
 
-def class_rooflines(st, base, ns, acc, peaks, tc):
+def tc_products_per_launch(L, nb):
+    """Products per launch of the tensor-core class over one sweep: a wrap (L of them) and a
+    measurement's transform (nb) are two products in one launch, a block's chain (nb) L / nb."""
+    return (2.0 * L + 2.0 * nb + L) / (L + 2.0 * nb)
+
+
+def class_rooflines(st, base, ns, acc, peaks, tc, tc_products=1.0):
     """Achieved vs peak for each timed kernel class of the path (algorithmic work per launch
     / average event-timed launch duration). Per launch, every class runs over the batch of
-    ns x chains matrices of N x N: products 2N^3 each (the tensor-core class: its 28 BF16
-    slice products, against the BF16 peak); QR with Q formed 8/3 N^3; Gauss-Jordan on
+    ns x chains matrices of N x N: products 2N^3 each (the tensor-core class: `tc_products`
+    products per launch, each its 21 FP16 digit products, against the BF16 peak); QR with Q formed 8/3 N^3; Gauss-Jordan on
     [X | N right-hand sides] 3N^3; a slice of flips, per accepted flip and spin, a rank-k
     flush share 2N^2 plus the panel column and row 2Nk (k = delay). Each class is quoted
     against the pipe it runs on: `peaks` holds the measured FP64 and FP32 SIMT peaks and the
@@ -116,8 +121,9 @@ def class_rooflines(st, base, ns, acc, peaks, tc):
                 "unit": "TFLOP/s", "frac": a / peak, "peak_source": src, **kw}
     out = {}
     if st.get("gemm_tc", (0,))[0]:
-        a = rate("gemm_tc", OZ_PRODUCTS * 2.0 * N ** 3 * batch)
-        tr = traffic_of("gemm_tc.cu")
+        oz = 28 if base == "fp64" else OZ_PRODUCTS   # (FP64: 7 digits)
+        a = rate("gemm_tc", tc_products * oz * 2.0 * N ** 3 * batch)
+        tr = traffic_of("wrap.cu")
         hbm = {}
         if tr:
             launches, timed, ms = st["gemm_tc"]
@@ -126,9 +132,9 @@ def class_rooflines(st, base, ns, acc, peaks, tc):
         out["gemm_tc"] = entry("tensor", TC_KERNEL, a, peaks["bf16"],
                                "MEASURED_PEAKS.json bf16_tflops (cuBLAS burst), of measured",
                                traffic=tr, **hbm,
-                               algorithmic=f"{OZ_PRODUCTS} BF16 slice products of 2N^3 per "
+                               algorithmic=f"{oz} FP16 digit products of 2N^3 per "
                                            "FP64-class product",
-                               achieved_fp64_class=a / OZ_PRODUCTS)
+                               achieved_fp64_class=a / oz)
     if st.get("gemm_df", (0,))[0]:
         a = rate("gemm_df", 2.0 * N ** 3 * batch)
         out["gemm_df"] = entry("alu", "k_gemm_df<64,64> (compensated FP32 pairs)", a,
@@ -141,16 +147,16 @@ def class_rooflines(st, base, ns, acc, peaks, tc):
                                  "FP32 FMA probe (nmc_fma_probe), of measured",
                                  frac_of_pair_ceiling=a / (peaks["fp32"] / PAIR_INSTR_PER_FMA))
     if st.get("gemm", (0,))[0]:
-        kern = {"fp64": "k_gemm<double,64>", "fp32": "k_gemm<float,64>",
-                "fp32x2": "k_gemm<double,64> (FP64 recompute, T updates)"}[base]
+        kern = {"fp64": "k_gemm_fx (FP64 by exact FP16 digits on mma.sync)", "fp32": "k_gemm<float,64>",
+                "fp32x2": "k_gemm_fx (FP64 recompute, T updates by exact FP16 digits on mma.sync)"}[base]
         pk = "fp32" if base == "fp32" else "fp64"
         a = rate("gemm", 2.0 * N ** 3 * batch)
         out["gemm"] = entry("alu", kern, a, peaks[pk],
                             f"{pk.upper()} FMA probe (nmc_fma_probe), of measured")
     if st.get("flip", (0,))[0]:
         a = rate("flip", acc * N * C * ns * (2.0 * N * N + 2.0 * N * k))
-        kern = {"fp64": "k_flip<double>", "fp32": "k_flip<float>",
-                "fp32x2": "k_flip_df"}[base]
+        kern = {"fp64": "k_flip_block<double>", "fp32": "k_flip<float>",
+                "fp32x2": "k_flip_block<FP32 pairs>"}[base]
         extra = {}
         if base == "fp32x2":
             extra["frac_of_pair_ceiling"] = a / (peaks["fp32"] / PAIR_INSTR_PER_FMA)
@@ -166,10 +172,10 @@ def class_rooflines(st, base, ns, acc, peaks, tc):
                             f"{simt.upper()} FMA probe (nmc_fma_probe), of measured",
                             algorithmic="per accepted flip and spin 2N^2 + 2Nk (delayed rank-k "
                                         "updates); one launch = one slice of every chain; "
-                                        "latency-bound (one sequential site loop per chain)",
+                                        "latency-bound (acceptances of a chain are sequential)",
                             **extra)
-    for cls, kname, flop in (("qrp", "k_qrp (FP64 column-pivoted QR + Q)", 8.0 / 3.0 * N ** 3),
-                             ("solve", "k_solve (FP64 Gauss-Jordan)", 3.0 * N ** 3)):
+    for cls, kname, flop in (("qrp", "k_qrp (column-pivoted QR + Q in 64-bit fixed point)", 8.0 / 3.0 * N ** 3),
+                             ("solve", "k_solve (FP64 blocked LU, updates on mma.sync)", 3.0 * N ** 3)):
         if st.get(cls, (0,))[0]:
             out[cls] = entry("alu", kname, rate(cls, flop * batch), peaks["fp64"],
                              "FP64 FMA probe (nmc_fma_probe), of measured")
@@ -584,7 +590,8 @@ def main():  # noqa: C901
     base = BASE[prec]
     tot_ms = max(sum(x[2] for x in st.values()), 1e-30)
     share = {k: v[2] / tot_ms for k, v in st.items() if v[0]}
-    rl = class_rooflines(st, base, ns, r["obs"].accept, peaks, prec == 2)
+    rl = class_rooflines(st, base, ns, r["obs"].accept, peaks, prec == 2,
+                         tc_products_per_launch(WL.L_tau, WL.L_tau // WL.n_wrap))
     roofline = dict(rl.get(dom) or rl[max(rl, key=lambda k: st[k][2])])
     roofline.update({"dominant_class": dom, "share": share})
     roofline["others"] = {k: {kk: v[kk] for kk in ("kernel", "bound", "achieved", "peak", "frac",

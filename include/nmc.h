@@ -58,10 +58,10 @@ typedef enum {
   NMC_FP32 = 1,       /* flips, delayed updates and wraps in FP32 (FP32 accumulation)     */
   NMC_SPLIT_BF16 = 2, /* compensated: G, flips and delayed-update panels in FP32 pairs
                          (error-free products and sums); every wrap, stack and measurement
-                         product on the BF16 tensor cores by exact integer slicing (each
-                         operand cut into 7 integer BF16 slices, slice products exact in FP32
-                         accumulators, ~2^-49 of the row/column maxima), and the rank-k fold
-                         too where that is faster; QR, recompute, ratios, measurement FP64 */
+                         product and the rank-k folds on the tensor cores by exact integer
+                         slicing (operands cut into 6 FP16 or, above 112 sites, 7 BF16 integer
+                         slices, slice products exact in FP32 accumulators, ~2^-49 of the
+                         row/column maxima); QR, recompute, ratios, measurement FP64       */
   NMC_TF32X3 = 3,     /* not built (NMC_EINVAL): three TF32 products accumulated in FP32 give
                          FP32-class products, which cannot hold the 1e-5 drift bar here   */
   NMC_FP32X2 = 4      /* compensated as NMC_SPLIT_BF16, with every product and fold in FP32
@@ -103,8 +103,10 @@ typedef struct {
                             results, but accumulate in FP32 pairs on the FP32 pipe (error-free
                             products and sums, ~2^-44 of the sum of |a_ik b_kj|) instead of FP64
                             FMAs; operands must lie within the FP32 range, which the stacks'
-                            D-split keeps them in. The QR and the Gauss-Jordan solve stay FP64.
-                            0: FP64 (SIMT FP64 pipe).                            default 0  */
+                            D-split keeps them in. The QR and the solve stay FP64. Only above
+                            256 sites: below, the FP64 products are the faster and the more
+                            accurate ones and are taken either way.
+                            0: FP64.                                             default 0  */
 } nmc_options;
 
 typedef struct {
