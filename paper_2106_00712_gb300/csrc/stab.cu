@@ -5,7 +5,7 @@
 //   column of largest norm (lowest index on ties) is swapped into place, a reflector
 //   H_p = I - tau v v^T zeroes it below the diagonal, and the trailing columns are updated;
 //   squared column norms are downdated and summed again when little of them is left. Outputs
-//   U = Q (formed in place by backward accumulation of the reflectors), D = |diag R| and
+//   U = Q (column by column, in registers), D = |diag R| and
 //   T = D^{-1} R P^T.
 // k_solve: Y = X^{-1} (Db_R^{-1} U_R^T) by blocked LU with partial pivoting; X is the
 //   well-scaled middle factor of the stabilized inverse, so partial pivoting is sufficient.
@@ -47,12 +47,16 @@ constexpr size_t kQrSmemLimit = 225 * 1024;
 // LPC lanes share a column (rows r = LPC j + lane, at most 4 NB each, held in registers between
 // the dot product and the update), so a matrix of 64 columns keeps 256 threads busy; one warp
 // searches the pivot and evaluates the reflector's scalars.
-// What bounds it: one matrix, the serial chain of a step (pivot search, column norm, reflector,
-// about 2500 cycles at N = 64, then 2200 for the update, and 2700 per step of forming Q); many, the
-// issue slots and the barriers around that chain (40% issue). Measured, us per launch against the
-// FP64 kernel with one thread per column (N, matrices): 242 / 582 (64, 6), 361 / 722 (64, 512),
-// 1221 / 1904 (72, 1024), 560 / 1281 (100, 128), 1082 / 2497 (144, 128), 42 / 71 (16, 2) and, with the
-// matrix in global memory, where lanes along the rows read whole lines, 5034 / 87627 (256, 64).
+// What bounds it: one matrix, the serial chain of a step (pivot search, column norm, reflector, then
+// the update, a barrier after each); many, the issue slots and the barriers around that chain.
+// Measured, us per launch against an FP64 kernel with one thread per column (N, matrices): 361 / 722
+// (64, 512), 1221 / 1904 (72, 1024), 560 / 1281 (100, 128), 42 / 71 (16, 2) and, with the matrix in
+// global memory, where lanes along the rows read whole lines, 5034 / 87627 (256, 64). Those formed Q
+// like R, one reflector on all columns and a barrier at a time; Q's columns are now each built in
+// registers, the pivot column is read once, and what is in shared memory is so at compile time. On one
+// set of graded and degenerate matrices, with the same bits: 45 -> 35 (16, 2), 143 -> 115 (36, 128),
+// 291 -> 230 (64, 6), 414 -> 340 (64, 512), 422 -> 369 (72, 6), 1397 -> 1229 (72, 1024), 717 -> 619
+// (100, 128), 1387 -> 1245 (144, 128), 5734 -> 5181 (256, 64), 37.5 -> 30.8 ms (512, 2).
 // max |U^T U - I| 7e-17 against 8e-16, columns of U D T to 1.5e-16 against 9e-16 (N = 64).
 constexpr int kLimb = 29, kFix = 58;
 
@@ -145,11 +149,16 @@ __host__ __device__ constexpr size_t qr_small_bytes(int rows, int N) {
   return (size_t)rows * 2 * 8 + (size_t)N * (2 * 8 + 2 * 4 + 2 * 4);
 }
 
+// The working matrix is in shared memory up to 160 sites (8 lanes), which is all that fits.
+__host__ __device__ constexpr bool qr_smem(int LPC) { return LPC < 16; }
+static_assert(((qr_small_bytes(160, 160) + 15) & ~(size_t)15) + 160 * qr_ld(160, 8) * 8 <= kQrSmemLimit, "");
+
 template <int LPC, int NB, int THREADS, int CTAS>
 __global__ void __launch_bounds__(THREADS, CTAS)
 k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__ D,
-      double* __restrict__ Tp, double* __restrict__ ws, int N, int use_smem) {
+      double* __restrict__ Tp, double* __restrict__ ws, int N) {
   constexpr int kRows = 4 * NB * LPC, ldw = qr_ld(kRows, LPC), ngrp = THREADS / LPC;
+  constexpr int kPer = (kRows + 31) / 32;        // rows per lane when a warp holds a column
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ int2 s_tau;
   __shared__ int s_bad;
@@ -162,9 +171,9 @@ k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__
   float* n2 = n1 + N;                            // [N] the same when last summed
   int* Eb = (int*)(n2 + N);                      // [N] biased exponent of the column's scale
   int* perm = Eb + N;                            // [N]
-  long long* W = use_smem
-      ? (long long*)(smraw + ((qr_small_bytes(kRows, N) + 15) & ~(size_t)15))
-      : (long long*)(ws + (long long)b * 2 * NN);
+  long long* W;
+  if constexpr (qr_smem(LPC)) W = (long long*)(smraw + ((qr_small_bytes(kRows, N) + 15) & ~(size_t)15));
+  else W = (long long*)(ws + (long long)b * 2 * NN);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int sub = tid % LPC, grp = tid / LPC, wgrp = warp * 32 / LPC;   // the warp's first group
   // the serial warp: on another sub-partition in each of the CTAs that share an SM (warp w issues
@@ -225,12 +234,23 @@ k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__
       bi = top == 0 ? p : (int)__reduce_min_sync(0xffffffffu, best == top ? (unsigned)bi : 0xffffu);
       const int piv = NMC_DCHECK(bi >= p && bi < N, 201) ? bi : p;
       long long* col = W + (long long)p * ldw;
+      long long* other = W + (long long)piv * ldw;
+      const long long alpha = other[p];
+      long long y[kPer];   // the pivot column; column p takes its place
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const int r = lane + 32 * i;
+        y[i] = r < N ? other[r] : 0;
+      }
+      __syncwarp();
       if (piv != p) {
-        long long* other = W + (long long)piv * ldw;
-        for (int r = lane; r < N; r += 32) {
-          const long long t0 = col[r];
-          col[r] = other[r];
-          other[r] = t0;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+          const int r = lane + 32 * i;
+          if (r < N) {
+            other[r] = col[r];
+            if (r < p) col[r] = y[i];
+          }
         }
         if (lane == 0) {
           n1[piv] = n1[p];
@@ -238,12 +258,12 @@ k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__
           int t = Eb[p]; Eb[p] = Eb[piv]; Eb[piv] = t;
           t = perm[p]; perm[p] = perm[piv]; perm[piv] = t;
         }
-        __syncwarp();
       }
       // squared norm from the diagonal down, exactly: HI 2^58 + MID 2^30 + LO
       long long hi = 0, mid = 0, lo = 0;
-      for (int r = p + lane; r < N; r += 32) {
-        const int2 c = limbs(col[r]);
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const int2 c = limbs(lane + 32 * i >= p ? y[i] : 0);
         mad_wide(hi, c.x, c.x);
         mad_wide(mid, c.x, c.y);
         mad_wide(lo, c.y, c.y);
@@ -253,7 +273,6 @@ k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__
       hi = warp_sum64(hi);
       mid = warp_sum64(mid);
       lo = warp_sum64(lo);
-      const long long alpha = col[p];
       int k = 0;
       long long head = 0, beta = 0;
       int2 tau = make_int2(0, 0);
@@ -270,11 +289,14 @@ k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__
       }
       __syncwarp();
       // the reflector's limbs, for this step and (below the diagonal) for Q
-      for (int r = p + 1 + lane; r < N; r += 32) {
-        const long long c = col[r];
-        const int2 l = limbs(k >= 0 ? c << k : c >> -k);
-        vp[r] = l;
-        ((int2*)col)[r] = l;
+#pragma unroll
+      for (int i = 0; i < kPer; ++i) {
+        const int r = lane + 32 * i;
+        if (r > p && r < N) {
+          const int2 l = limbs(k >= 0 ? y[i] << k : y[i] >> -k);
+          vp[r] = l;
+          ((int2*)col)[r] = l;
+        }
       }
       if (lane == 0) {
         const int2 hl = limbs(head);
@@ -373,34 +395,41 @@ k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__
     Tb[r * N + perm[c]] = bad ? nan : t;
   }
   __syncthreads();   // T and D are out: W's upper triangle is free
-  // Q = H_0 H_1 ... H_{N-1} in place over W, 1 = 2^58, by backward accumulation: before step p,
-  // columns > p hold H_{p+1} ... H_{N-1} in rows > p (rows <= p still hold R and count as zero: the
-  // reflector buffers are zero there); step p applies H_p to those columns, writing their row p,
-  // and turns column p (the limbs of its reflector) into H_p e_p. The reflector of step p - 1 is
-  // copied out meanwhile.
-  for (int r = tid; r < 2 * kRows; r += THREADS) vl[r] = make_int2(0, 0);
+  // Q = H_0 H_1 ... H_{N-1}, 1 = 2^58: column c is H_0 ... H_c e_c (the later ones leave e_c alone),
+  // so columns need nothing from each other: LPC lanes hold one in registers from e_c on, without a
+  // barrier, the warp's 32 / LPC columns starting together (a reflection that comes too early for a
+  // column multiplies zeros). With one column per group the second four of every eight warps take
+  // their blocks backwards, so that each quarter of the SM (warp w on w % 4) gets long and short
+  // ones; with several, rounds alternate. Against applying each reflector to all columns, a barrier
+  // apiece: see the figures above.
+  for (int c = warp; c < N; c += THREADS / 32) {   // whole reflectors, zero above the diagonal
+    int2* v = (int2*)(W + (long long)c * ldw);
+    for (int r = lane; r < c; r += 32) v[r] = make_int2(0, 0);
+    if (lane == 0) v[c] = vhead[c];
+  }
   __syncthreads();
-  for (int p = N - 1; p >= 0; --p) {
-    const int2* v0 = vl + (p & 1) * kRows;
-    const int2 tau = taus[p], head = vhead[p];
-    if (p > 0) {
-      int2* vn = vl + ((p - 1) & 1) * kRows;
-      const int2* src = (const int2*)(W + (long long)(p - 1) * ldw);
-      for (int r = p + tid; r < N; r += THREADS) vn[r] = src[r];
-    }
-    const int bs = p / (4 * LPC);
-    for (int c0 = p + 1; c0 + wgrp < N; c0 += ngrp) {
-      const int c = min(c0 + grp, N - 1);
-      const bool on = c0 + grp < N;
-      long long* col = W + (long long)c * ldw + sub;
-      const int2* v = v0 + sub;
-      long long x[NB][4], hi = 0, mid = 0;
+  constexpr int nw = THREADS / 32, wcols = 32 / LPC;
+  double* Ub = U + (long long)b * NN;
+  for (int rd = 0; rd * ngrp < N; ++rd) {
+    const int slot = N <= ngrp ? (warp & 4 ? min(warp | 3, nw - 1) - (warp & 3) : warp)
+                               : (rd & 1 ? nw - 1 - warp : warp);
+    const int cw = (rd * nw + slot) * wcols, c = cw + lane / LPC;
+    if (cw >= N) continue;
+    long long x[NB][4];
+#pragma unroll
+    for (int q = 0; q < NB; ++q)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[q][i] = (4 * q + i) * LPC + sub == c ? 1ll << kFix : 0;
+    for (int p = min(cw + wcols, N) - 1; p >= 0; --p) {
+      const int2 tau = taus[p];
+      const int2* v = (const int2*)(W + (long long)p * ldw) + sub;
+      const int bs = p / (4 * LPC);
+      long long hi = 0, mid = 0;
 #pragma unroll
       for (int q = 0; q < NB; ++q) {
         if (q < bs) continue;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          x[q][i] = col[(4 * q + i) * LPC];
           const int2 l = limbs(x[q][i]), w = v[(4 * q + i) * LPC];
           mad_wide(hi, w.x, l.x);
           mad_wide(mid, w.x, l.y);
@@ -413,29 +442,22 @@ k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__
         mid += __shfl_xor_sync(0xffffffffu, mid, o);
       }
       const int2 f = limbs(-madq(0, limbs(fold(hi, mid)), tau));
-      if (on) {
 #pragma unroll
-        for (int q = 0; q < NB; ++q) {
-          if (q < bs) continue;
+      for (int q = 0; q < NB; ++q) {
+        if (q < bs) continue;
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            col[(4 * q + i) * LPC] = madq(x[q][i], v[(4 * q + i) * LPC], f);
-        }
-        if (sub == p % LPC) (col - sub)[p] = madq(0, head, f);
+        for (int i = 0; i < 4; ++i) x[q][i] = madq(x[q][i], v[(4 * q + i) * LPC], f);
       }
     }
-    {   // column p itself: v . e_p = v_p
-      const int2 f = limbs(-madq(0, head, tau));
-      long long* col = W + (long long)p * ldw;
-      for (int r = tid; r < N; r += THREADS)
-        col[r] = r < p ? 0 : r == p ? madq(1ll << kFix, head, f) : madq(0, v0[r], f);
+    if (c < N) {
+#pragma unroll
+      for (int q = 0; q < NB; ++q)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = (4 * q + i) * LPC + sub;
+          if (r < N) Ub[(long long)r * N + c] = bad ? nan : pow2_scale((double)x[q][i], -kFix);
+        }
     }
-    __syncthreads();
-  }
-  double* Ub = U + (long long)b * NN;
-  for (int e = tid; e < (int)NN; e += THREADS) {
-    const int r = e / N, c = e - r * N;
-    Ub[e] = bad ? nan : pow2_scale((double)W[(long long)c * ldw + r], -kFix);
   }
 }
 
@@ -804,10 +826,9 @@ void qrp_udt(const double* X, double* U, double* D, double* Tp, double* ws, int 
   auto run = [&](auto kernel, int LPC, int NB, int threads) {
     const int rows = 4 * NB * LPC;
     const size_t small = (qr_small_bytes(rows, N) + 15) & ~(size_t)15;
-    const size_t big = small + (size_t)N * qr_ld(rows, LPC) * sizeof(long long);
-    const int use_smem = big <= kQrSmemLimit;
+    const size_t big = qr_smem(LPC) ? (size_t)N * qr_ld(rows, LPC) * sizeof(long long) : 0;
     allow_max_dynamic_smem((const void*)kernel);
-    kernel<<<batch, threads, use_smem ? big : small, st>>>(X, U, D, Tp, ws, N, use_smem);
+    kernel<<<batch, threads, small + big, st>>>(X, U, D, Tp, ws, N);
   };
   if (N <= 16) run(k_qrp<4, 1, 64, 4>, 4, 1, 64);
   else if (N <= 32) run(k_qrp<4, 2, 128, 4>, 4, 2, 128);
