@@ -81,8 +81,8 @@ __global__ void k_convt_fwd(const float* __restrict__ in, int Cin, Shape3 is,
   }
 }
 
-// The same convolution for many samples, lanes on samples: in [Cin][q][n], so that a warp's input
-// reads are contiguous, its weights uniform, and its tap ranges the same for all lanes. A warp
+// The same convolution for many samples, lanes on samples: in [Cin][q][ld], ld = n rounded up to 4,
+// so that a warp's input reads are contiguous and 16-byte copies aligned for every n, its weights uniform, and its tap ranges the same for all lanes. A warp
 // takes kTo0 outputs along the first axis (the long one of both kernels and inputs, so that nearly
 // every tap serves all of them) at one (o1, o2), a thread NS consecutive samples: one 16-byte
 // read each of inputs and weights serves 16 multiply-adds. Per input channel and q0 the CTA (one
@@ -106,7 +106,7 @@ template <int NS, bool TOUT>
 __global__ void __launch_bounds__(32 * kSampleWarps)
 k_convt_samples(const float* __restrict__ in, int Cin, Shape3 is, const float* __restrict__ W,
                 const float* __restrict__ bias, int Cout, Shape3 ks, float* __restrict__ out,
-                int n, SamplePlan pl) {
+                int n, int ld, SamplePlan pl) {
   extern __shared__ __align__(16) float sx[];
   const Shape3 os{is.d0 + ks.d0 - 1, is.d1 + ks.d1 - 1, is.d2 + ks.d2 - 1};
   constexpr int L = 32 * NS;
@@ -119,31 +119,19 @@ k_convt_samples(const float* __restrict__ in, int Cin, Shape3 is, const float* _
   const int q1a = max(0, o1 - ks.d1 + 1), q1b = min(is.d1 - 1, o1);
   const int q2a = max(0, o2 - ks.d2 + 1), q2b = min(is.d2 - 1, o2);
   const int is12 = is.d1 * is.d2, ks12 = ks.d1 * ks.d2, steps = Cin * nq0;
-  const bool vec = n % 4 == 0;
 
   auto fetch = [&](int step) {
     if (step < steps) {
       const int ci = step / nq0, q0 = q0b - (step - ci * nq0);
       float* dst = sx + step % kSampleStages * (pl.xs + pl.ws);
-      const float* src = in + (long long)(ci * is.d0 + q0) * is12 * n + s0;
-      if (vec) {
-        for (int e = tid; e < is12 * (L / 4); e += blockDim.x) {
-          const int r = e / (L / 4), c = 4 * (e % (L / 4));
-          if (s0 + c < n)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
-                             (unsigned)__cvta_generic_to_shared(dst + r * L + c)),
-                         "l"(src + (long long)r * n + c)
-                         : "memory");
-        }
-      } else {
-        for (int e = tid; e < is12 * L; e += blockDim.x) {
-          const int r = e / L, c = e % L;
-          if (s0 + c < n)
-            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
-                             (unsigned)__cvta_generic_to_shared(dst + r * L + c)),
-                         "l"(src + (long long)r * n + c)
-                         : "memory");
-        }
+      const float* src = in + (long long)(ci * is.d0 + q0) * is12 * ld + s0;
+      for (int e = tid; e < is12 * (L / 4); e += blockDim.x) {
+        const int r = e / (L / 4), c = 4 * (e % (L / 4));
+        if (s0 + c < ld)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(
+                           (unsigned)__cvta_generic_to_shared(dst + r * L + c)),
+                       "l"(src + (long long)r * ld + c)
+                       : "memory");
       }
       // weights [k1 k2][j]: tap k0 = o0 + j - q0 of output j
       const float* w = W + ((long long)ci * Cout + co) * ks.size();
@@ -185,6 +173,9 @@ k_convt_samples(const float* __restrict__ in, int Cin, Shape3 is, const float* _
           if constexpr (NS == 4) {
             const float4 u = *reinterpret_cast<const float4*>(xr + (q2 - i) * L);
             v[i][0] = u.x; v[i][1] = u.y; v[i][2] = u.z; v[i][3] = u.w;
+          } else if constexpr (NS == 2) {
+            const float2 u = *reinterpret_cast<const float2*>(xr + (q2 - i) * L);
+            v[i][0] = u.x; v[i][1] = u.y;
           } else {
             v[i][0] = xr[(q2 - i) * L];
           }
@@ -212,7 +203,7 @@ k_convt_samples(const float* __restrict__ in, int Cin, Shape3 is, const float* _
       const int m = s0 + lane * NS + s;
       if (m >= n) continue;
       const float y = 1.0f / (1.0f + expf(-acc[j][s]));
-      if (TOUT) out[((long long)co * os.size() + o) * n + m] = y;
+      if (TOUT) out[((long long)co * os.size() + o) * ld + m] = y;
       else out[((long long)m * Cout + co) * os.size() + o] = y;
     }
   }
@@ -293,14 +284,14 @@ __global__ void k_sigmoid_bwd(float* __restrict__ g, const float* __restrict__ y
 
 __global__ void k_gen_input(const long long* __restrict__ ids, long long n0, int n, int zsize,
                             uint32_t stream, uint32_t k0, uint32_t k1, float* __restrict__ z,
-                            int transposed) {
+                            int ld) {   // ld > 0: z [element][ld samples]
   const int total = n * zsize;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
     const int b = e / zsize, el = e - b * zsize;
     const long long id = ids ? ids[b] : n0 + b;
     uint32_t c[4] = {(uint32_t)el, (uint32_t)id, stream, kTagGenZ};
     philox4x32_10(c, k0, k1);
-    z[transposed ? el * n + b : e] = (c[0] >> 31) ? -1.f : 1.f;
+    z[ld ? el * ld + b : e] = (c[0] >> 31) ? -1.f : 1.f;
   }
 }
 
@@ -789,7 +780,7 @@ size_t sample_plan(const Shape3& is, const Shape3& ks, int NS, SamplePlan& pl) {
 }
 
 template <int NS>
-bool forward_samples(nmc_gen* g, int n) {
+bool forward_samples(nmc_gen* g, int n, int ld) {
   SamplePlan p1, p2;
   const size_t b1 = sample_plan(g->zs, g->k1s, NS, p1), b2 = sample_plan(g->hs, g->k2s, NS, p2);
   const unsigned groups = (n + 32 * NS - 1) / (32 * NS);
@@ -800,20 +791,41 @@ bool forward_samples(nmc_gen* g, int n) {
   allow_max_dynamic_smem((const void*)k_convt_samples<NS, false>);
   k_convt_samples<NS, true><<<dim3((g->hs.d0 + kTo0 - 1) / kTo0, groups, g->arch.c1 * p1.chunks), 32 * p1.warps, b1,
                               g->stream>>>(g->dZ, 1, g->zs, g->W1(), g->b1(), g->arch.c1, g->k1s,
-                                           g->dH1, n, p1);
+                                           g->dH1, n, ld, p1);
   k_convt_samples<NS, false><<<dim3((g->os.d0 + kTo0 - 1) / kTo0, groups, p2.chunks),
                                32 * p2.warps, b2, g->stream>>>(
-      g->dH1, g->arch.c1, g->hs, g->W2(), g->b2(), 1, g->k2s, g->dPo, n, p2);
+      g->dH1, g->arch.c1, g->hs, g->W2(), g->b2(), 1, g->k2s, g->dPo, n, ld, p2);
   return true;
 }
 
-// forward() into dPo alone, for samples that need no gradient: from 32 samples on with the lanes
-// on samples (dZ and dH1 then hold [element][sample]), unless a layer's planes are too large
+// forward() into dPo alone, for samples that need no gradient, with the lanes on samples (dZ and dH1
+// then hold [element][sample]) unless a layer's planes are too large.
+// When: k_convt_samples walks the second layer's input planes one after the other, so it takes some
+// 10 to 25% longer than k_convt_fwd while neither fills the GPU; it wins once enough multiply-adds
+// share a step of that walk, n hs.d1 hs.d2 k2.size() of them. us a probs and a sample_fields call,
+// k_convt_fwd / k_convt_samples: honeycomb 3x3, 60 slices, 8 channels: 279 / 292 at 64 samples (92 k),
+// 321 / 294 at 96 (138 k); square 6x6, 30 slices: 172 / 177 at 65 (124 k), 217 / 179 at 128 (243 k);
+// square 8x8, 20 slices: 131 / 124 at 64 (163 k); 18 sites, 20 slices: 127 / 140 at 128 (60 k).
+// How many samples a thread takes: as few as let the second layer's CTAs run at once (one to an SM),
+// at most 4. honeycomb 6x6, 60 slices, one, two or four: 320, 339, 354 us at 32 samples, 561 -> 369,
+// 340, 357 at 64, 735, 560, 435 at 256; square 6x6, 30 slices, at 128: 179, 183, 191.
+constexpr long long kSampleWork = 140000;
+
 void forward_only(nmc_gen* g, long long n0, int n, uint32_t stream) {
-  if (n >= 32) {
+  if (n >= 32 && (long long)n * g->hs.d1 * g->hs.d2 * g->k2s.size() >= kSampleWork) {
+    const int ld = (n + 3) & ~3;
     k_gen_input<<<blocks_for((long long)n * g->zs.size()), kThreads, 0, g->stream>>>(
-        nullptr, n0, n, g->zs.size(), stream, (uint32_t)g->seed, (uint32_t)(g->seed >> 32), g->dZ, 1);
-    if (n >= 64 ? forward_samples<4>(g, n) : forward_samples<1>(g, n)) return;
+        nullptr, n0, n, g->zs.size(), stream, (uint32_t)g->seed, (uint32_t)(g->seed >> 32), g->dZ, ld);
+    SamplePlan pl;
+    sample_plan(g->hs, g->k2s, 1, pl);
+    const long long per = (long long)((g->os.d0 + kTo0 - 1) / kTo0) * pl.chunks;   // CTAs per 32 NS samples
+    if (per * ((n + 31) / 32) <= sm_count()) {
+      if (forward_samples<1>(g, n, ld)) return;
+    } else if (per * ((n + 63) / 64) <= sm_count()) {
+      if (forward_samples<2>(g, n, ld)) return;
+    } else if (forward_samples<4>(g, n, ld)) {
+      return;
+    }
   }
   forward(g, nullptr, n0, n, stream);
 }
@@ -894,8 +906,9 @@ nmc_status nmc_gen_create(int lattice, int Lx, int Ly, double t, double U, doubl
   nmc_status s = NMC_OK;
   auto A_ = [&](auto*& p, long long n) { if (s == NMC_OK) s = galloc(g, p, n); };
   A_(g->dP, g->nP); A_(g->dGP, g->nP); A_(g->dM, g->nP); A_(g->dV, g->nP);
-  A_(g->dZ, (long long)g->Bf * zs.size());
-  A_(g->dH1, (long long)g->Bf * a.c1 * hs.size());
+  const long long Bs = (g->Bf + 3) & ~3;   // (a sample's stride in k_convt_samples)
+  A_(g->dZ, Bs * zs.size());
+  A_(g->dH1, Bs * a.c1 * hs.size());
   A_(g->dGh1, (long long)g->Bf * a.c1 * hs.size());
   A_(g->dPo, (long long)g->Bf * os.size());
   A_(g->dGa2, (long long)g->Bf * os.size());
