@@ -15,6 +15,8 @@
 #include "fold16.cuh"
 #include "nmc_internal.cuh"
 
+#include <type_traits>
+
 namespace nmc {
 
 namespace {
@@ -56,7 +58,8 @@ constexpr size_t kQrSmemLimit = 225 * 1024;
 // registers, the pivot column is read once, and what is in shared memory is so at compile time. On one
 // set of graded and degenerate matrices, with the same bits: 45 -> 35 (16, 2), 143 -> 115 (36, 128),
 // 291 -> 230 (64, 6), 414 -> 340 (64, 512), 422 -> 369 (72, 6), 1397 -> 1229 (72, 1024), 717 -> 619
-// (100, 128), 1387 -> 1245 (144, 128), 5734 -> 5181 (256, 64), 37.5 -> 30.8 ms (512, 2).
+// (100, 128), 1387 -> 1245 (144, 128), 5734 -> 5181 (256, 64), 37.5 -> 30.8 ms (512, 2); with the rows'
+// loops without tests per block 33, 107, 195, 338, 275, 1137, 571, 1100, 3861 us and 23.5 ms.
 // max |U^T U - I| 7e-17 against 8e-16, columns of U D T to 1.5e-16 against 9e-16 (N = 64).
 constexpr int kLimb = 29, kFix = 58;
 
@@ -152,6 +155,42 @@ __host__ __device__ constexpr size_t qr_small_bytes(int rows, int N) {
 // The working matrix is in shared memory up to 160 sites (8 lanes), which is all that fits.
 __host__ __device__ constexpr bool qr_smem(int LPC) { return LPC < 16; }
 static_assert(((qr_small_bytes(160, 160) + 15) & ~(size_t)15) + 160 * qr_ld(160, 8) * 8 <= kQrSmemLimit, "");
+
+// f(block number as a type) for the first block bs in [B, NB): one straight run of code for each first
+// block, where a test per block would keep a block's loads from starting before the last one's sums
+template <int B, int NB, class F>
+__device__ __forceinline__ void from_block(int bs, F&& f) {
+  if constexpr (B + 1 < NB) {
+    if (bs > B) {
+      from_block<B + 1, NB>(bs, f);
+      return;
+    }
+  }
+  f(std::integral_constant<int, B>{});
+}
+
+// dot product of a column, x in registers, and a reflector's limbs, as hi + mid / 2^29, in this lane's
+// rows of the blocks from B on
+template <int B, int NB, int LPC>
+__device__ __forceinline__ void dot_rows(const long long (&x)[NB][4], const int2* v, long long& hi, long long& mid) {
+  long long m0 = 0, m1 = 0;   // two chains (wrapping sums: any order gives the same)
+  hi = 0;
+#pragma unroll
+  for (int q = B; q < NB; ++q)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int2 l = limbs(x[q][i]), w = v[(4 * q + i) * LPC];
+      mad_wide(hi, w.x, l.x);
+      mad_wide(m0, w.x, l.y);
+      mad_wide(m1, w.y, l.x);
+    }
+  mid = m0 + m1;
+#pragma unroll
+  for (int o = 1; o < LPC; o <<= 1) {
+    hi += __shfl_xor_sync(0xffffffffu, hi, o);
+    mid += __shfl_xor_sync(0xffffffffu, mid, o);
+  }
+}
 
 template <int LPC, int NB, int THREADS, int CTAS>
 __global__ void __launch_bounds__(THREADS, CTAS)
@@ -317,57 +356,45 @@ k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__
       const bool on = c0 + grp < N;
       long long* col = W + (long long)c * ldw + sub;
       const int2* v = vp + sub;
-      long long x[NB][4], hi = 0, mid = 0;
+      const float a2 = n2[c], a0 = n1[c];
+      from_block<0, NB>(bs, [&](auto first) {
+        constexpr int B = decltype(first)::value;
+        long long x[NB][4], hi, mid;
 #pragma unroll
-      for (int q = 0; q < NB; ++q) {
-        if (q < bs) continue;
+        for (int q = B; q < NB; ++q)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          x[q][i] = col[(4 * q + i) * LPC];
-          const int2 l = limbs(x[q][i]), w = v[(4 * q + i) * LPC];
-          mad_wide(hi, w.x, l.x);
-          mad_wide(mid, w.x, l.y);
-          mad_wide(mid, w.y, l.x);
-        }
-      }
+          for (int i = 0; i < 4; ++i) x[q][i] = col[(4 * q + i) * LPC];
+        dot_rows<B, NB, LPC>(x, v, hi, mid);
+        const int2 f = limbs(-madq(0, limbs(fold(hi, mid)), tau));
 #pragma unroll
-      for (int o = 1; o < LPC; o <<= 1) {
-        hi += __shfl_xor_sync(0xffffffffu, hi, o);
-        mid += __shfl_xor_sync(0xffffffffu, mid, o);
-      }
-      const int2 f = limbs(-madq(0, limbs(fold(hi, mid)), tau));
+        for (int q = B; q < NB; ++q)
 #pragma unroll
-      for (int q = 0; q < NB; ++q) {
-        if (q < bs) continue;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {   // (rows above p: v is zero there)
-          x[q][i] = madq(x[q][i], v[(4 * q + i) * LPC], f);
-          if (on) col[(4 * q + i) * LPC] = x[q][i];
-        }
-      }
-      // trailing norm: downdated by row p's entry, summed again when less than 2^-12 of the last
-      // sum is left
-      __syncwarp();
-      const float rp = (float)(col - sub)[p] * 0x1p-58f, a2 = n2[c];
-      float a1 = fmaf(-rp, rp, n1[c]);
-      const bool again = on && !(a1 > 0x1p-12f * a2);
-      if (__any_sync(0xffffffffu, again)) {
-        float s = 0.f;
-#pragma unroll
-        for (int q = 0; q < NB; ++q) {
-          if (q < bs) continue;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float y = (4 * q + i) * LPC + sub > p ? (float)x[q][i] * 0x1p-58f : 0.f;
-            s = fmaf(y, y, s);
+          for (int i = 0; i < 4; ++i) {   // (rows above p: v is zero there)
+            x[q][i] = madq(x[q][i], v[(4 * q + i) * LPC], f);
+            if (on) col[(4 * q + i) * LPC] = x[q][i];
           }
-        }
+        // trailing norm: downdated by row p's entry, summed again when less than 2^-12 of the last
+        // sum is left
+        __syncwarp();
+        const float rp = (float)(col - sub)[p] * 0x1p-58f;
+        float a1 = fmaf(-rp, rp, a0);
+        const bool again = on && !(a1 > 0x1p-12f * a2);
+        if (__any_sync(0xffffffffu, again)) {
+          float s = 0.f;
 #pragma unroll
-        for (int o = 1; o < LPC; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (again && sub == 0) n2[c] = s;
-        if (again) a1 = s;
-      }
-      if (on && sub == 0) n1[c] = a1;
+          for (int q = B; q < NB; ++q)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float y = (4 * q + i) * LPC + sub > p ? (float)x[q][i] * 0x1p-58f : 0.f;
+              s = fmaf(y, y, s);
+            }
+#pragma unroll
+          for (int o = 1; o < LPC; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+          if (again && sub == 0) n2[c] = s;
+          if (again) a1 = s;
+        }
+        if (on && sub == 0) n1[c] = a1;
+      });
     }
     __syncthreads();
   }
@@ -423,31 +450,16 @@ k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__
     for (int p = min(cw + wcols, N) - 1; p >= 0; --p) {
       const int2 tau = taus[p];
       const int2* v = (const int2*)(W + (long long)p * ldw) + sub;
-      const int bs = p / (4 * LPC);
-      long long hi = 0, mid = 0;
+      from_block<0, NB>(p / (4 * LPC), [&](auto first) {
+        constexpr int B = decltype(first)::value;
+        long long hi, mid;
+        dot_rows<B, NB, LPC>(x, v, hi, mid);
+        const int2 f = limbs(-madq(0, limbs(fold(hi, mid)), tau));
 #pragma unroll
-      for (int q = 0; q < NB; ++q) {
-        if (q < bs) continue;
+        for (int q = B; q < NB; ++q)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int2 l = limbs(x[q][i]), w = v[(4 * q + i) * LPC];
-          mad_wide(hi, w.x, l.x);
-          mad_wide(mid, w.x, l.y);
-          mad_wide(mid, w.y, l.x);
-        }
-      }
-#pragma unroll
-      for (int o = 1; o < LPC; o <<= 1) {
-        hi += __shfl_xor_sync(0xffffffffu, hi, o);
-        mid += __shfl_xor_sync(0xffffffffu, mid, o);
-      }
-      const int2 f = limbs(-madq(0, limbs(fold(hi, mid)), tau));
-#pragma unroll
-      for (int q = 0; q < NB; ++q) {
-        if (q < bs) continue;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) x[q][i] = madq(x[q][i], v[(4 * q + i) * LPC], f);
-      }
+          for (int i = 0; i < 4; ++i) x[q][i] = madq(x[q][i], v[(4 * q + i) * LPC], f);
+      });
     }
     if (c < N) {
 #pragma unroll
@@ -819,8 +831,12 @@ k_solve(const double* __restrict__ X, const double* __restrict__ UR, long long s
 
 }  // namespace
 
-// The lanes per column follow from N alone (results must not depend on the batch): as few as keep
-// a lane's rows within 16 or 20 register pairs, and as many threads as columns need up to 512.
+// The lanes per column follow from N alone: as few as keep a lane's rows within 16 or 20 register
+// pairs, and as many threads as columns need up to 512. Up to 64 sites a batch that fits the SMs at two
+// (three) CTAs each takes the kernel with that many, which spills no registers, a larger one the kernel
+// that puts four (five) there; the arithmetic is the same. us at two / four: 195 / 209 (64, 6), 426 / 338
+// (64, 512); at three / five: 107 / 112 (36, 128). Up to 80 sites two are better than three either way:
+// 275 / 305 (72, 6), 1137 / 1220 (72, 1024).
 void qrp_udt(const double* X, double* U, double* D, double* Tp, double* ws, int N, int batch,
              cudaStream_t st) {
   auto run = [&](auto kernel, int LPC, int NB, int threads) {
@@ -832,9 +848,11 @@ void qrp_udt(const double* X, double* U, double* D, double* Tp, double* ws, int 
   };
   if (N <= 16) run(k_qrp<4, 1, 64, 4>, 4, 1, 64);
   else if (N <= 32) run(k_qrp<4, 2, 128, 4>, 4, 2, 128);
-  else if (N <= 48) run(k_qrp<4, 3, 192, 5>, 4, 3, 192);
-  else if (N <= 64) run(k_qrp<4, 4, 256, 4>, 4, 4, 256);
-  else if (N <= 80) run(k_qrp<4, 5, 320, 3>, 4, 5, 320);
+  else if (N <= 48 && batch > 3 * sm_count()) run(k_qrp<4, 3, 192, 5>, 4, 3, 192);
+  else if (N <= 48) run(k_qrp<4, 3, 192, 3>, 4, 3, 192);
+  else if (N <= 64 && batch > 2 * sm_count()) run(k_qrp<4, 4, 256, 4>, 4, 4, 256);
+  else if (N <= 64) run(k_qrp<4, 4, 256, 2>, 4, 4, 256);
+  else if (N <= 80) run(k_qrp<4, 5, 320, 2>, 4, 5, 320);
   else if (N <= 128) run(k_qrp<8, 4, 512, 1>, 8, 4, 512);
   else if (N <= 160) run(k_qrp<8, 5, 512, 1>, 8, 5, 512);
   else if (N <= 256) run(k_qrp<16, 4, 512, 1>, 16, 4, 512);
