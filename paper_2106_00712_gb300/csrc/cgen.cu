@@ -16,12 +16,13 @@
 //                ReLU mask of that input (it is the previous layer's output), as BF16;
 //   k_cg_bwd_w_tc dL/dW[co][ci][k] = sum_{n,p} g[n][co][p] in[n][ci][p + d_k] and
 //                dL/db[co] = sum g[n][co][p], as one product over all positions;
-//   k_cg_fwd, k_cg_bwd_in, k_cg_bwd_w: the same one output per thread (or CTA), for shapes
-//                whose halo does not fit shared memory or whose rows have odd length;
+//   k_cg_fwd, k_cg_bwd_in, k_cg_bwd_w: the same one output per thread (or CTA), for small calls and
+//                shapes whose halo does not fit shared memory or whose rows have odd length;
 //   k_cg_adam    Adam on the FP32 master weights, then their BF16 copy.
 // Noise and Bernoulli draws are Philox4x32-10 words (counter (p, sample, stream, tag)).
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <new>
 #include <string>
@@ -318,10 +319,19 @@ k_cg_conv(const __nv_bfloat16* __restrict__ in, int Cin, const float* __restrict
   }
 }
 
-// FP32 copies of one layer's BF16 weights as k_cg_conv reads them: wf [k][Cin][CoP], wb
-// [k][Cout][CiP] (the padding zero)
-__global__ void k_cg_layout(const __nv_bfloat16* __restrict__ W, int Cin, int Cout, int CoP,
-                            int CiP, float* __restrict__ wf, float* __restrict__ wb) {
+// FP32 copies of the layers' BF16 weights as k_cg_conv reads them, a layer per blockIdx.y: wf
+// [k][Cin][CoP], wb [k][Cout][CiP] (the padding zero)
+struct LayoutArgs {
+  const __nv_bfloat16* W[kLayers];
+  float *wf[kLayers], *wb[kLayers];
+  int cin[kLayers], cout[kLayers];
+};
+__host__ __device__ constexpr int pad8(int c) { return (c + 7) & ~7; }
+
+__global__ void k_cg_layout(LayoutArgs a) {
+  const int j = blockIdx.y, Cin = a.cin[j], Cout = a.cout[j], CoP = pad8(Cout), CiP = pad8(Cin);
+  const __nv_bfloat16* W = a.W[j];
+  float *wf = a.wf[j], *wb = a.wb[j];
   const int nf = kK * Cin * CoP, total = nf + kK * Cout * CiP;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
     const bool f = e < nf;
@@ -597,8 +607,6 @@ nmc_status cg_last(void) {
   return e == cudaSuccess ? NMC_OK : NMC_ECUDA;
 }
 
-int pad8(int c) { return (c + 7) & ~7; }
-
 constexpr size_t kConvSmem = 200 * 1024;
 
 // Shared memory of a k_cg_conv tile of PT positions and cos channels: the slices that PT
@@ -611,13 +619,27 @@ size_t conv_smem(const Dims& d, int Cin, int PT, int cos) {
   return ((words + 3) & ~(size_t)3) * 4 + 2 * 3 * (size_t)Cin * cos * 4;
 }
 
-// One convolution (or its transpose) by the tiled kernel; false: its halo does not fit. 256
+// From how many outputs of a middle layer on the tiled kernel takes the convolutions: it keeps 16 to 64
+// sums per thread and one or two CTAs per SM, so below, most of the GPU waits for a few, and one output
+// per thread is faster. us a sampling call, one per thread / tiled (outputs): 8 channels 61 / 81 (15 k),
+// 88 / 84 (95 k), 115 / 84 (192 k); 16 channels 72 / 101 (10 k), 113 / 106 (123 k), 166 / 106 (246 k);
+// 32 channels 90 / 150 (20 k), 149 / 152 (123 k), 234 / 156 (246 k). The bits are the same.
+constexpr long long kTileOutputs = 125000;
+// The same for the weight gradients, in positions: the one product has a fixed cost of some 25 us (8
+// channels) to 60 (32) a call. us a gradient call, a CTA per channel pair / one product (positions): 8
+// channels 138 / 159 (1280), 171 / 166 (2560), 242 / 194 (6000); 16 channels 165 / 196 (1280), 208 / 211
+// (2560), 313 / 268 (6000); 32 channels 231 / 272 (960), 369 / 344 (2560), 505 / 409 (4000).
+constexpr long long kTcPositions = 2600;
+
+// One convolution (or its transpose) by the tiled kernel; false: its halo does not fit or there are too
+// few outputs. 256
 // positions per CTA, or 64 while those would not give every SM two CTAs (37 x 1080 positions, 32
 // channels: 121 us per middle layer with 64, 127 with 128).
 template <int MODE>
 bool conv_tiled(nmc_cgen* g, const __nv_bfloat16* in, int Cin, const float* wt, const float* bias,
                 int Cout, int n, const __nv_bfloat16* act, __nv_bfloat16* out_h, float* out_f) {
   const int S = g->d.S();
+  if ((long long)n * S * g->C < kTileOutputs) return false;
   auto run = [&](auto kernel, int TP, int TC) {
     const int groups = (Cout + TC - 1) / TC, wco = TC == 2 ? 1 : groups >= 3 ? 4 : groups;
     const int PT = kConvThreads / wco * TP;
@@ -653,11 +675,12 @@ void forward(nmc_cgen* g, int n) {
 }
 
 // Weight and bias gradients of one layer as one product over all positions; false: rows of odd
-// length (a pair of positions would straddle two), more than 32 channels, or slices that do not
-// fit shared memory.
+// length (a pair of positions would straddle two), more than 32 channels, too few positions, or
+// slices that do not fit shared memory.
 bool bwd_w_tc(nmc_cgen* g, int j, const __nv_bfloat16* gin, int n) {
   const Dims& d = g->d;
   const int Cin = g->cin[j], Cout = g->cout[j];
+  if ((long long)n * d.S() < kTcPositions) return false;
   if (d.B % 2 || Cin > 32 || Cout > 32 || !g->part) return false;
   const int MT = Cout > 16 ? 2 : 1, NC = Cin > 16 ? 4 : Cin > 8 ? 2 : 1;
   BwTile t{};
@@ -714,11 +737,18 @@ void backward(nmc_cgen* g, const int8_t* d_fields, int n) {
 
 // the convolutions' layouts of the current BF16 weights
 void layout(nmc_cgen* g) {
+  LayoutArgs a;
+  int most = 0;
   for (int j = 0; j < kLayers; ++j) {
     const int ci = g->cin[j], co = g->cout[j];
-    k_cg_layout<<<grid_for((long long)kK * (ci * pad8(co) + co * pad8(ci)), 256), 256, 0, g->st>>>(
-        g->thb + g->oW[j], ci, co, pad8(co), pad8(ci), g->wf[j], g->wb[j]);
+    a.W[j] = g->thb + g->oW[j];
+    a.wf[j] = g->wf[j];
+    a.wb[j] = g->wb[j];
+    a.cin[j] = ci;
+    a.cout[j] = co;
+    most = std::max(most, kK * (ci * pad8(co) + co * pad8(ci)));
   }
+  k_cg_layout<<<dim3(grid_for(most, 256), kLayers), 256, 0, g->st>>>(a);
 }
 
 void noise(nmc_cgen* g, long long n0, int n, uint32_t stream) {
