@@ -528,9 +528,10 @@ k_chain(const ChainArgs<V> g) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int c = column(nt, 4 * h);
-        const char2 sc = c < N ? *(const char2*)(s + c) : make_char2(1, 1);   // (N is even)
+        // one byte at a time: nmc_green_noalloc's caller may have the fields at any address (N is even)
+        const int8_t s0 = c < N ? s[c] : 1, s1 = c < N ? s[c + 1] : 1;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) y[j][4 * h + i] = field(y[j][4 * h + i], (i & 1) ? sc.y : sc.x);
+        for (int i = 0; i < 4; ++i) y[j][4 * h + i] = field(y[j][4 * h + i], (i & 1) ? s1 : s0);
       }
     }
     if (k == 0) __syncthreads();   // the staged digits are read: their place is the fragments'
