@@ -81,7 +81,10 @@ typedef enum { NMC_SQUARE = 0, NMC_HONEYCOMB = 1 } nmc_lattice;
 
 typedef struct {
   int n_chains;          /* independent chains held by this context (>= 1)       default 1  */
-  int delay_k;           /* accepted flips folded per rank-k delayed update (>= 1) def. 16   */
+  int delay_k;           /* most accepted flips folded into G at once (>= 1): small values, FP32
+                            and the largest lattices fold after so many, otherwise after each
+                            block of min(delay_k, 16) sites. The same decisions and, up to
+                            rounding, the same G for every value.              default 16   */
   int precision;         /* nmc_precision                                        default 0  */
   double drift_tol;      /* NMC_ENUMERIC if max|G_wrapped - G_recomputed| exceeds this;
                             <= 0 selects 1e-6 (FP64), 1e-3 (FP32), 1e-5 (SPLIT_BF16,

@@ -12,9 +12,9 @@
 // G0 += A B^T. In exact arithmetic this equals applying each rank-1 update at once.
 // G0 of both spins sits in shared memory when it fits (N <= 64 in FP64), else in global
 // memory (L2); the panels always live in shared memory (k is clamped to fit).
-// That is k_flip in FP32, above some 560 sites in FP64, and k_flip_df above some 430 in FP32 pairs
-// without tensor cores (with them there are 320 at most); below, FP64 and FP32 pairs take k_flip_block,
-// which decides blocks of up to min(k, 16) sites apart.
+// That is k_flip in FP32, and in FP64 for small k and above some 560 sites; and k_flip_df in FP32 pairs
+// for small k and above some 430 sites without tensor cores (with them there are 320 at most). Between,
+// FP64 and FP32 pairs take k_flip_block, which decides blocks of up to min(k, 16) sites apart.
 #include <cooperative_groups.h>
 
 #include "fold16.cuh"
@@ -993,15 +993,34 @@ void flip_slice<float>(const FlipArgs<float>& f, int n_chains, cudaStream_t st) 
   flip_old(f, n_chains, st);
 }
 
+// Small delays: a block of min(delay, 16) sites holds at most so many accepted flips, but a block's fixed
+// costs (its submatrix, the vectors over all sites, the digits) want some five of them; below, one flip at
+// a time is faster, while its matrices fit shared memory (FP64: twice to an SM). The line follows the
+// delay and delay x sites, not the number of chains, so a chain's results do not depend on those beside it.
+// us a slice, one at a time / blocks, 60% accepted, by delay:
+//   FP32 pairs   16 sites x 512, delay 1 55 / 141, 4 40 / 61, 8 37 / 44, 12 38 / 45, 16 37 / 36;
+//                64 x 256, 1 208 / 544, 4 139 / 204, 6 133 / 155, 8 131 / 126;
+//                80 x 200, 3 285 / 537, 5 355 / 361, 8 331 / 259;  100 x 64, 4 317 / 344, 5 326 / 286;
+//   FP64         16 x 512, 1 76 / 231, 6 72 / 84, 8 73 / 70;  36 x 256, 1 143 / 440, 6 121 / 125, 8 123 / 114;
+//                64 x 256, 1 408 / 1007, 4 324 / 371, 5 326 / 317;  100 x 64, 2 956 / 975, 3 823 / 711;
+//   FP32X2       64 x 256, 1 208 / 287, 4 139 / 186, 8 131 / 164 (at 44% accepted about even there).
+// With every delay in blocks a whole sweep was up to twice as long as with one flip at a time (16 sites x 1 in
+// FP64, delay 1: 2.3 / 4.5 ms a pair).
+constexpr int kSingleDelay = 8, kSingleWork = 430;           // FP32 pairs
+constexpr int kSingleDelay64 = 6, kSingleWork64 = 300;       // FP64
+
 template <>
 void flip_slice<double>(const FlipArgs<double>& f, int n_chains, cudaStream_t st) {
-  if (!flip_block<double, kFoldTensor>(f, n_chains, st)) flip_old(f, n_chains, st);
+  const bool single = f.kk <= kSingleDelay64 && f.kk * f.N <= kSingleWork64 && f.g_in_smem &&
+                      flip_smem_bytes(f.N, f.kk, sizeof(double), 1, f.ns) <= kBlockSmem / 2;
+  if (single || !flip_block<double, kFoldTensor>(f, n_chains, st)) flip_old(f, n_chains, st);
 }
 
 template <>
 void flip_slice<df2>(const FlipArgs<df2>& f, int n_chains, cudaStream_t st) {
-  if (f.tc_fold ? flip_block<df2, kFoldTensor>(f, n_chains, st)
-                : flip_block<df2, kFoldPairs>(f, n_chains, st))
+  const bool single = f.kk <= kSingleDelay && f.kk * f.N <= kSingleWork && f.g_in_smem;
+  if (!single && (f.tc_fold ? flip_block<df2, kFoldTensor>(f, n_chains, st)
+                            : flip_block<df2, kFoldPairs>(f, n_chains, st)))
     return;
   const size_t bytes = flip_smem_bytes(f.N, f.kk, sizeof(df2), f.g_in_smem, f.ns);
   allow_max_dynamic_smem((const void*)k_flip_df);
