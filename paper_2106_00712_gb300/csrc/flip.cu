@@ -482,12 +482,7 @@ template <> struct Arith<df2> {
   static __device__ __forceinline__ df2 add(df2 a, df2 b) { return df_add(a, b); }
   static __device__ __forceinline__ void fma_acc(df2& c, df2 a, df2 b) { df_fma_acc(c, a, b); }
   static __device__ __forceinline__ df2 finish(df2 a) { return df_finish(a); }
-  // a / b: approximate FP32 reciprocal r (2^-23), its residual 1 - b r as the low part (2^-46)
-  static __device__ __forceinline__ df2 div(df2 a, df2 b) {
-    const float r = __fdividef(1.f, b.hi);
-    const float e = __fmaf_rn(-b.lo, r, __fmaf_rn(-b.hi, r, 1.f));
-    return df_mul(a, df2{r, __fmul_rn(r, e)});
-  }
+  static __device__ __forceinline__ df2 div(df2 a, df2 b) { return df_div(a, b); }
 };
 template <> struct Arith<double> {
   static __device__ __forceinline__ double zero() { return 0.0; }

@@ -1,8 +1,14 @@
-"""The FP64 quotient of the flips (csrc/quotient.cuh) against the division, compiled into a program of its
-own: 2^24 pairs of random mantissas over the exponents that it handles itself, over all exponents, and
-every pair of special values. The quotient before its last rounding is off by less than 2^-48 units of the
-last place (derived in the header), so a result other than the division's has a chance of 2^-47 a pair, and
-none is expected."""
+"""The flips' quotients, each compiled into a program of its own.
+
+FP64 (csrc/quotient.cuh) against the division: 2^24 pairs of random mantissas over the exponents that it
+handles itself, 2^24 over all exponents, and every pair of special values. The quotient before its last
+rounding is off by less than 2^-48 units of the last place (derived in the header), so a result other than
+the division's has a chance of 2^-47 a pair, and none is expected.
+
+FP32 pairs (df_div of csrc/df.cuh) against the FP64 quotient of the same values: 2^24 random pairs, off by at
+most the 2.75 x 2^-46 derived there (and the reference's 2^-53) and, where the quotient's low part is
+subnormal, three products' and a sum's roundings of 2^-150; and divisors between 2^126 and the largest,
+where the FP32 reciprocal has some 22 bits: 2^-20."""
 import os
 import shutil
 import subprocess
@@ -61,7 +67,45 @@ int main() {
 '''
 
 
-def test_quotient_is_the_division(tmp_path):
+PAIRS = r'''
+#include <cstdio>
+#include <cstring>
+#include "nmc_internal.cuh"
+using namespace nmc;
+__device__ df2 number(unsigned hi, unsigned lo, int emin, int span) {   // |low part| <= half a unit of the high one
+  const float h = __uint_as_float((hi & 0x807fffffu) | ((unsigned)(emin + (lo & 0xffffu) % (unsigned)span) << 23));
+  const float ulp = __uint_as_float((__float_as_uint(h) & 0x7f800000u)) * 0x1p-24f;
+  return df_norm(h, ulp * ((float)(int)(lo & 0xffff8000u) * 0x1p-31f));
+}
+__global__ void check(int set, unsigned long long* bad, unsigned* worst) {
+  unsigned c[4] = {blockIdx.x * blockDim.x + threadIdx.x, (unsigned)set, 0u, 1u};
+  philox4x32_10(c, 7u, 11u);
+  const df2 a = number(c[0], c[1], set ? 200 : 67, set ? 40 : 120);
+  const df2 b = number(c[2], c[3], set ? 253 : 67, set ? 2 : 120);
+  const double w = df_to_double(a) / df_to_double(b), q = df_to_double(df_div(a, b));
+  const double off = fmax(fabs(q - w) - 4 * 0x1p-150, 0.0) / fabs(w);
+  if (!set) atomicMax(worst, __float_as_uint((float)off));
+  if (!(off <= (set ? 0x1p-20 : 2.75 * 0x1p-46 + 0x1p-53)) && atomicAdd(bad, 1ull) < 8)
+    printf("set %d: %.17g / %.17g off by %.3g\n", set, df_to_double(a), df_to_double(b), off);
+}
+int main() {
+  unsigned long long *bad, n = 0;
+  unsigned w = 0;
+  cudaMalloc(&bad, 16);
+  cudaMemset(bad, 0, 16);
+  for (int set = 0; set < 2; ++set) check<<<65536, 256>>>(set, bad, (unsigned*)(bad + 1));
+  const bool ok = cudaMemcpy(&n, bad, 8, cudaMemcpyDeviceToHost) == cudaSuccess &&
+                  cudaMemcpy(&w, bad + 1, 4, cudaMemcpyDeviceToHost) == cudaSuccess;
+  float f;
+  memcpy(&f, &w, 4);
+  printf("%s, %llu off, at most %.3g\n", ok ? "done" : "failed", n, f);
+  return ok && n == 0 ? 0 : 1;
+}
+'''
+
+
+@pytest.mark.parametrize("program", [PROGRAM, PAIRS], ids=["fp64", "pairs"])
+def test_quotients(tmp_path, program):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -69,8 +113,9 @@ def test_quotient_is_the_division(tmp_path):
     nvcc = build_lib._nvcc()
     assert shutil.which(nvcc), nvcc
     src, exe = tmp_path / "quotients.cu", tmp_path / "quotients"
-    src.write_text(PROGRAM)
+    src.write_text(program)
     subprocess.run([nvcc, str(src), "-o", str(exe), "-I", build_lib.CSRC] + build_lib.ARCH
                    + build_lib.NVCC_FLAGS, check=True, timeout=300)
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
+    print(r.stdout)
     assert r.returncode == 0, r.stdout + r.stderr
