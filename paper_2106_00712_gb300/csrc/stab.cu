@@ -588,13 +588,6 @@ __host__ __device__ inline size_t solve_small_bytes(int N, int chunk, int nw) {
          + (size_t)N * 8 + (size_t)((N + 3) & ~3) * 4 + 64;             // 1 / pivots, row map, block's pivots
 }
 
-__device__ __forceinline__ double rcp64(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);   // 2^-20: 1 / x = r (1 + e + e^2 + O(2^-60))
-  return fma(r, fma(e, e, e), r);
-}
-
 // RP: rows per thread of a panel. lda: row stride of the augmented matrix; chunk: columns whose digits
 // are held at a time (a multiple of 16).
 template <int THREADS, int RP, int CTAS, bool SMEM>
@@ -690,7 +683,7 @@ k_solve(const double* __restrict__ X, const double* __restrict__ UR, long long s
 #pragma unroll
         for (int i = 0; i < RP; ++i)
           if (i == ci) {
-            cinv[p & 1][warp] = rcp64(a[i][p]);
+            cinv[p & 1][warp] = 1.0 / a[i][p];
 #pragma unroll
             for (int c = 0; c < 16; ++c)
               if (c >= p) cand[p & 1][warp][c] = a[i][c];
