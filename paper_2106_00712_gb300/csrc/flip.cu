@@ -13,8 +13,8 @@
 // G0 of both spins sits in shared memory when it fits (N <= 64 in FP64), else in global
 // memory (L2); the panels always live in shared memory (k is clamped to fit).
 // That is k_flip in FP32, and in FP64 for small k and above some 560 sites; and k_flip_df in FP32 pairs
-// for small k and above some 430 sites without tensor cores (with them there are 320 at most). Between,
-// FP64 and FP32 pairs take k_flip_block, which decides blocks of up to min(k, 16) sites apart.
+// for small k, and without tensor cores for most sizes. Elsewhere FP64 and FP32 pairs take k_flip_block,
+// which decides blocks of up to min(k, 16) sites apart (the rules stand at flip_slice).
 #include <cooperative_groups.h>
 
 #include "fold16.cuh"
@@ -460,11 +460,11 @@ __global__ void __launch_bounds__(kThreadsDf, 2) k_flip_df(const FlipArgs<df2> f
 // (fold16.cuh), cut straight from the registers the vectors were formed in.
 // Without tensor cores (FP32X2) the vectors go through shared memory to the FP32-pair loop.
 //
-// One slice, us, 44% of the flips accepted, one flip at a time (k_flip, k_flip_df) -> here:
-//   64 sites x 256 chains, both spins: FP32 pairs 133 -> 75, FP64 357 -> 139, FP32X2 133 -> 110
-//   72 x 1024, one spin: 625 -> 242;  256 x 32: 2950 -> 391;  100 x 64: 481 -> 118;
-//   16 x 1 in FP64: 31 -> 16.
-// What bounds it at 64 x 256 (two CTAs per SM): latency. Of a slice's 146k cycles the decisions take
+// One slice, us, one flip at a time (k_flip, k_flip_df) -> here, two thirds of the flips accepted (U = 4):
+//   64 sites x 256 chains, both spins: FP32 pairs 133 -> 90, FP64 356 -> 181; a third of them (U = 8): 104 -> 74,
+//   244 -> 137; 72 x 1024, one spin, pairs: 420 -> 307; 256 x 32: 2751 -> 444; 100 x 64: 315 -> 140;
+//   16 x 256 in FP64: 50 -> 37. (FP32X2: see flip_slice.)
+// What bounds it at 64 x 256 (two CTAs per SM): latency. Of a slice's 146k cycles (44% accepted) the decisions take
 // 45k (28 acceptances of some 1500: two ratios, a reciprocal and four rows' updates in a dependent
 // chain), the folds 47k (of which the MMAs' issue is 23k), the digits 24k, the vectors 13k. In FP64
 // the pipe's one instruction per 20 cycles bounds vectors and fold sums.
@@ -987,13 +987,12 @@ void flip_slice<float>(const FlipArgs<float>& f, int n_chains, cudaStream_t st) 
 // costs (its submatrix, the vectors over all sites, the digits) want some five of them; below, one flip at
 // a time is faster, while its matrices fit shared memory (FP64: twice to an SM). The line follows the
 // delay and delay x sites, not the number of chains, so a chain's results do not depend on those beside it.
-// us a slice, one at a time / blocks, 60% accepted, by delay:
+// us a slice, one at a time / blocks, 66% accepted, by delay:
 //   FP32 pairs   16 sites x 512, delay 1 55 / 141, 4 40 / 61, 8 37 / 44, 12 38 / 45, 16 37 / 36;
 //                64 x 256, 1 208 / 544, 4 139 / 204, 6 133 / 155, 8 131 / 126;
 //                80 x 200, 3 285 / 537, 5 355 / 361, 8 331 / 259;  100 x 64, 4 317 / 344, 5 326 / 286;
 //   FP64         16 x 512, 1 76 / 231, 6 72 / 84, 8 73 / 70;  36 x 256, 1 143 / 440, 6 121 / 125, 8 123 / 114;
 //                64 x 256, 1 408 / 1007, 4 324 / 371, 5 326 / 317;  100 x 64, 2 956 / 975, 3 823 / 711;
-//   FP32X2       64 x 256, 1 208 / 287, 4 139 / 186, 8 131 / 164 (at 44% accepted about even there).
 // With every delay in blocks a whole sweep was up to twice as long as with one flip at a time (16 sites x 1 in
 // FP64, delay 1: 2.3 / 4.5 ms a pair).
 constexpr int kSingleDelay = 8, kSingleWork = 430;           // FP32 pairs
@@ -1006,11 +1005,23 @@ void flip_slice<double>(const FlipArgs<double>& f, int n_chains, cudaStream_t st
   if (single || !flip_block<double, kFoldTensor>(f, n_chains, st)) flip_old(f, n_chains, st);
 }
 
+// FP32X2, without tensor cores: a block's fold costs as much as the folds of single flips, and the vectors come
+// on top, so blocks pay only for a few sites, and where both spins' matrices fit beside a block but not beside
+// k_flip_df's panels twice to an SM (its 288 threads alone are too few). us a slice at delay 16, one at a time / blocks, 66% accepted, both spins: 16 sites x 256
+// 22.7 / 21.9, 36 x 256 53.9 / 59.0, 64 x 256 133 / 154, 80 x 200 341 / 311, 100 x 64 318 / 275, 112 x 64 398 / 434,
+// 144 x 64 742 / 811, 256 x 32 2742 / 3368; one spin: 72 x 1024 422 / 471, 120 x 256 436 / 518.
+bool pairs_one_at_a_time(const FlipArgs<df2>& f) {
+  if (f.kk <= kSingleDelay && f.kk * f.N <= kSingleWork && f.g_in_smem) return true;
+  if (f.tc_fold) return false;
+  const bool two_ctas = f.g_in_smem && flip_smem_bytes(f.N, f.kk, sizeof(df2), 1, f.ns) <= kBlockSmem / 2;
+  const bool held = block_smem<df2>(f.N, f.ns, true, kFoldPairs, f.N + 2) <= kBlockSmem;
+  return f.N > 24 && !(f.ns == 2 && held && !two_ctas);
+}
+
 template <>
 void flip_slice<df2>(const FlipArgs<df2>& f, int n_chains, cudaStream_t st) {
-  const bool single = f.kk <= kSingleDelay && f.kk * f.N <= kSingleWork && f.g_in_smem;
-  if (!single && (f.tc_fold ? flip_block<df2, kFoldTensor>(f, n_chains, st)
-                            : flip_block<df2, kFoldPairs>(f, n_chains, st)))
+  if (!pairs_one_at_a_time(f) && (f.tc_fold ? flip_block<df2, kFoldTensor>(f, n_chains, st)
+                                            : flip_block<df2, kFoldPairs>(f, n_chains, st)))
     return;
   const size_t bytes = flip_smem_bytes(f.N, f.kk, sizeof(df2), f.g_in_smem, f.ns);
   allow_max_dynamic_smem((const void*)k_flip_df);
