@@ -20,6 +20,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/nmc_gen.h"
@@ -82,19 +83,21 @@ __global__ void k_convt_fwd(const float* __restrict__ in, int Cin, Shape3 is,
 }
 
 // The same convolution for many samples, lanes on samples: in [Cin][q][ld], ld = n rounded up to 4,
-// so that a warp's input reads are contiguous and 16-byte copies aligned for every n, its weights uniform, and its tap ranges the same for all lanes. A warp
+// so that a warp's input reads are contiguous and 16-byte copies aligned for every n, its weights
+// uniform, and its tap ranges the same for all lanes. A warp
 // takes kTo0 outputs along the first axis (the long one of both kernels and inputs, so that nearly
 // every tap serves all of them) at one (o1, o2), a thread NS consecutive samples: one 16-byte
 // read each of inputs and weights serves 16 multiply-adds. Per input channel and q0 the CTA (one
 // range of o0, 32 NS samples, up to 9 warps) stages the plane of inputs and the kTo0 planes of
 // weights that meet there, interleaved and zero outside the kernel (cp.async, two stages ahead).
 // Inputs run downwards, so each output's taps k run upwards in the order of k_convt_fwd, and a
-// zero weight adds nothing: the same bits. Bound by instruction issue (51% busy on average, the SMs
-// with two long CTAs nearly fully) around the multiply-adds.
+// plane outside an output's kernel is left out: the same bits, NaN included. Bound by instruction
+// issue (51% busy on average, the SMs with two long CTAs nearly fully) around the multiply-adds.
 // Measured, 256 samples of the paper's second layer (2.3 G multiply-adds): 807 us against 4757
 // with one output per thread (two loads and a bounds walk per multiply-add); 918 with 18 warps per
-// CTA, 1663 with the
-// outputs of a warp along the second axis, where half the taps serve none of them.
+// CTA, 1663 with the outputs of a warp along the second axis, where half the taps serve none of
+// them. Leaving out the planes outside the kernel, which had multiplied by zero: 1738 -> 1688 us
+// for two passes of both layers.
 constexpr int kTo0 = 4, kRow = 3, kSampleStages = 3, kSampleWarps = 9;
 
 struct SamplePlan {
@@ -154,7 +157,7 @@ k_convt_samples(const float* __restrict__ in, int Cin, Shape3 is, const float* _
     for (int s = 0; s < NS; ++s) acc[j][s] = bias[co];
   fetch(0);
   fetch(1);
-  for (int step = 0; step < steps; ++step) {
+  for (int step = 0, q0 = q0b; step < steps; ++step, q0 = q0 > q0a ? q0 - 1 : q0b) {
     asm volatile("cp.async.wait_group 1;" ::: "memory");
     __syncthreads();   // this step's planes are here, the last step's are read
     fetch(step + 2);
@@ -162,36 +165,45 @@ k_convt_samples(const float* __restrict__ in, int Cin, Shape3 is, const float* _
     const float* x = sx + step % kSampleStages * (pl.xs + pl.ws);
     const float* w = x + pl.xs + (o1 * ks.d2 + o2) * kTo0;
     x += lane * NS;
-    for (int q1 = q1b; q1 >= q1a; --q1) {
-      const float* xr = x + q1 * is.d2 * L;
-      const float* wr = w - q1 * ks.d2 * kTo0;
-      for (int q2 = q2b; q2 >= q2a; q2 -= kRow) {   // a row's reads together, then its sums
-        float v[kRow][NS], wv[kRow][kTo0];
+    // outputs ja .. jb - 1 meet the kernel here; the others' weights are zero, but a NaN among the inputs
+    // would still reach them
+    const int ja = q0 - o0, jb = ja + ks.d0;
+    auto plane = [&](auto whole) {
+      for (int q1 = q1b; q1 >= q1a; --q1) {
+        const float* xr = x + q1 * is.d2 * L;
+        const float* wr = w - q1 * ks.d2 * kTo0;
+        for (int q2 = q2b; q2 >= q2a; q2 -= kRow) {   // a row's reads together, then its sums
+          float v[kRow][NS], wv[kRow][kTo0];
 #pragma unroll
-        for (int i = 0; i < kRow; ++i) {
-          if (q2 - i < q2a) break;
-          if constexpr (NS == 4) {
-            const float4 u = *reinterpret_cast<const float4*>(xr + (q2 - i) * L);
-            v[i][0] = u.x; v[i][1] = u.y; v[i][2] = u.z; v[i][3] = u.w;
-          } else if constexpr (NS == 2) {
-            const float2 u = *reinterpret_cast<const float2*>(xr + (q2 - i) * L);
-            v[i][0] = u.x; v[i][1] = u.y;
-          } else {
-            v[i][0] = xr[(q2 - i) * L];
+          for (int i = 0; i < kRow; ++i) {
+            if (q2 - i < q2a) break;
+            if constexpr (NS == 4) {
+              const float4 u = *reinterpret_cast<const float4*>(xr + (q2 - i) * L);
+              v[i][0] = u.x; v[i][1] = u.y; v[i][2] = u.z; v[i][3] = u.w;
+            } else if constexpr (NS == 2) {
+              const float2 u = *reinterpret_cast<const float2*>(xr + (q2 - i) * L);
+              v[i][0] = u.x; v[i][1] = u.y;
+            } else {
+              v[i][0] = xr[(q2 - i) * L];
+            }
+            const float4 u = *reinterpret_cast<const float4*>(wr - (q2 - i) * kTo0);
+            wv[i][0] = u.x; wv[i][1] = u.y; wv[i][2] = u.z; wv[i][3] = u.w;
           }
-          const float4 u = *reinterpret_cast<const float4*>(wr - (q2 - i) * kTo0);
-          wv[i][0] = u.x; wv[i][1] = u.y; wv[i][2] = u.z; wv[i][3] = u.w;
-        }
 #pragma unroll
-        for (int i = 0; i < kRow; ++i) {
-          if (q2 - i < q2a) break;
+          for (int i = 0; i < kRow; ++i) {
+            if (q2 - i < q2a) break;
 #pragma unroll
-          for (int j = 0; j < kTo0; ++j)
+            for (int j = 0; j < kTo0; ++j) {
+              if (!decltype(whole)::value && (j < ja || j >= jb)) continue;
 #pragma unroll
-            for (int s = 0; s < NS; ++s) acc[j][s] = fmaf(v[i][s], wv[i][j], acc[j][s]);
+              for (int s = 0; s < NS; ++s) acc[j][s] = fmaf(v[i][s], wv[i][j], acc[j][s]);
+            }
+          }
         }
       }
-    }
+    };
+    if (ja <= 0 && jb >= kTo0) plane(std::true_type());
+    else plane(std::false_type());
   }
   if (!live) return;
 #pragma unroll
