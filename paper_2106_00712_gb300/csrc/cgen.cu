@@ -576,7 +576,7 @@ struct nmc_cgen {
   __nv_bfloat16 *thb = nullptr, *act[kLayers] = {}, *gA = nullptr, *gB = nullptr;
   double* dloss = nullptr;
   // the weights as k_cg_conv reads them (FP32, per layer forward and backward), and the
-  // partial sums of k_cg_bwd_w_tc ([parts][the largest layer])
+  // partial sums of k_cg_bwd_w_tc ([parts][the largest layer]), where the largest call takes those kernels
   float *wf[kLayers] = {}, *wb[kLayers] = {}, *part = nullptr;
   int parts = 0;
   long long steps = 0;
@@ -735,8 +735,10 @@ void backward(nmc_cgen* g, const int8_t* d_fields, int n) {
   }
 }
 
-// the convolutions' layouts of the current BF16 weights
+// the convolutions' layouts of the current BF16 weights, if any call reads them (a launch of some 5 us
+// behind every change of the weights)
 void layout(nmc_cgen* g) {
+  if (!g->wf[0]) return;
   LayoutArgs a;
   int most = 0;
   for (int j = 0; j < kLayers; ++j) {
@@ -800,11 +802,11 @@ nmc_status nmc_cgen_create(int Lx, int Ly, int L_tau, int channels, uint64_t see
   if (s == NMC_OK) s = cg_alloc(g, g->gA, nb * C * S);
   if (s == NMC_OK) s = cg_alloc(g, g->gB, nb * C * S);
   if (s == NMC_OK) s = cg_alloc(g, g->dloss, 1);
-  for (int j = 0; j < kLayers; ++j) {
+  for (int j = 0; j < kLayers && nb * S * C >= kTileOutputs; ++j) {
     if (s == NMC_OK) s = cg_alloc(g, g->wf[j], (long long)kK * ci[j] * pad8(co[j]));
     if (s == NMC_OK) s = cg_alloc(g, g->wb[j], (long long)kK * co[j] * pad8(ci[j]));
   }
-  if (Lx % 2 == 0 && C <= 32) {
+  if (Lx % 2 == 0 && C <= 32 && nb * S >= kTcPositions) {
     g->parts = nmc::sm_count();
     if (s == NMC_OK) s = cg_alloc(g, g->part, g->parts * ((long long)C * C * kK + C));
   }
