@@ -348,20 +348,28 @@ __global__ void k_cg_layout(LayoutArgs a) {
 // nine warps, one per (t, y) neighbour, holds all 27 Cin Cout sums; per tile of TT slices of one
 // sample it stages g [co][position] and h three times, shifted by -1, 0, 1 along x, with a
 // halo in t and y, so that a warp's B operand (pairs of consecutive positions) is a 4-byte read
-// at a constant offset. The tensor core cuts the low bits of long sums, so they are added to a
-// second set of sums in shared memory after every tile (FP32, to nearest), written out once per
-// CTA and added up over the CTAs in a fixed order (k_cg_sum).
+// at a constant offset. The tensor core cuts the low bits of its sums, so it adds 16 positions at a time
+// only: their sums are added in registers (FP32, to nearest), a tile's in shared memory, and the CTAs'
+// in a fixed order with the rounding errors carried along (k_cg_sum; how the tiles are shared out, and so
+// the last bits, follow the SM count).
 // What bounds it: staging (the product itself is 9.1 GFLOP per middle layer, 20 us). Measured per
-// middle layer at batch 64 x 40 x 8 x 8, 32 channels: 3105 us with one CTA per (ci, co), 108 now.
+// middle layer at batch 64 x 40 x 8 x 8, 32 channels: 3105 us with one CTA per (ci, co), 108 with a tile's
+// 512 positions left to the tensor core and the CTAs' sums added one after the other. Errors were then up to
+// 1.4e-6 of a layer's largest entry (1e-7 to 3e-7 rms), with one CTA per (ci, co) 1.9e-7 (2e-8), now 7e-8
+// (1e-8); the whole gradient call takes 1565 us instead of 1524.
 constexpr int kBwThreads = 288;
 
-__device__ __forceinline__ void mma_bf(float (&d)[4], const unsigned (&a)[4], unsigned b0,
+// acc += a b, the product of 16 terms by the tensor core and its sum added with rounding to nearest
+__device__ __forceinline__ void mma_bf(float (&acc)[4], const unsigned (&a)[4], unsigned b0,
                                        unsigned b1) {
+  float d[4];
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-      "{%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+      "{%8,%9}, {%10,%10,%10,%10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) acc[i] = __fadd_rn(acc[i], d[i]);
 }
 
 struct BwTile {
@@ -500,10 +508,14 @@ k_cg_bwd_w_tc(const __nv_bfloat16* __restrict__ g, int Cout, const __nv_bfloat16
 __global__ void k_cg_sum(const float* __restrict__ part, int P, int parts, float* __restrict__ out) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= P) return;
-  float s = 0.f;
+  float s = 0.f, low = 0.f;   // (with what each addition rounds off, by TwoSum)
 #pragma unroll 8
-  for (int c = 0; c < parts; ++c) s += part[(long long)c * P + i];
-  out[i] = s;
+  for (int c = 0; c < parts; ++c) {
+    const float x = part[(long long)c * P + i], t = __fadd_rn(s, x), z = __fsub_rn(t, s);
+    low = __fadd_rn(low, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(x, z)));
+    s = t;
+  }
+  out[i] = __fadd_rn(s, low);
 }
 
 __global__ void k_cg_adam(float* __restrict__ th, const float* __restrict__ gr,
