@@ -84,7 +84,7 @@ def traffic_of(src):
 def step_flop(N, L, nb, chains, ns, acc):
     """Algorithmic flop of one sweep of every chain, counted per step of the sweep (both
     spins unless ns = 1): wraps 2 products per slice, stack products 1 per slice, the
-    recompute (3 products, Gauss-Jordan 3N^3) and QR with Q (8/3 N^3) and the T update
+    recompute (3 products, elimination 3N^3) and QR with Q (8/3 N^3) and the T update
     (1 product) per stabilization, the measurement (2 products) per stabilization, and the
     delayed updates 2N^2 per accepted flip. Products are 2N^3."""
     p = 2.0 * N ** 3
@@ -103,11 +103,16 @@ def class_rooflines(st, base, ns, acc, peaks, tc, tc_products=1.0):
     """Achieved vs peak for each timed kernel class of the path (algorithmic work per launch
     / average event-timed launch duration). Per launch, every class runs over the batch of
     ns x chains matrices of N x N: products 2N^3 each (the tensor-core class: `tc_products`
-    products per launch, each its 21 FP16 digit products, against the BF16 peak); QR with Q formed 8/3 N^3; Gauss-Jordan on
-    [X | N right-hand sides] 3N^3; a slice of flips, per accepted flip and spin, a rank-k
-    flush share 2N^2 plus the panel column and row 2Nk (k = delay). Each class is quoted
-    against the pipe it runs on: `peaks` holds the measured FP64 and FP32 SIMT peaks and the
-    BF16 tensor peak (TFLOP/s)."""
+    products per launch, each its 21 FP16 digit products, against the BF16 peak); QR with Q formed
+    8/3 N^3; the solve 3N^3, what elimination of [X | N right-hand sides] takes; a slice of flips,
+    per accepted flip and spin, a rank-k flush share 2N^2 plus the panel column and row 2Nk
+    (k = delay). `peaks` holds the measured FP64 and FP32 SIMT peaks and the BF16 tensor peak
+    (TFLOP/s).
+
+    `frac` is against the pipe that the class's arithmetic is of. FP64 products, QR and solve do
+    FP64-class work on other pipes (exact FP16 digits on the tensor cores, 64-bit fixed point, tensor
+    core updates), so theirs compares with an FP64 kernel and may exceed 1: they carry `equivalent`
+    (saying so), `pipe`, and, where the work of the pipe itself is counted, `frac_of_pipe`."""
     N, C, k = WL.N, WL.n_chains, WL.delay_k
     batch = ns * C
     simt = "fp32" if base in ("fp32", "fp32x2") else "fp64"
@@ -151,12 +156,16 @@ def class_rooflines(st, base, ns, acc, peaks, tc, tc_products=1.0):
                 "fp32x2": "k_gemm_fx (FP64 recompute, T updates by exact FP16 digits on mma.sync)"}[base]
         pk = "fp32" if base == "fp32" else "fp64"
         a = rate("gemm", 2.0 * N ** 3 * batch)
-        out["gemm"] = entry("alu", kern, a, peaks[pk],
-                            f"{pk.upper()} FMA probe (nmc_fma_probe), of measured")
+        slices = {}
+        if pk == "fp64" and 16 < N <= 256:   # 28 FP16 digit products per product
+            slices = {"equivalent": "FP64", "pipe": "tensor (mma.sync)", "achieved_of_pipe": 28 * a,
+                      "frac_of_pipe": 28 * a / peaks["bf16"]}
+        out["gemm"] = entry("tensor" if slices else "alu", kern, a, peaks[pk],
+                            f"{pk.upper()} FMA probe (nmc_fma_probe), of measured", **slices)
     if st.get("flip", (0,))[0]:
         a = rate("flip", acc * N * C * ns * (2.0 * N * N + 2.0 * N * k))
         kern = {"fp64": "k_flip_block<double>", "fp32": "k_flip<float>",
-                "fp32x2": "k_flip_block<FP32 pairs>"}[base]
+                "fp32x2": "k_flip_block<FP32 pairs>" if tc else "k_flip_df (FP32 pairs)"}[base]
         extra = {}
         if base == "fp32x2":
             extra["frac_of_pair_ceiling"] = a / (peaks["fp32"] / PAIR_INSTR_PER_FMA)
@@ -174,11 +183,16 @@ def class_rooflines(st, base, ns, acc, peaks, tc, tc_products=1.0):
                                         "updates); one launch = one slice of every chain; "
                                         "latency-bound (acceptances of a chain are sequential)",
                             **extra)
-    for cls, kname, flop in (("qrp", "k_qrp (column-pivoted QR + Q in 64-bit fixed point)", 8.0 / 3.0 * N ** 3),
-                             ("solve", "k_solve (FP64 blocked LU, updates on mma.sync)", 3.0 * N ** 3)):
+    lu = N > 40   # (up to there Gauss-Jordan in FP64)
+    for cls, kname, flop, kw in (
+            ("qrp", "k_qrp (column-pivoted QR + Q in 64-bit fixed point)", 8.0 / 3.0 * N ** 3,
+             {"equivalent": "FP64", "pipe": "integer"}),
+            ("solve", "k_solve (FP64 blocked LU, updates on mma.sync)" if lu else "k_solve_gj", 3.0 * N ** 3,
+             {"equivalent": "FP64 elimination (the LU itself is 8/3 N^3)",
+              "pipe": "FP64, tensor and integer"} if lu else {})):
         if st.get(cls, (0,))[0]:
             out[cls] = entry("alu", kname, rate(cls, flop * batch), peaks["fp64"],
-                             "FP64 FMA probe (nmc_fma_probe), of measured")
+                             "FP64 FMA probe (nmc_fma_probe), of measured", **kw)
     for v in out.values():
         v.setdefault("traffic", None)
     return out
