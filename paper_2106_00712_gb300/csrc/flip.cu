@@ -575,7 +575,9 @@ __device__ __forceinline__ void decide_block(const FlipArgs<T>& f, BlockStage<T>
   bar_decide();
   int m = 0;
   for (int lo = 0; lo < kb;) {   // sites below lo are decided
-    // every remaining site as if it were the next: lane j site j
+    // every remaining site as if it were the next: lane j site j. (A faster warp may already update its rows
+    // below the flip that all warps are about to find: only entries of sites beyond that flip change, and
+    // neither the first accepted site nor anything taken from it depends on them.)
     const T gu = st.S[0][jj][jj], gd = ns == 2 ? st.S[1][jj][jj] : gu;
     const float hu = 1.f - A::top(gu), hd = ns == 2 ? 1.f - A::top(gd) : A::top(gu);
     const float R32 = (1.f + du * hu) * (1.f + dd * hd);

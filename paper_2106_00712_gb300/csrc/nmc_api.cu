@@ -633,7 +633,7 @@ void flip(nmc_ctx* x, int l, const uint8_t* replay) {
     };
     FlipArgs<df2> f{x->dG2, x->dS, x->N, x->Lt, l, x->kk, x->g_in_smem, k0, k1,
                     (uint32_t)x->sweep_counter, x->opt.chain_offset, dm, dp, x->dSign,
-                    x->dCounts, replay, nullptr, split(dm), split(dp), x->ns(), x->dCtr};
+                    x->dCounts, replay, split(dm), split(dp), x->ns(), x->dCtr};
     f.tc_fold = x->tc() ? 1 : 0;
     f.chain_id = x->dChainId;
     f.sweep_base = x->dSweepBase;
@@ -641,14 +641,14 @@ void flip(nmc_ctx* x, int l, const uint8_t* replay) {
   } else if (x->fp32()) {
     FlipArgs<float> f{x->dGf, x->dS, x->N, x->Lt, l, x->kk, x->g_in_smem, k0, k1,
                       (uint32_t)x->sweep_counter, x->opt.chain_offset, dm, dp, x->dSign,
-                      x->dCounts, replay, nullptr, df2{0.f, 0.f}, df2{0.f, 0.f}, x->ns(), x->dCtr};
+                      x->dCounts, replay, df2{0.f, 0.f}, df2{0.f, 0.f}, x->ns(), x->dCtr};
     f.chain_id = x->dChainId;
     f.sweep_base = x->dSweepBase;
     launch(x, KC_FLIP, [&] { flip_slice(f, x->chains(), x->st()); });
   } else {
     FlipArgs<double> f{x->dG, x->dS, x->N, x->Lt, l, x->kk, x->g_in_smem, k0, k1,
                        (uint32_t)x->sweep_counter, x->opt.chain_offset, dm, dp, x->dSign,
-                       x->dCounts, replay, nullptr, df2{0.f, 0.f}, df2{0.f, 0.f}, x->ns(), x->dCtr};
+                       x->dCounts, replay, df2{0.f, 0.f}, df2{0.f, 0.f}, x->ns(), x->dCtr};
     f.chain_id = x->dChainId;
     f.sweep_base = x->dSweepBase;
     launch(x, KC_FLIP, [&] { flip_slice(f, x->chains(), x->st()); });

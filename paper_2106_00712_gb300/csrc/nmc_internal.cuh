@@ -177,7 +177,8 @@ void gemm_tc(const DfGemmArgs& g, bool const_is_a, const void* tmap, int* err, c
 void split_to_df(const double* x, df2* y, long long n, cudaStream_t st);
 
 // ---------------------------------------------------------------------------- UDT
-// Column-pivoted Householder QR of X[b] (N x N row-major): X P = Q R. Writes Q (U),
+// Column-pivoted Householder QR of X[b] (N x N row-major): X P = Q R, pivots by norms compared to
+// 2^-19 (lowest index among equals). Writes Q (U),
 // D = |diag R| and Tp = D^{-1} R P^T. ws: per-matrix global workspace of 2*N*N doubles
 // (used when the matrix does not fit in shared memory).
 void qrp_udt(const double* X, double* U, double* D, double* Tp, double* ws, int N, int batch,
@@ -202,11 +203,10 @@ struct FlipArgs {
   double* sign;              // per chain
   unsigned long long* counts;  // per chain: attempts, accepts, disagreements
   const uint8_t* replay;     // [chain][L][N] or null
-  T* panels_g;               // unused (panels live in shared memory)
   df2 dm2, dp2;              // dm, dp as FP32 pairs (compensated mode)
   int ns;                    // 2 spins, or 1: spin up only, G_dn = I - P G_up^T P
   const long long* ctr;      // device counters (ctr[0] = sweep counter) or null: use sweep
-  int tc_fold = 0;           // compensated mode: 1 = rank-k fold may use the tensor cores
+  int tc_fold = 0;           // compensated mode: 1 = folds may use the tensor cores
   const long long* chain_id = nullptr;    // per chain: global index (Philox word 2), or null
   const long long* sweep_base = nullptr;  // per chain: sweep counter at its start, or null
 };

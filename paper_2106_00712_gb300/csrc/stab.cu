@@ -2,7 +2,8 @@
 // B-matrix products and the stable recompute of G = (I + R L)^{-1}.
 //
 // k_qrp: Householder QR with column pivoting (Businger-Golub): at step p the remaining
-//   column of largest norm (lowest index on ties) is swapped into place, a reflector
+//   column of largest norm is swapped into place (norms are FP32, compared to 2^-19, lowest index on
+//   ties: near-ties may fall either way, so D need not be ordered to the last bits), a reflector
 //   H_p = I - tau v v^T zeroes it below the diagonal, and the trailing columns are updated;
 //   squared column norms are downdated and summed again when little of them is left. Outputs
 //   U = Q (column by column, in registers), D = |diag R| and
@@ -414,7 +415,7 @@ k_qrp(const double* __restrict__ X, double* __restrict__ U, double* __restrict__
   for (int e = tid; e < (int)NN; e += THREADS) {
     const int r = e / N, c = e - r * N;
     double t = 0.0;
-    if (c >= r) {   // the quotient from the reciprocal, with one correction
+    if (c >= r) {   // the quotient from the reciprocal, corrected by its remainder (as in quotient.cuh)
       const double w = (double)W[(long long)c * ldw + r], d = rd[r].x;
       t = w * rd[r].y;
       t = pow2_scale(fma(fma(-t, d, w), rd[r].y, t), Eb[c] - Eb[r]);
