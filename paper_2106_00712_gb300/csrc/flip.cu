@@ -1008,16 +1008,17 @@ void flip_slice<double>(const FlipArgs<double>& f, int n_chains, cudaStream_t st
 }
 
 // FP32X2, without tensor cores: a block's fold costs as much as the folds of single flips, and the vectors come
-// on top, so blocks pay only for a few sites, and where both spins' matrices fit beside a block but not beside
-// k_flip_df's panels twice to an SM (its 288 threads alone are too few). us a slice at delay 16, one at a time / blocks, 66% accepted, both spins: 16 sites x 256
-// 22.7 / 21.9, 36 x 256 53.9 / 59.0, 64 x 256 133 / 154, 80 x 200 341 / 311, 100 x 64 318 / 275, 112 x 64 398 / 434,
-// 144 x 64 742 / 811, 256 x 32 2742 / 3368; one spin: 72 x 1024 422 / 471, 120 x 256 436 / 518.
+// on top, so blocks pay only for a few sites, and with both spins above 64 sites, where k_flip_df's 256 threads
+// take the panels' entries in several passes, as long as G fits a block's shared memory. us a slice at delay 16,
+// one at a time / blocks, 66% accepted, both spins: 16 sites x 256 22.7 / 21.9, 36 x 256 53.9 / 59.0, 64 x 256
+// 133 / 154, 72 x 16 159 / 133, 72 x 512 592 / 466 (delay 8: 154 / 140 and 406 / 495), 80 x 200 341 / 311,
+// 100 x 64 318 / 275, 112 x 64 398 / 434, 144 x 64 742 / 811, 256 x 32 2742 / 3368; one spin: 72 x 1024
+// 422 / 471, 120 x 256 436 / 518.
 bool pairs_one_at_a_time(const FlipArgs<df2>& f) {
   if (f.kk <= kSingleDelay && f.kk * f.N <= kSingleWork && f.g_in_smem) return true;
   if (f.tc_fold) return false;
-  const bool two_ctas = f.g_in_smem && flip_smem_bytes(f.N, f.kk, sizeof(df2), 1, f.ns) <= kBlockSmem / 2;
   const bool held = block_smem<df2>(f.N, f.ns, true, kFoldPairs, f.N + 2) <= kBlockSmem;
-  return f.N > 24 && !(f.ns == 2 && held && !two_ctas);
+  return f.N > 24 && !(f.ns == 2 && f.N > 64 && held);
 }
 
 template <>

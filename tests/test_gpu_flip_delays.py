@@ -2,9 +2,8 @@
 every field after every sweep equals the FP64 oracle's, and G at the end. Sizes where the delay alone
 sets the line (16, 36 sites), where delay x sites does (64, 100) and where shared memory does (100 and
 120 sites, one spin, in FP64), lattices smaller than the default delay (2 and 8 sites), and blocks cut
-short of 16 sites (9 and 13). FP32X2 on both sides of its own lines: 24 and 26 sites, delays that leave one
-CTA of single flips to an SM and two (72 sites), G in shared memory for blocks or not (100, 104), and G in
-global memory for both (112).
+short of 16 sites (9 and 13). FP32X2 on both sides of its own lines: 24 and 26 sites, 64 and 66, both spins
+and one (100), and G that fits a block's shared memory or not (100, 104, 112).
 
 Bar on G: 1e-10 of max|G| in FP64, 1e-8 in FP32 pairs (the bars of the blocks' own tests: FP32 pairs
 carry 2^-46 of a wrap's terms over five slices, amplified by the propagators by a few 1e2)."""
@@ -21,7 +20,7 @@ CASES = [("fp64", 4, 4, k, 0) for k in (1, 6, 7, 9)] + [("fp64", 6, 6, k, 0) for
         [("split", 4, 4, k, 0) for k in (1, 8, 9)] + [("split", 8, 8, k, 0) for k in (6, 7, 13)] + \
         [("split", 10, 10, k, 0) for k in (4, 5)] + [("split", 12, 10, 3, 1)] + \
         [("x2", 6, 6, 8, 0), ("x2", 6, 6, 9, 0), ("x2", 8, 8, 6, 1), ("x2", 8, 8, 7, 1)] + \
-        [("x2", 6, 4, 16, 0), ("x2", 26, 1, 16, 0), ("x2", 12, 6, 12, 0), ("x2", 12, 6, 16, 0)] + \
+        [("x2", 6, 4, 16, 0), ("x2", 26, 1, 16, 0), ("x2", 16, 4, 16, 0), ("x2", 66, 1, 12, 0)] + \
         [("x2", 10, 10, 16, ph) for ph in (0, 1)] + [("x2", 26, 4, 16, 0), ("x2", 28, 4, 16, 0)] + \
         [(m, Lx, Ly, 16, 0) for m in ("fp64", "split", "x2") for Lx, Ly in ((2, 1), (4, 2))]
 
