@@ -26,6 +26,7 @@
 #include <cmath>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "nmc_cgen.h"
@@ -348,26 +349,31 @@ __global__ void k_cg_layout(LayoutArgs a) {
 // nine warps, one per (t, y) neighbour, holds all 27 Cin Cout sums; per tile of TT slices of one
 // sample it stages g [co][position] and h three times, shifted by -1, 0, 1 along x, with a
 // halo in t and y, so that a warp's B operand (pairs of consecutive positions) is a 4-byte read
-// at a constant offset. The tensor core cuts the low bits of its sums, so it adds 16 positions at a time
+// at a constant offset. The tensor core cuts the low bits of its sums, so it adds 32 positions at a time
 // only: their sums are added in registers (FP32, to nearest), a tile's in shared memory, and the CTAs'
 // in a fixed order with the rounding errors carried along (k_cg_sum; how the tiles are shared out, and so
 // the last bits, follow the SM count).
 // What bounds it: staging (the product itself is 9.1 GFLOP per middle layer, 20 us). Measured per
 // middle layer at batch 64 x 40 x 8 x 8, 32 channels: 3105 us with one CTA per (ci, co), 108 with a tile's
 // 512 positions left to the tensor core and the CTAs' sums added one after the other. Errors were then up to
-// 1.4e-6 of a layer's largest entry (1e-7 to 3e-7 rms), with one CTA per (ci, co) 1.9e-7 (2e-8), now 7e-8
-// (1e-8); the whole gradient call takes 1565 us instead of 1524.
+// 1.4e-6 of a layer's largest entry (1e-7 to 3e-7 rms), with one CTA per (ci, co) 1.9e-7 (2e-8), now 8e-8
+// (1e-8); the whole gradient call takes 1542 us instead of 1522 (16 positions at a time: 7e-8, 1561).
 constexpr int kBwThreads = 288;
 
-// acc += a b, the product of 16 terms by the tensor core and its sum added with rounding to nearest
-__device__ __forceinline__ void mma_bf(float (&acc)[4], const unsigned (&a)[4], unsigned b0,
+__device__ __forceinline__ void mma_bf(float (&d)[4], const unsigned (&a)[4], unsigned b0,
                                        unsigned b1) {
-  float d[4];
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-      "{%8,%9}, {%10,%10,%10,%10};"
-      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+      "{%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// acc += a b over K steps of 16 terms: the tensor core sums these, the addition rounds to nearest
+template <int K>
+__device__ __forceinline__ void add_products(float (&acc)[4], const unsigned (&a)[K][4], const unsigned (&b)[K][2]) {
+  float d[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < K; ++k) mma_bf(d, a[k], b[k][0], b[k][1]);
 #pragma unroll
   for (int i = 0; i < 4; ++i) acc[i] = __fadd_rn(acc[i], d[i]);
 }
@@ -447,27 +453,38 @@ k_cg_bwd_w_tc(const __nv_bfloat16* __restrict__ g, int Cout, const __nv_bfloat16
     for (int ts = 0; ts < t.TT; ++ts) {
       const __nv_bfloat16* hb = Hs + (lane >> 2) * t.hld + ((ts + 1 + dt) * A2 + 1 + da) * d.B +
                                 2 * (lane & 3);
-      for (int q = 0; q < t.ABp; q += 16) {
-        unsigned af[MT][4];
+      auto positions = [&](int q, auto steps) {   // 16 positions each
+        constexpr int K = decltype(steps)::value;
+        unsigned af[MT][K][4];
 #pragma unroll
         for (int m = 0; m < MT; ++m)
-          asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                       : "=r"(af[m][0]), "=r"(af[m][1]), "=r"(af[m][2]), "=r"(af[m][3])
-                       : "r"(ga + (m * 16 * t.gld + ts * t.ABp + q) * 2));
+#pragma unroll
+          for (int k = 0; k < K; ++k)
+            asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                         : "=r"(af[m][k][0]), "=r"(af[m][k][1]), "=r"(af[m][k][2]), "=r"(af[m][k][3])
+                         : "r"(ga + (m * 16 * t.gld + ts * t.ABp + q + 16 * k) * 2));
 #pragma unroll
         for (int b = 0; b < 3; ++b)
 #pragma unroll
           for (int c = 0; c < NC; ++c) {
             const unsigned* hw = reinterpret_cast<const unsigned*>(hb + b * copy + c * 8 * t.hld + q);
-            const unsigned b0 = hw[0], b1 = hw[4];
+            unsigned bf[K][2];
 #pragma unroll
-            for (int m = 0; m < MT; ++m) mma_bf(acc[m][b][c], af[m], b0, b1);
+            for (int k = 0; k < K; ++k) bf[k][0] = hw[8 * k], bf[k][1] = hw[8 * k + 4];
+#pragma unroll
+            for (int m = 0; m < MT; ++m) add_products<K>(acc[m][b][c], af[m], bf);
           }
         if (warp == 4) {   // a column of ones: the bias gradient
+          unsigned ones[K][2];
 #pragma unroll
-          for (int m = 0; m < MT; ++m) mma_bf(ab[m], af[m], 0x3f803f80u, 0x3f803f80u);
+          for (int k = 0; k < K; ++k) ones[k][0] = ones[k][1] = 0x3f803f80u;
+#pragma unroll
+          for (int m = 0; m < MT; ++m) add_products<K>(ab[m], af[m], ones);
         }
-      }
+      };
+      int q = 0;
+      for (; q + 32 <= t.ABp; q += 32) positions(q, std::integral_constant<int, 2>());
+      if (q < t.ABp) positions(q, std::integral_constant<int, 1>());
     }
 #pragma unroll
     for (int m = 0; m < MT; ++m) {
