@@ -200,10 +200,11 @@ template <> struct Cut<double> {
   }
 };
 
-// Two warps share 16 rows for 4 tiles, one CTA's 8 warps on two of an SM's places: 512 matrices of 64
-// sites take 47 us in pairs of warps against 60 (before the carries) (three places of 4 warps: 456, for which the last 56
-// wait), 72 against 103 in FP64. Elsewhere one warp has its rows alone and waits for no other: 72 sites
-// x 1024 183 us against 248 in pairs, chains of 36 x 128 56 against 70.
+// Two warps share 16 rows for 4 tiles, one CTA's 8 warps on two of an SM's places: us, in pairs of warps / one
+// warp to 16 rows, 512 matrices of 64 sites a wrap 48 / 61 (FP64 69 / 82) and a chain of ten 242 / 264 (334 /
+// 350), 6 matrices 18 / 29 and 73 / 102. Elsewhere the tiles do not halve evenly or one warp has its rows alone
+// and waits for no other: in an earlier form of these kernels pairs took 248 us against 183 for a wrap of 72
+// sites x 1024, and 70 against 56 for chains of 36 x 128.
 template <int T> constexpr int tiles_per_warp() { return T == 4 ? 2 : T; }
 
 // A warp's tiles of a matrix of 16 T sites: 16 rows, H of the T columns of tiles
