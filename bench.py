@@ -68,10 +68,10 @@ TRAFFIC = {
     # dram__bytes_read.sum,dram__bytes_write.sum: a wrap reads 16.98 MB (the operand as FP32
     # pairs, once), a chain 10.5 MB (its FP64 operand is partly in L2), neither writes (the
     # results stay in L2); weighted by the sweep's launch mix (88 : 8)
-    "wrap.cu": ("39b15370818c6987", 16.44e6),
-    # k_flip_block (FP32 pairs), same configuration (one slice of 256 chains x 2 spins): 16.91 MB
+    "wrap.cu": ("ad3da1cbefc48b97", 16.44e6),
+    # k_flip_block (FP32 pairs), same configuration (one slice of 256 chains x 2 spins): 16.92 MB
     # read (G as FP32 pairs, once), 0 written (stays in L2)
-    "flip.cu": ("8f4cc10c59ca6120", 16.91e6),
+    "flip.cu": ("afc034d5b0c9252a", 16.92e6),
 }
 
 
@@ -609,7 +609,8 @@ def main():  # noqa: C901
     roofline = dict(rl.get(dom) or rl[max(rl, key=lambda k: st[k][2])])
     roofline.update({"dominant_class": dom, "share": share})
     roofline["others"] = {k: {kk: v[kk] for kk in ("kernel", "bound", "achieved", "peak", "frac",
-                                                  "traffic", "hbm_gbs", "hbm_frac") if kk in v}
+                                                  "traffic", "hbm_gbs", "hbm_frac", "equivalent", "pipe",
+                                                  "achieved_of_pipe", "frac_of_pipe") if kk in v}
                           for k, v in rl.items() if k != dom}
     sf = step_flop(WL.N, WL.L_tau, WL.L_tau // WL.n_wrap, WL.n_chains, ns, r["obs"].accept)
     whole_step = {"algorithmic_tflop_per_step": sf / 1e12,
