@@ -71,7 +71,7 @@ TRAFFIC = {
     "wrap.cu": ("ad3da1cbefc48b97", 16.44e6),
     # k_flip_block (FP32 pairs), same configuration (one slice of 256 chains x 2 spins): 16.92 MB
     # read (G as FP32 pairs, once), 0 written (stays in L2)
-    "flip.cu": ("afc034d5b0c9252a", 16.92e6),
+    "flip.cu": ("83a974b05637a70c", 16.92e6),
 }
 
 

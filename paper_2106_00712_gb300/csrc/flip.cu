@@ -809,7 +809,7 @@ k_flip_block(const FlipArgs<T> f, int kb_max) {
 // all decisions (from the same G, so the same ones), forms and folds the rows of its share of 16-row
 // tiles, and forms the columns of the same share, whose digits it writes to every CTA of the cluster.
 // Each entry sees the operations of k_flip_block in the same order. The barriers do not depend on what
-// was decided. 256 sites x 32 chains, us: one CTA per chain 966, two 557, four 391; eight (x 16 chains)
+// was decided. 256 sites x 32 chains, us (44% accepted): one CTA per chain 966, two 557, four 391; eight (x 16 chains)
 // 585 for four's 383. 100 x 64 with two 118 against 133 with G in shared memory; 64 x 32 59 against 55,
 // hence kClusterMinN where shared memory would do.
 constexpr int kClusterMinN = 96;

@@ -31,7 +31,7 @@ constexpr int kSolveThreads = 512;
 constexpr int kSolveWarps = kSolveThreads / 32;
 constexpr size_t kSmemLimit = 200 * 1024;
 // Up to here Gauss-Jordan is faster: 16 sites x 2 matrices 23 us against 29, 36 x 128 73 against 91;
-// 48 x 6 110 against 107, 48 x 512 296 against 220.
+// 48 x 6 110 against 111, 48 x 512 296 against 229.
 constexpr int kGaussJordanMax = 40;
 constexpr size_t kQrSmemLimit = 225 * 1024;
 
@@ -576,11 +576,12 @@ k_solve_gj(const double* __restrict__ X, const double* __restrict__ UR, long lon
 // Elimination in FP64 throughout took 1.5 N^3 multiply-adds at one warp operation per 20 cycles and
 // SM (246k cycles a matrix at N = 64); here the FP64 pipe adds once per entry and block (28k), and
 // does the triangles (48k) and the panels (26k).
-// us, Gauss-Jordan -> here: 64 sites x 512 583 -> 321, 64 x 6 197 -> 150, 72 x 1024 1430 -> 925,
-// 100 x 128 582 -> 302, 144 x 128 2800 -> 600, 256 x 64 (in global memory) 16100 -> 2100; the error of
-// Y against 64-bit-mantissa elimination is about half of before.
-// What bounds it: a matrix's dependent chain. Of 300k cycles at N = 64 the panels take 95k (1500 a
-// column: search, reciprocal, barrier, and some ten FP64 operations at 80 cycles from one warp), the
+// us, Gauss-Jordan -> here: 64 sites x 512 583 -> 335, 64 x 6 197 -> 155, 72 x 1024 1430 -> 971,
+// 100 x 128 582 -> 313, 144 x 128 2800 -> 619, 256 x 64 (in global memory) 16100 -> 2150; the error of
+// Y against 64-bit-mantissa elimination is about half of before. (With the pivots' reciprocals from an
+// approximation, an ulp off and wrong for the smallest and largest, 325, 151, 926, 305, 606, 2121.)
+// What bounds it: a matrix's dependent chain. Of 310k cycles at N = 64 the panels take 105k (1600 a
+// column: search, division, barrier, and some ten FP64 operations at 80 cycles from one warp), the
 // triangles 80k, the updates 70k; two matrices on an SM run in the time of one.
 __host__ __device__ inline size_t solve_small_bytes(int N, int chunk, int nw) {
   const int rows = max((N - 1) & ~15, 16);   // digit rows: all but the first (last) block's
